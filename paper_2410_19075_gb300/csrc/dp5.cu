@@ -101,15 +101,13 @@ __global__ void __launch_bounds__(kRingThreads, DpMinBlocks<M>::value)
     }
     if (i < N) {
         if (DS >= 1) {
-            int64_t qo[NQ];
-            double fo[NQ];
-            i128 W[NQ];
-            ring_window<NQ>(P, P.lam[pin], s_bases, tid, i, qo, fo, W);
+            int64_t qo[NQ], S[NQ];
+            ring_window<M, NQ>(P, P.lam[pin], s_bases, tid, sub, i, qo, S);
             double X[NX > 0 ? NX : 1];
 #pragma unroll
             for (int g = 0; g < NX; ++g) X[g] = DS == 1 ? y[(XOFF + g) * N + i] : P.xg[pin][g * N + i];
             const double Iext = (M == 2 && P.node_param) ? P.node_param[i] : 0.0;
-            Mo::rhs(P.mp, P.F, fo, qo, W, X, Iext, k);
+            Mo::rhs_ring(P.mp, qo, S, X, Iext, k);
         }
         if (DS <= 6) {
             double xn[D];

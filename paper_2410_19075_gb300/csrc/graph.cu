@@ -24,6 +24,7 @@ namespace simk {
 
 // Exact prefix P(pos) = sum_{m < pos} Q_m of component c on the periodic
 // extension, pos in [0, 2N).
+template <int NQ>
 __device__ __forceinline__ i128 graph_prefix_at(const RingPlan &P, const RingStageIO &a, int c, int64_t pos)
 {
     const int64_t N = P.N;
@@ -36,7 +37,7 @@ __device__ __forceinline__ i128 graph_prefix_at(const RingPlan &P, const RingSta
     if (pos == 0) return base;
     const int64_t s = (pos - 1) >> kSubLog2;
     return base + ldg_i128(grpofs + (s >> kGroupLog2)) + ldg_i128(a.ingrp_in + c * P.nsub + s) +
-           (i128)__ldg(a.lam_in + c * N + pos - 1);
+           (i128)__ldg(a.lam_in + (pos - 1) * NQ + c);
 }
 
 // Per-CTA bases of the run ends: for run r, end 2r is i + a (the run's first
@@ -89,7 +90,7 @@ __device__ __forceinline__ void graph_load_bases(const GraphPlan &G, const RingS
     __syncthreads();
 }
 
-template <int NQ> struct GraphGather {
+template <int M, int NQ> struct GraphGather {
     struct Pre {
         int64_t l[NQ], lp[NQ];
     };
@@ -100,20 +101,21 @@ template <int NQ> struct GraphGather {
     int64_t sub; // the CTA's sub-tile
     __device__ __forceinline__ void load(int tid, int64_t i, Pre &pre) const
     {
-        const int64_t N = G.r.N;
+        lam_load<NQ>(a.lam_in + i * NQ, pre.l);
 #pragma unroll
-        for (int c = 0; c < NQ; ++c) {
-            const int64_t *lam = a.lam_in + c * N;
-            pre.l[c] = __ldg(lam + i);
-            pre.lp[c] = tid ? __ldg(lam + i - 1) : 0;
-        }
+        for (int c = 0; c < NQ; ++c) pre.lp[c] = 0;
+        if (tid) lam_load<NQ>(a.lam_in + (i - 1) * NQ, pre.lp);
     }
     __device__ __forceinline__ void sync() const { graph_load_bases<NQ>(G, a, sub, nb, B); }
-    __device__ __forceinline__ void finish(int tid, int64_t i, const Pre &pre, int64_t (&qo)[NQ], double (&fo)[NQ],
-                                           i128 (&W)[NQ], int64_t &wsize, double &cs) const
+    template <int D>
+    __device__ __forceinline__ void finish(int tid, int64_t i, const Pre &pre, const double *X, double Iext,
+                                           double (&k)[D]) const
     {
         const RingPlan &P = G.r;
         const int64_t N = P.N;
+        int64_t qo[NQ];
+        double fo[NQ];
+        i128 W[NQ];
 #pragma unroll
         for (int c = 0; c < NQ; ++c) {
             qo[c] = pre.l[c] - pre.lp[c];
@@ -128,19 +130,17 @@ template <int NQ> struct GraphGather {
             const int kl = (lo >= B.start[el][1]) + (lo >= B.start[el][2]);
             const int kh = (hi >= B.start[eh][1]) + (hi >= B.start[eh][2]);
             const int64_t pl = lo - B.qn[el][kl], ph = hi - B.qn[eh][kh];
+            int64_t ll[NQ] = {}, lh[NQ] = {};
+            if (pl & (kSubTile - 1)) lam_load<NQ>(a.lam_in + (pl - 1) * NQ, ll);
+            if (ph & (kSubTile - 1)) lam_load<NQ>(a.lam_in + (ph - 1) * NQ, lh);
 #pragma unroll
-            for (int c = 0; c < NQ; ++c) {
-                const int64_t *lam = a.lam_in + c * N;
-                const int64_t ll = (pl & (kSubTile - 1)) ? __ldg(lam + pl - 1) : 0;
-                const int64_t lh = (ph & (kSubTile - 1)) ? __ldg(lam + ph - 1) : 0;
-                W[c] += (B.base[eh][kh][c] - B.base[el][kl][c]) + (i128)(lh - ll);
-            }
+            for (int c = 0; c < NQ; ++c) W[c] += (B.base[eh][kh][c] - B.base[el][kl][c]) + (i128)(lh[c] - ll[c]);
         }
         for (int r = nb; r < G.nruns; ++r) {
             const int2 run = __ldg(G.runs + r); // (a, len), a + len <= N
             const int64_t lo = i + run.x, hi = lo + run.y;
 #pragma unroll
-            for (int c = 0; c < NQ; ++c) W[c] += graph_prefix_at(P, a, c, hi) - graph_prefix_at(P, a, c, lo);
+            for (int c = 0; c < NQ; ++c) W[c] += graph_prefix_at<NQ>(P, a, c, hi) - graph_prefix_at<NQ>(P, a, c, lo);
         }
         // the node's difference entry: signed single links
         const int e = __ldg(G.ent + i);
@@ -149,15 +149,13 @@ template <int NQ> struct GraphGather {
             const int2 d = __ldg(G.dpos + t); // (offset, sign)
             int64_t j = i + d.x;
             j -= j >= N ? N : 0;
+            int64_t lj[NQ], lq[NQ] = {};
+            lam_load<NQ>(a.lam_in + j * NQ, lj);
+            if (j & (kSubTile - 1)) lam_load<NQ>(a.lam_in + (j - 1) * NQ, lq);
 #pragma unroll
-            for (int c = 0; c < NQ; ++c) {
-                const int64_t *lam = a.lam_in + c * N;
-                const int64_t q = (j & (kSubTile - 1)) ? __ldg(lam + j) - __ldg(lam + j - 1) : __ldg(lam + j);
-                W[c] += d.y > 0 ? (i128)q : -(i128)q;
-            }
+            for (int c = 0; c < NQ; ++c) W[c] += d.y > 0 ? (i128)(lj[c] - lq[c]) : -(i128)(lj[c] - lq[c]);
         }
-        wsize = __ldg(G.ek + e);
-        cs = __ldg(G.ecs + e);
+        Model<M>::rhs(P.mp, P.F, fo, qo, W, X, Iext, k, __ldg(G.ek + e), __ldg(G.ecs + e));
     }
 };
 
@@ -174,7 +172,7 @@ __global__ void __launch_bounds__(kRingThreads, GraphMinBlocks<M>::value)
     __shared__ GraphBases<NQ> s_bases;
     const RingStageIO a = stage_io<M, STAGE>(g.r);
     const int nb = g.nruns < kGraphSmemRuns ? g.nruns : kGraphSmemRuns;
-    stage_body<M, STAGE>(g.r, a, h, blockIdx.x, GraphGather<NQ>{g, a, s_bases, nb, (int64_t)blockIdx.x});
+    stage_body<M, STAGE>(g.r, a, h, blockIdx.x, GraphGather<M, NQ>{g, a, s_bases, nb, (int64_t)blockIdx.x});
 }
 
 template <int M>

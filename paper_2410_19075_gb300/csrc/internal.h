@@ -35,7 +35,8 @@ struct RingPlan {
     double *acc;        // D * N, RK4 accumulator k1 + 2 k2 + 2 k3
     double *xg[2];      // NX * N each, local stage-input variables (HH gates)
     const double *node_param; // N (HH I_ext) or nullptr
-    int64_t *lam[2];    // NQ * N each: inclusive prefix of Q(f) inside each sub-tile
+    int64_t *lam[2];    // NQ * N each: inclusive prefix of Q(f) inside each sub-tile, the NQ
+                        // components of a node adjacent (lam[i * NQ + c])
     i128 *ingrp[2];     // NQ * nsub each: exclusive prefix of each sub-tile inside its group
     i128 *grpofs[2];    // NQ * (ngroups + 1) each: exclusive prefix at group starts, then the total
     int64_t *subtot;    // NQ * nsub: sub-tile totals (scratch of the launch)
@@ -255,7 +256,7 @@ struct CubeBatchGroup {
 cudaError_t cube_batch_step(const CubeBatchGroup &g, double dt, cudaStream_t s); // one RK4 step of every member
 int lattice_row_warps(int64_t N1); // warps per CTA of the x pass for edge N1
 void lattice_rotation(LatticePlan &p, double alpha); // rot_* and mp.c[5] of a lattice (sim_api.cu)
-void ring_coupling_constants(ModelParams &mp, int model, int F); // ksh and c[5] of a Kuramoto ring (sim_api.cu)
+void ring_coupling_constants(ModelParams &mp, int model, const double *params, int F); // ksh and the scaled coupling constants of a ring (sim_api.cu)
 
 // Per-kernel timing of sim_step_timed: while set on the launching host thread,
 // every stage-kernel launch of ring_step, graph_step, lattice_step and

@@ -14,10 +14,11 @@ namespace simk {
 // cos of the phase through the integer-only fixed_sincos for the Kuramoto
 // models; u, v or V themselves otherwise), checking |f| < 2^lim (ok = false
 // outside it or for a non-finite value).
-// Every rhs() takes the node's window sums W; on a general link matrix it also
-// takes the node's link count (wsize, the FHN/HH self-term multiplier; -1 = the
-// network's) and a coupling scale cs = 1/K_i applied to the converted sums (the
-// constants c then carry K = 1).  The ring and lattice paths use the defaults.
+// rhs() (general link matrices) takes the node's window sums W, its link count
+// (wsize, the FHN/HH self-term multiplier) and a coupling scale cs = 1/K_i
+// applied to the converted sums (the constants c then carry K = 1).  rhs_ring()
+// takes the ring's window sums shifted right by ksh into int64 (ring_sums),
+// OWN_OUT: without the node itself (unless it is one of its own links).
 
 // Derived constants, computed once on the host in FP64.
 struct ModelParams {
@@ -25,7 +26,11 @@ struct ModelParams {
     int64_t q[2];     // Kuramoto models: cos alpha and sin alpha on the grid 2^-62
     uint64_t a0[2];   // Kuramoto models: alpha = aq pi/2 + alpha0, alpha0 in [0, pi/2):
     int aq;           //   cos alpha0, sin alpha0 on the grid 2^-63 (non-negative), aq in 0..3
-    int ksh;          // Kuramoto rings: right shift taking the exact window sums into int64
+    int ksh;          // rings: right shift taking the exact window sums into int64
+    uint64_t wsm;     // FHN and HH rings: wsize 2^(56 - ksh), for own_multiple
+    int fx;           // FHN rings: 1 = the slope's bracket in integer arithmetic (kq, a54 in range)
+    int64_t kq[4];    //   (sigma/K) b00, b01, b10, b11 times 2^(ksh + 67)
+    int64_t a54;      //   a on the grid 2^-54
     MathTables tab;   // device tables of the fast elementary functions
     int64_t wsize;    // window size including the node itself (2R+1 or (2P+1)^3)
     int include_self; // 1: the node is one of its own links
@@ -91,12 +96,9 @@ __device__ __forceinline__ double lattice_coupling_term(const ModelParams &P, co
 // with the non-negative cos alpha0, sin alpha0 (grid 2^-61), then aq quarter
 // turns.  Two signed high products give T on the grid 2^-(F - sh - 3).  No FP64
 // instruction and no conversion until the caller's single one.
-__device__ __forceinline__ int64_t ring_coupling(const ModelParams &P, const int64_t (&qo)[2], int F,
-                                                 const i128 (&W)[2], int sh)
+__device__ __forceinline__ int64_t ring_coupling(const ModelParams &P, const int64_t (&qo)[2], int F, int64_t S_s,
+                                                 int64_t S_c)
 {
-    const i128 ss = P.include_self ? W[0] : W[0] - (i128)qo[0];
-    const i128 sc = P.include_self ? W[1] : W[1] - (i128)qo[1];
-    const int64_t S_s = (int64_t)(ss >> sh), S_c = (int64_t)(sc >> sh);
     const int64_t s = qo[0] * (int64_t(1) << (62 - F)), c = qo[1] * (int64_t(1) << (62 - F));
     const int64_t c1 = mulhi_su(c, P.a0[0]) - mulhi_su(s, P.a0[1]); // e^{i alpha0} (c + i s), grid 2^-61
     const int64_t s1 = mulhi_su(s, P.a0[0]) + mulhi_su(c, P.a0[1]);
@@ -108,6 +110,22 @@ __device__ __forceinline__ int64_t ring_coupling(const ModelParams &P, const int
     default: ca = s1; sa = -c1; break;
     }
     return mulhi_ss(ca, S_s) - mulhi_ss(sa, S_c);
+}
+
+// The same from a node's 128-bit window sums (node included), shifted here.
+__device__ __forceinline__ int64_t ring_coupling_wide(const ModelParams &P, const int64_t (&qo)[2], int F,
+                                                      const i128 (&W)[2], int sh)
+{
+    const i128 ss = P.include_self ? W[0] : W[0] - (i128)qo[0];
+    const i128 sc = P.include_self ? W[1] : W[1] - (i128)qo[1];
+    return ring_coupling(P, qo, F, (int64_t)(ss >> sh), (int64_t)(sc >> sh));
+}
+
+// floor(q wsize 2^-ksh) for a node's own quantity |q| < 2^54: one high product,
+// (q 2^8) (wsize 2^(56 - ksh)) 2^-64.
+__device__ __forceinline__ int64_t own_multiple(const ModelParams &P, int64_t q)
+{
+    return mulhi_su((int64_t)((uint64_t)q << 8), P.wsm);
 }
 
 // The shift and the scale of ring_coupling's T for a window of ws links (the
@@ -132,6 +150,7 @@ __device__ __forceinline__ double ring_coupling_scale(int64_t ws, int F, double 
 // 2^-62.  Coupled quantity (sin phi, cos phi).
 template <> struct Model<0> {
     static constexpr int D = 1, NQ = 2, NX = 0, F = 53;
+    static constexpr bool OWN_OUT = true;
     __device__ __forceinline__ static void coupled_q(const ModelParams &P, const double (&x)[D], int F, int,
                                                      bool &ok, int64_t (&q)[NQ])
     {
@@ -140,16 +159,20 @@ template <> struct Model<0> {
         q[0] = q62_to(s62, F);
         q[1] = q62_to(c62, F);
     }
-    // Rings and link matrices: c[5] = (mu/K) 2^(ksh + 3 - F) (rings; a link
-    // matrix's node of wsize links scales mu cs instead).
+    // Link matrices: a node of wsize links scales mu cs.
     __device__ __forceinline__ static void rhs(const ModelParams &P, int F_, const double (&)[NQ],
-                                               const int64_t (&qo)[NQ], const i128 (&W)[NQ],
-                                               const double *, double, double (&k)[D],
-                                               int64_t wsize = -1, double cs = 1.0, const int64_t * = nullptr)
+                                               const int64_t (&qo)[NQ], const i128 (&W)[NQ], const double *, double,
+                                               double (&k)[D], int64_t wsize, double cs)
     {
-        int sh = P.ksh;
-        const double sc = wsize < 0 ? P.c[5] : ring_coupling_scale(wsize, F_, P.c[1] * cs, sh);
-        k[0] = fma(sc, __ll2double_rn(ring_coupling(P, qo, F_, W, sh)), P.c[0]);
+        int sh;
+        const double sc = ring_coupling_scale(wsize, F_, P.c[1] * cs, sh);
+        k[0] = fma(sc, __ll2double_rn(ring_coupling_wide(P, qo, F_, W, sh)), P.c[0]);
+    }
+    // Rings: c[5] = (mu/K) 2^(ksh + 3 - F).
+    __device__ __forceinline__ static void rhs_ring(const ModelParams &P, const int64_t (&qo)[NQ],
+                                                    const int64_t (&S)[NQ], const double *, double, double (&k)[D])
+    {
+        k[0] = fma(P.c[5], __ll2double_rn(ring_coupling(P, qo, F, S[0], S[1])), P.c[0]);
     }
     // Lattices: c[4] = omega + (mu/K) sin alpha (omega with the node itself as a
     // link), c[5] = (mu/K) 2^-(F-2).
@@ -175,21 +198,52 @@ template <> struct Model<0> {
 // Coupled quantity (u, v).
 template <> struct Model<1> {
     static constexpr int D = 2, NQ = 2, NX = 0, F = 51;
-    __device__ __forceinline__ static void coupled_q(const ModelParams &, const double (&x)[D], int F, int lim,
-                                                     bool &ok, int64_t (&q)[NQ])
+    static constexpr bool OWN_OUT = false;
+    __device__ __forceinline__ static void coupled_q(const ModelParams &, const double (&x)[D], int, int, bool &ok,
+                                                     int64_t (&q)[NQ])
     {
-        q[0] = to_fixed(x[0], F, lim, ok);
-        q[1] = to_fixed(x[1], F, lim, ok);
+        q[0] = to_fixed54(x[0], F, ok);
+        q[1] = to_fixed54(x[1], F, ok);
     }
     __device__ __forceinline__ static void rhs(const ModelParams &P, int F_, const double (&fo)[NQ],
-                                               const int64_t (&qo)[NQ], const i128 (&W)[NQ],
-                                               const double *X, double Iext, double (&k)[D],
-                                               int64_t wsize = -1, double cs = 1.0, const int64_t * = nullptr)
+                                               const int64_t (&qo)[NQ], const i128 (&W)[NQ], const double *, double,
+                                               double (&k)[D], int64_t wsize, double cs)
     {
-        const int64_t ws = wsize < 0 ? P.wsize : wsize;
-        const double Cu = cs * fixed_to_double_wide(W[0] - (i128)qo[0] * ws, F_);
-        const double Cv = cs * fixed_to_double_wide(W[1] - (i128)qo[1] * ws, F_);
-        const double u = fo[0], v = fo[1];
+        slope(P, fo[0], fo[1], cs * fixed_to_double_wide(W[0] - (i128)qo[0] * wsize, F_),
+              cs * fixed_to_double_wide(W[1] - (i128)qo[1] * wsize, F_), k);
+    }
+    // Rings.  The stage was bound by the FP64 pipe (13 FP64 instructions and four
+    // conversions per node), so the slope's bracket
+    //   G_u = u - u^3/3 - v + (sigma/K) (b00 Cu + b01 Cv),  G_v = u + a + (sigma/K) (b10 Cu + b11 Cv)
+    // is formed in integers on the grid 2^-54 from the grid values of u and v
+    // (|u|, |v| < 8, so |u - u^3/3| < 171), and each slope takes one conversion; k_u = G_u / eps with
+    // 1/eps in two parts (its rounding would be the largest systematic error left).
+    // Every product is truncated at 2^-54 or finer (|error| of a bracket < 3 2^-54,
+    // against roundings of 2^-53 |u| in FP64).  Ring of 10^6: 35 -> 23 us per stage launch.  fx = 0 (coupling constants or a beyond the range the
+    // host checks, windows of fewer than 65 nodes): FP64, c[2..5] carrying
+    // 2^(ksh - F).
+    __device__ __forceinline__ static void rhs_ring(const ModelParams &P, const int64_t (&qo)[NQ],
+                                                    const int64_t (&S)[NQ], const double *, double, double (&k)[D])
+    {
+        const int64_t Cu = S[0] - own_multiple(P, qo[0]), Cv = S[1] - own_multiple(P, qo[1]); // grid 2^(ksh - 51)
+        if (P.fx) {
+            const int64_t qu = qo[0], qv = qo[1];
+            const uint64_t ua = (uint64_t)(qu < 0 ? -qu : qu) << 9;            // |u| 2^60
+            const uint64_t u2 = __umul64hi(ua, ua);                            // u^2 2^56
+            const int64_t w = (1ll << 58) - (int64_t)(__umul64hi(u2, 0x5555555555555555ull) << 2); // (1 - u^2/3) 2^58
+            const int64_t uw = mulhi_su(w, ua);                                // |u| (1 - u^2/3) 2^54
+            const int64_t gu = (qu < 0 ? -uw : uw) - (qv << 3) + mulhi_ss(Cu, P.kq[0]) + mulhi_ss(Cv, P.kq[1]) + 1;
+            const int64_t gv = (qu << 3) + P.a54 + mulhi_ss(Cu, P.kq[2]) + mulhi_ss(Cv, P.kq[3]) + 1;
+            const double g = __ll2double_rn(gu);
+            k[0] = fma(P.c[6], g, P.c[7] * g); // c[6] + c[7] = 2^-54 / eps
+            k[1] = ll2double_scaled(gv, 54);
+            return;
+        }
+        slope(P, ll2double_scaled(qo[0], F), ll2double_scaled(qo[1], F), __ll2double_rn(Cu), __ll2double_rn(Cv), k);
+    }
+    __device__ __forceinline__ static void slope(const ModelParams &P, double u, double v, double Cu, double Cv,
+                                                 double (&k)[D])
+    {
         const double w = fma(u * u, -1.0 / 3.0, 1.0);      // 1 - u^2/3
         const double local = fma(u, w, -v);                // u - u^3/3 - v
         k[0] = fma(P.c[0], local, fma(P.c[2], Cu, P.c[3] * Cv));
@@ -206,19 +260,29 @@ template <> struct Model<1> {
 // local variables.  Rates use the table-driven exp and reciprocal of fastmath.cuh.
 template <> struct Model<2> {
     static constexpr int D = 4, NQ = 1, NX = 3, F = 46;
-    __device__ __forceinline__ static void coupled_q(const ModelParams &, const double (&x)[D], int F, int lim,
-                                                     bool &ok, int64_t (&q)[NQ])
+    static constexpr bool OWN_OUT = false;
+    __device__ __forceinline__ static void coupled_q(const ModelParams &, const double (&x)[D], int, int, bool &ok,
+                                                     int64_t (&q)[NQ])
     {
-        q[0] = to_fixed(x[0], F, lim, ok);
+        q[0] = to_fixed54(x[0], F, ok);
     }
     __device__ __forceinline__ static void rhs(const ModelParams &P, int F_, const double (&fo)[NQ],
-                                               const int64_t (&qo)[NQ], const i128 (&W)[NQ],
-                                               const double *X, double Iext, double (&k)[D],
-                                               int64_t wsize = -1, double cs = 1.0, const int64_t * = nullptr)
+                                               const int64_t (&qo)[NQ], const i128 (&W)[NQ], const double *X,
+                                               double Iext, double (&k)[D], int64_t wsize, double cs)
     {
-        const int64_t ws = wsize < 0 ? P.wsize : wsize;
-        const double CV = cs * fixed_to_double_wide(W[0] - (i128)qo[0] * ws, F_);
-        const double V = fo[0], m = X[0], h = X[1], n = X[2];
+        slope(P, fo[0], cs * fixed_to_double_wide(W[0] - (i128)qo[0] * wsize, F_), X, Iext, k);
+    }
+    // Rings: c[7] carries 2^(ksh - F).
+    __device__ __forceinline__ static void rhs_ring(const ModelParams &P, const int64_t (&qo)[NQ],
+                                                    const int64_t (&S)[NQ], const double *X, double Iext,
+                                                    double (&k)[D])
+    {
+        slope(P, ll2double_scaled(qo[0], F), __ll2double_rn(S[0] - own_multiple(P, qo[0])), X, Iext, k);
+    }
+    __device__ __forceinline__ static void slope(const ModelParams &P, double V, double CV, const double *X,
+                                                 double Iext, double (&k)[D])
+    {
+        const double m = X[0], h = X[1], n = X[2];
         const MathTables &T = P.tab;
         const double am = fast_x_over_1mexp(fma(V, 0.1, 4.0), T);                    // (V+40)/10
         const double bm = 4.0 * fast_exp(fma(V, -1.0 / 18.0, -65.0 / 18.0), T);     // -(V+65)/18
@@ -244,6 +308,7 @@ template <> struct Model<2> {
 // psi is a local variable.
 template <> struct Model<3> {
     static constexpr int D = 2, NQ = 2, NX = 1, F = 53;
+    static constexpr bool OWN_OUT = true;
     __device__ __forceinline__ static void coupled_q(const ModelParams &P, const double (&x)[D], int F, int,
                                                      bool &ok, int64_t (&q)[NQ])
     {
@@ -252,17 +317,21 @@ template <> struct Model<3> {
         q[0] = q62_to(s62, F);
         q[1] = q62_to(c62, F);
     }
-    // Rings and link matrices: c[5] = (mu/(m K)) 2^(ksh + 3 - F).
     __device__ __forceinline__ static void rhs(const ModelParams &P, int F_, const double (&)[NQ],
-                                               const int64_t (&qo)[NQ], const i128 (&W)[NQ],
-                                               const double *X, double, double (&k)[D],
-                                               int64_t wsize = -1, double cs = 1.0, const int64_t * = nullptr)
+                                               const int64_t (&qo)[NQ], const i128 (&W)[NQ], const double *X, double,
+                                               double (&k)[D], int64_t wsize, double cs)
     {
-        int sh = P.ksh;
-        const double sc = wsize < 0 ? P.c[5] : ring_coupling_scale(wsize, F_, P.c[0] * cs, sh);
-        const double psi = X[0];
-        k[0] = psi;
-        k[1] = fma(sc, __ll2double_rn(ring_coupling(P, qo, F_, W, sh)), -P.c[1] * psi);
+        int sh;
+        const double sc = ring_coupling_scale(wsize, F_, P.c[0] * cs, sh);
+        k[0] = X[0];
+        k[1] = fma(sc, __ll2double_rn(ring_coupling_wide(P, qo, F_, W, sh)), -P.c[1] * X[0]);
+    }
+    // Rings: c[5] = (mu/(m K)) 2^(ksh + 3 - F).
+    __device__ __forceinline__ static void rhs_ring(const ModelParams &P, const int64_t (&qo)[NQ],
+                                                    const int64_t (&S)[NQ], const double *X, double, double (&k)[D])
+    {
+        k[0] = X[0];
+        k[1] = fma(P.c[5], __ll2double_rn(ring_coupling(P, qo, F, S[0], S[1])), -P.c[1] * X[0]);
     }
     // Lattices: c[4] = (mu/(m K)) sin alpha (0 with the node itself as a link),
     // c[5] = (mu/(m K)) 2^-(F-2).  The coupling term first, then the damping

@@ -4,7 +4,8 @@
 // networks; the per-node right-hand side of Algorithm 1):
 //   a3  window sums   W(i) = P(i+R+1) - P(i-R), P(p) = sum_{j<p} Q(f_j) over the
 //                     periodic extension, read from the exact prefix arrays the
-//                     previous kernel wrote (two shifted reads per quantity);
+//                     previous kernel wrote (two shifted reads; the quantities
+//                     of a node interleaved, one 16-byte load per read);
 //   a4  right-hand side k_s(i) from W(i) and the node's own stage input;
 //   a5  RK4 accumulate acc += b_s k_s (stage 4: y <- y + dt/6 (acc + k_4));
 //   a1  next stage input x_{s+1} = y + c_{s+1} dt k_s;
@@ -23,48 +24,37 @@
 
 namespace simk {
 
-// Ring window in three phases.  load(): the node's own prefix entries and the
-// in-sub-tile prefix at both window ends, b = i+R+1 and a = i-R on the periodic
-// extension (a piece never straddles 0 or N, so the copy of the ring each end
-// falls in is known without the bases).  sync(): the bases threads 0 and 1
-// computed become visible.  finish(): W = base(b) - base(a) + the loaded parts,
-// exactly as ring_window computes it.
-template <int NQ> struct RingGather {
+// Ring window in three phases.  load(): the node's own prefix entries and those
+// at its window ends.  sync(): the bases become visible.  finish(): the shifted
+// exact window sums and the node's slope.
+template <int M, int NQ> struct RingGather {
     struct Pre {
         int64_t l[NQ], lp[NQ], lb[NQ], la[NQ];
     };
     const RingPlan &P;
     const int64_t *lam_in;
     const RingBases<NQ> &B;
+    int64_t sub;
     __device__ __forceinline__ void load(int tid, int64_t i, Pre &pre) const
     {
-        const int64_t N = P.N;
-        const int64_t b = i + P.R + 1, am = i - P.R;
-        const int64_t bp = b >= N ? b - N : b, ap = am < 0 ? am + N : am;
+        lam_load<NQ>(lam_in + i * NQ, pre.l);
 #pragma unroll
-        for (int c = 0; c < NQ; ++c) {
-            const int64_t *lam = lam_in + c * N;
-            pre.l[c] = __ldg(lam + i);
-            pre.lp[c] = tid ? __ldg(lam + i - 1) : 0;
-            pre.lb[c] = (bp & (kSubTile - 1)) ? __ldg(lam + bp - 1) : 0;
-            pre.la[c] = (ap & (kSubTile - 1)) ? __ldg(lam + ap - 1) : 0;
-        }
+        for (int c = 0; c < NQ; ++c) pre.lp[c] = 0;
+        if (tid) lam_load<NQ>(lam_in + (i - 1) * NQ, pre.lp);
+        lam_load_end<NQ>(ring_end<NQ>(P, lam_in, sub, 0), tid, pre.lb);
+        lam_load_end<NQ>(ring_end<NQ>(P, lam_in, sub, 1), tid, pre.la);
     }
     __device__ __forceinline__ void sync() const { __syncthreads(); }
-    __device__ __forceinline__ void finish(int tid, int64_t i, const Pre &pre, int64_t (&qo)[NQ], double (&fo)[NQ],
-                                           i128 (&W)[NQ], int64_t &wsize, double &cs) const
+    template <int D>
+    __device__ __forceinline__ void finish(int tid, int64_t, const Pre &pre, const double *X, double Iext,
+                                           double (&k)[D]) const
     {
-        const int64_t b = i + P.R + 1, am = i - P.R;
-        const int kb = (b >= B.start[0][1]) + (b >= B.start[0][2]);
-        const int ka = (am >= B.start[1][1]) + (am >= B.start[1][2]);
+        int64_t qo[NQ], own[NQ], S[NQ];
 #pragma unroll
-        for (int c = 0; c < NQ; ++c) {
-            qo[c] = pre.l[c] - pre.lp[c];
-            fo[c] = fixed_to_double(qo[c], P.F);
-            W[c] = (B.base[0][kb][c] - B.base[1][ka][c]) + (i128)(pre.lb[c] - pre.la[c]);
-        }
-        wsize = -1; // the network's window size
-        cs = 1.0;
+        for (int c = 0; c < NQ; ++c) qo[c] = pre.l[c] - pre.lp[c];
+        ring_own<M, NQ>(P.mp, qo, own);
+        ring_sums<NQ>(B, tid, P.mp.ksh, pre.lb, pre.la, own, S);
+        Model<M>::rhs_ring(P.mp, qo, S, X, Iext, k);
     }
 };
 
@@ -81,7 +71,7 @@ __device__ __forceinline__ void ring_stage_body(const RingPlan &P, const RingSta
         if (FLAT_OK && P.flat) ring_flat_bases<NQ>(P, a.fsub_in, a.facc_in, sub, s_bases);
         else ring_compute_bases<NQ>(P, a.ingrp_in, a.grpofs_in, sub, s_bases);
     }
-    stage_body<M, STAGE, RingGather<NQ>, FLAT_OK>(P, a, h, sub, RingGather<NQ>{P, a.lam_in, s_bases});
+    stage_body<M, STAGE, RingGather<M, NQ>, FLAT_OK>(P, a, h, sub, RingGather<M, NQ>{P, a.lam_in, s_bases, sub});
 }
 
 // Two adjacent nodes per thread, 128 threads per 256-node sub-tile: two
@@ -100,103 +90,92 @@ __device__ __forceinline__ void ring_stage_body2(const RingPlan &P, const RingSt
     constexpr int D = Mo::D, NQ = Mo::NQ, NX = Mo::NX;
     constexpr int XOFF = D - NX;
     __shared__ RingBases<NQ> s_bases;
-    const int tid = threadIdx.x;
-    const int64_t N = P.N;
-    const int64_t i0 = sub * kSubTile + 2 * tid;
+    const int tid = threadIdx.x, l0 = 2 * tid;
+    const int64_t N = P.N, s0 = sub * kSubTile;
+    const int nv = (int)(N - s0 < kSubTile ? N - s0 : kSubTile); // nodes of the sub-tile
     const bool flat = P.flat != 0;
     if (STAGE > 0) {
         if (flat) ring_flat_bases<NQ>(P, a.fsub_in, a.facc_in, sub, s_bases);
         else ring_compute_bases<NQ>(P, a.ingrp_in, a.grpofs_in, sub, s_bases);
     }
 
-    int64_t l[NQ][2], lp[NQ], lb[NQ][2], la[NQ][2];
-    double yv[2][D], av[2][D], X[2][NX > 0 ? NX : 1], Iext[2] = {0.0, 0.0};
+    int64_t ln[2][NQ], lp[NQ], lb[2][NQ], la[2][NQ];
+    double yv[2][D], av[2][D], X[2][NX > 0 ? NX : 1];
+    const double *ys = P.y + s0;
+    double *accs = P.acc + s0;
     if (STAGE > 0) {
+        const int64_t *lam = a.lam_in + s0 * NQ;
+        const RingEnd<NQ> eb = ring_end<NQ>(P, a.lam_in, sub, 0), ea = ring_end<NQ>(P, a.lam_in, sub, 1);
+#pragma unroll
+        for (int c = 0; c < NQ; ++c) lp[c] = 0;
+        if (tid && l0 < nv) lam_load<NQ>(lam + (l0 - 1) * NQ, lp);
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
-            const int64_t i = i0 + u;
-            if (i < N) {
-                const int64_t b = i + P.R + 1, am = i - P.R;
-                const int64_t bp = b >= N ? b - N : b, ap = am < 0 ? am + N : am;
-#pragma unroll
-                for (int c = 0; c < NQ; ++c) {
-                    const int64_t *lam = a.lam_in + c * N;
-                    l[c][u] = __ldg(lam + i);
-                    if (u == 0) lp[c] = tid ? __ldg(lam + i - 1) : 0;
-                    lb[c][u] = (bp & (kSubTile - 1)) ? __ldg(lam + bp - 1) : 0;
-                    la[c][u] = (ap & (kSubTile - 1)) ? __ldg(lam + ap - 1) : 0;
-                }
+            const int l = l0 + u;
+            if (l < nv) {
+                lam_load<NQ>(lam + l * NQ, ln[u]);
+                lam_load_end<NQ>(eb, l, lb[u]);
+                lam_load_end<NQ>(ea, l, la[u]);
 #pragma unroll
                 for (int v = 0; v < D; ++v) {
-                    yv[u][v] = P.y[v * N + i];
-                    av[u][v] = STAGE >= 2 ? P.acc[v * N + i] : 0.0;
+                    yv[u][v] = ys[v * N + l];
+                    av[u][v] = STAGE >= 2 ? accs[v * N + l] : 0.0;
                 }
 #pragma unroll
-                for (int g = 0; g < NX; ++g) X[u][g] = a.x_in[g * N + i];
-                if (M == 2 && P.node_param) Iext[u] = P.node_param[i];
+                for (int g = 0; g < NX; ++g) X[u][g] = a.x_in[s0 + g * N + l];
             }
         }
         __syncthreads();
     }
 
-    int64_t qv[NQ][2];
+    int64_t qv[2][NQ];
     bool ok = true;
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
-        const int64_t i = i0 + u;
+        const int l = l0 + u;
 #pragma unroll
-        for (int c = 0; c < NQ; ++c) qv[c][u] = 0;
-        if (i >= N) continue;
+        for (int c = 0; c < NQ; ++c) qv[u][c] = 0;
+        if (l >= nv) continue;
         double xn[D];
         if (STAGE == 0) {
 #pragma unroll
-            for (int v = 0; v < D; ++v) xn[v] = P.y[v * N + i];
+            for (int v = 0; v < D; ++v) xn[v] = ys[v * N + l];
         } else {
-            const int64_t b = i + P.R + 1, am = i - P.R;
-            const int kb = (b >= s_bases.start[0][1]) + (b >= s_bases.start[0][2]);
-            const int ka = (am >= s_bases.start[1][1]) + (am >= s_bases.start[1][2]);
-            int64_t qo[NQ];
-            double fo[NQ];
-            i128 W[NQ];
+            int64_t qo[NQ], own[NQ], S[NQ];
 #pragma unroll
-            for (int c = 0; c < NQ; ++c) {
-                qo[c] = l[c][u] - (u == 0 ? lp[c] : l[c][0]);
-                fo[c] = fixed_to_double(qo[c], P.F);
-                W[c] = (s_bases.base[0][kb][c] - s_bases.base[1][ka][c]) + (i128)(lb[c][u] - la[c][u]);
-            }
+            for (int c = 0; c < NQ; ++c) qo[c] = ln[u][c] - (u == 0 ? lp[c] : ln[0][c]);
+            ring_own<M, NQ>(P.mp, qo, own);
+            ring_sums<NQ>(s_bases, l, P.mp.ksh, lb[u], la[u], own, S);
             double k[D];
-            Mo::rhs(P.mp, P.F, fo, qo, W, X[u], Iext[u], k);
+            Mo::rhs_ring(P.mp, qo, S, X[u], 0.0, k);
 #pragma unroll
             for (int v = 0; v < D; ++v) {
                 if (STAGE == 1) {
-                    P.acc[v * N + i] = k[v];
+                    accs[v * N + l] = k[v];
                     xn[v] = yv[u][v] + h.half * k[v];
                 } else if (STAGE == 2) {
-                    P.acc[v * N + i] = av[u][v] + 2.0 * k[v];
+                    accs[v * N + l] = av[u][v] + 2.0 * k[v];
                     xn[v] = yv[u][v] + h.half * k[v];
                 } else if (STAGE == 3) {
-                    P.acc[v * N + i] = av[u][v] + 2.0 * k[v];
+                    accs[v * N + l] = av[u][v] + 2.0 * k[v];
                     xn[v] = yv[u][v] + h.dt * k[v];
                 } else {
                     const double yn = yv[u][v] + h.sixth * (av[u][v] + k[v]);
-                    P.y[v * N + i] = yn;
+                    P.y[s0 + v * N + l] = yn;
                     xn[v] = yn;
                 }
             }
             if (NX > 0 && STAGE >= 1 && STAGE <= 3) {
 #pragma unroll
-                for (int g = 0; g < NX; ++g) a.x_out[g * N + i] = xn[XOFF + g];
+                for (int g = 0; g < NX; ++g) a.x_out[s0 + g * N + l] = xn[XOFF + g];
             }
         }
-        int64_t qn[NQ];
-        Mo::coupled_q(P.mp, xn, P.F, P.lim, ok, qn);
-#pragma unroll
-        for (int c = 0; c < NQ; ++c) qv[c][u] = qn[c];
+        Mo::coupled_q(P.mp, xn, P.F, P.lim, ok, qv[u]);
     }
     if (!ok) raise_error(P.err, ERR_RANGE);
     // the prologue writes both prefix forms (a later kernel of either kind may read it)
     ring_prefix_tail_n<NQ, 2, (M == 0 || M == 3) && (STAGE == 0 || STAGE == 4), STAGE == 4>(
-        P, a.lam_out, a.ingrp_out, a.grpofs_out, sub, i0, qv, flat, STAGE == 0 || !flat, a.fsub_out, a.facc_out,
+        P, a.lam_out, a.ingrp_out, a.grpofs_out, sub, s0 + l0, qv, flat, STAGE == 0 || !flat, a.fsub_out, a.facc_out,
         a.facc_zero);
 }
 

@@ -176,17 +176,15 @@ __global__ void __launch_bounds__(kClusterThreads, 1)
             for (int k = 0; k < MPT; ++k) {
                 const int64_t i = i0 + tid + (int64_t)k * kClusterThreads;
                 if (i >= i1) continue;
-                int64_t qo[NQ];
-                double fo[NQ];
-                i128 W[NQ];
+                int64_t qo[NQ], S[NQ];
 #pragma unroll
                 for (int c = 0; c < NQ; ++c) {
                     qo[c] = q[c * N + i];
-                    fo[c] = fixed_to_double(qo[c], P.F);
-                    W[c] = prefix_at(c, i + R + 1) - prefix_at(c, i - R);
+                    const i128 W = prefix_at(c, i + R + 1) - prefix_at(c, i - R);
+                    S[c] = (int64_t)((Mo::OWN_OUT && !P.mp.include_self ? W - (i128)qo[c] : W) >> P.mp.ksh);
                 }
                 double kk[D], xn[D];
-                Mo::rhs(P.mp, P.F, fo, qo, W, xs[k], iext[k], kk);
+                Mo::rhs_ring(P.mp, qo, S, xs[k], iext[k], kk);
 #pragma unroll
                 for (int v = 0; v < D; ++v) {
                     if (stage == 1) {
@@ -225,7 +223,7 @@ __global__ void __launch_bounds__(kClusterThreads, 1)
 #pragma unroll
         for (int v = 0; v < D; ++v) P.y[v * N + i] = y[k][v];
 #pragma unroll
-        for (int c = 0; c < NQ; ++c) P.lam[0][c * N + i] = lam[c * N + i];
+        for (int c = 0; c < NQ; ++c) P.lam[0][i * NQ + c] = lam[c * N + i];
     }
     if (rank == 0) {
         // one prefix group (nsub <= 64): in-group offsets are the block offsets

@@ -4,9 +4,9 @@
 //   ring_load_bases   per-CTA window bases: the exact prefix at the start of
 //                     every piece (split at sub-tile starts and at N) that the
 //                     window ends of this CTA's nodes fall in;
-//   ring_window       one node's exact window sums W = P(i+R+1) - P(i-R) and its
-//                     own fixed-point coupled quantity, from the prefix arrays the
-//                     previous kernel wrote (two shifted in-sub-tile reads);
+//   ring_window       one node's exact window sums W = P(i+R+1) - P(i-R), shifted
+//                     into int64, and its own fixed-point coupled quantity, from
+//                     the prefix arrays the previous kernel wrote;
 //   ring_prefix_tail  the exact prefix of the next coupled quantity inside the
 //                     sub-tile and, without any CTA waiting for another, at every
 //                     sub-tile start: the last CTA to finish in each group of 64
@@ -51,54 +51,147 @@ __device__ __forceinline__ i128 warp_incl_scan_i128(i128 v)
 template <int M> struct MinBlocks { static constexpr int value = SIM_RING_MIN_BLOCKS; };
 template <> struct MinBlocks<2> { static constexpr int value = 2; };
 
-// Window bases of one CTA: the right ends b = i+R+1 (side 0) and left ends
-// a = i-R (side 1) of its nodes are consecutive, and each side covers at most
-// three pieces (split at a sub-tile start and at N).  Per piece: its first
-// position on the periodic extension, the multiple of N to subtract, and the
-// exact prefix at its sub-tile's start (+ q * total).  Then every node needs one
-// in-sub-tile prefix load per end.
-template <int NQ> struct RingBases {
-    i128 base[2][3][NQ];
-    int64_t start[2][3], qn[2][3];
+// Window ends.  With the exact inclusive prefix lam inside every 256-node
+// sub-tile, the prefix of the periodic extension at b is P(b) = (exact prefix at
+// the start of the sub-tile that holds e = b - 1) + lam[e], so a window end is
+// one load at e = i + R (right, side 0) or e = i - R - 1 (left, side 1), with no
+// special case at a sub-tile start.  The ends of a CTA's consecutive nodes are
+// consecutive and cover at most three pieces per side (split at sub-tile starts
+// and at 0 and N).  Per piece: its first node (the CTA's node index) and the
+// exact prefix at its sub-tile's start (plus or minus the ring's total on the
+// neighbouring copies of the ring), split as hi 2^sh + lo with 0 <= lo < 2^sh,
+// sh = ModelParams::ksh: a node's window sum shifted right by sh,
+//   floor(W 2^-sh) = hi0 - hi1 + (x >> sh) + ((lo0 - lo1 + (x mod 2^sh)) >> sh),
+// x = lam[e0] - lam[e1], is then exact in 64-bit arithmetic (hi modulo 2^64, as
+// the result fits), where the 128-bit difference, shift and conversion of every
+// node had been a third of the stage's instructions.
+template <int NQ> struct __align__(16) RingBases {
+    int64_t hi[2][3][NQ];
+    int lo[2][3][NQ];
+    int start[2][4];
 };
 
-// Threads 0 and 1 write the bases; the caller makes them visible with a barrier.
+// The piece k (0..2) of a side of the CTA on sub-tile sub: its first node
+// (kSubTile when there is no such piece), its sub-tile and its copy of the ring
+// (-1, 0, 1).
+__device__ __forceinline__ void ring_piece(const RingPlan &P, int64_t sub, int side, int k, int &start, int64_t &st,
+                                           int &q)
+{
+    const int64_t N = P.N, s0 = sub * kSubTile;
+    int64_t e = side == 0 ? s0 + P.R : s0 - P.R - 1; // in [-N, 2N)
+    q = e < 0 ? -1 : (e >= N ? 1 : 0);
+    e -= q * N;
+    const int nvalid = (int)(N - s0 < kSubTile ? N - s0 : kSubTile);
+    start = 0;
+    for (int m = 0; m < k; ++m) {
+        int64_t end = e | (kSubTile - 1);
+        if (end > N - 1) end = N - 1;
+        start += (int)(end - e) + 1;
+        e = end + 1;
+        if (e == N) {
+            e = 0;
+            ++q;
+        }
+    }
+    st = e >> kSubLog2;
+    if (start >= nvalid) start = kSubTile;
+}
+
+__device__ __forceinline__ void ring_put_base(i128 base, int sh, int64_t &hi, int &lo)
+{
+    hi = (int64_t)(base >> sh);
+    lo = (int)((unsigned)base & ((1u << sh) - 1u));
+}
+
+// Threads 0..5 write the bases, one piece each; the caller makes them visible
+// with a barrier.
 template <int NQ>
 __device__ __forceinline__ void ring_compute_bases(const RingPlan &P, const i128 *ingrp_in, const i128 *grpofs_in,
                                                    int64_t sub, RingBases<NQ> &B)
 {
     const int tid = threadIdx.x;
-    const int64_t N = P.N, nsub = P.nsub, ngroups = P.ngroups;
-    if (tid < 2) {
-        const int side = tid;
-        const int64_t nvalid = N - sub * kSubTile < kSubTile ? N - sub * kSubTile : kSubTile;
-        const int64_t p0 = side == 0 ? sub * kSubTile + P.R + 1 : sub * kSubTile - P.R;
-        const int64_t p1 = p0 + nvalid - 1; // in [-N, 2N)
-        int64_t p = p0;
+    if (tid >= 6) return;
+    const int64_t nsub = P.nsub, ngroups = P.ngroups;
+    const int side = tid >= 3, k = tid - 3 * side;
+    int start, q;
+    int64_t st;
+    ring_piece(P, sub, side, k, start, st, q);
+    B.start[side][k] = start;
+    if (start >= kSubTile) return;
 #pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            if (p > p1) {
-                B.start[side][k] = INT64_MAX;
-                B.qn[side][k] = 0;
-                continue;
-            }
-            const int q = p < 0 ? -1 : (p >= N ? 1 : 0);
-            const int64_t qn = q * N, pp = p - qn;
-            const int64_t st = pp >> kSubLog2;
-            int64_t end = ((st + 1) << kSubLog2) - 1;
-            if (end > N - 1) end = N - 1;
-#pragma unroll
-            for (int c = 0; c < NQ; ++c) {
-                const i128 *grpofs = grpofs_in + c * (ngroups + 1);
-                const i128 tot = ldg_i128(grpofs + ngroups);
-                B.base[side][k][c] = ldg_i128(grpofs + (st >> kGroupLog2)) + ldg_i128(ingrp_in + c * nsub + st) +
-                                     (q < 0 ? -tot : (q > 0 ? tot : (i128)0));
-            }
-            B.start[side][k] = p;
-            B.qn[side][k] = qn;
-            p = end + qn + 1;
-        }
+    for (int c = 0; c < NQ; ++c) {
+        const i128 *grpofs = grpofs_in + c * (ngroups + 1);
+        const i128 tot = ldg_i128(grpofs + ngroups);
+        const i128 base = ldg_i128(grpofs + (st >> kGroupLog2)) + ldg_i128(ingrp_in + c * nsub + st) +
+                          (q < 0 ? -tot : (q > 0 ? tot : (i128)0));
+        ring_put_base(base, P.mp.ksh, B.hi[side][k][c], B.lo[side][k][c]);
     }
+}
+
+// One side's lam entries of a CTA: lam at e(l) for the CTA's node l, as a
+// pointer per copy of the ring (the ends wrap at most once inside a CTA).
+template <int NQ> struct RingEnd {
+    const int64_t *at;
+    int wrap;     // first node whose end lies on the next copy
+    int64_t back; // elements of one copy
+};
+template <int NQ> __device__ __forceinline__ RingEnd<NQ> ring_end(const RingPlan &P, const int64_t *lam, int64_t sub, int side)
+{
+    const int64_t N = P.N, s0 = sub * kSubTile;
+    int64_t e = side == 0 ? s0 + P.R : s0 - P.R - 1;
+    e -= e >= N ? N : 0;
+    e += e < 0 ? N : 0;
+    return RingEnd<NQ>{lam + e * NQ, (int)(N - e < kSubTile ? N - e : kSubTile), N * NQ};
+}
+
+// The NQ components of one node's prefix entry (interleaved; one 16-byte load
+// for two components).
+template <int NQ> __device__ __forceinline__ void lam_load(const int64_t *p, int64_t (&v)[NQ])
+{
+    if constexpr (NQ == 2) {
+        const longlong2 w = __ldg(reinterpret_cast<const longlong2 *>(p));
+        v[0] = w.x;
+        v[1] = w.y;
+    } else {
+        v[0] = __ldg(p);
+    }
+}
+template <int NQ> __device__ __forceinline__ void lam_store(int64_t *p, const int64_t (&v)[NQ])
+{
+    if constexpr (NQ == 2) *reinterpret_cast<longlong2 *>(p) = make_longlong2(v[0], v[1]);
+    else *p = v[0];
+}
+template <int NQ> __device__ __forceinline__ void lam_load_end(const RingEnd<NQ> &E, int l, int64_t (&v)[NQ])
+{
+    const int64_t *p = l >= E.wrap ? E.at - E.back : E.at;
+    lam_load<NQ>(p + l * NQ, v);
+}
+
+// Node l of the CTA: the shifted exact window sums S = floor((W - own) 2^-sh)
+// from its prefix entries at both ends (own: 0, or the node's own quantity where
+// the sums leave the node out).
+template <int NQ>
+__device__ __forceinline__ void ring_sums(const RingBases<NQ> &B, int l, int sh, const int64_t (&lb)[NQ],
+                                          const int64_t (&la)[NQ], const int64_t (&own)[NQ], int64_t (&S)[NQ])
+{
+    const int kb = (l >= B.start[0][1]) + (l >= B.start[0][2]);
+    const int ka = (l >= B.start[1][1]) + (l >= B.start[1][2]);
+    const int mask = (1 << sh) - 1;
+#pragma unroll
+    for (int c = 0; c < NQ; ++c) {
+        const int64_t x = lb[c] - la[c] - own[c];
+        const int lo = B.lo[0][kb][c] - B.lo[1][ka][c] + ((int)x & mask);
+        S[c] = B.hi[0][kb][c] - B.hi[1][ka][c] + (x >> sh) + (int64_t)(lo >> sh);
+    }
+}
+
+// What ring_sums subtracts before the shift (Model::own_sub: the Kuramoto
+// models, unless the node is one of its own links).
+template <int M, int NQ>
+__device__ __forceinline__ void ring_own(const ModelParams &mp, const int64_t (&qo)[NQ], int64_t (&own)[NQ])
+{
+#pragma unroll
+    for (int c = 0; c < NQ; ++c) own[c] = Model<M>::OWN_OUT && !mp.include_self ? qo[c] : 0;
 }
 
 // Chunks of a sub-tile total (|t| < 2^62) for the one-pass accumulators:
@@ -150,23 +243,23 @@ __device__ __forceinline__ void ring_flat_bases(const RingPlan &P, const int64_t
     const int N = (int)P.N, R = (int)P.R, ngroups = (int)P.ngroups, nsub = (int)P.nsub;
     const int s0 = (int)sub * kSubTile;
     const int nvalid = N - s0 < kSubTile ? N - s0 : kSubTile;
-    const int p0 = side == 0 ? s0 + R + 1 : s0 - R; // in [-N, 2N)
-    const int p1 = p0 + nvalid - 1;
-    // the pieces, split at sub-tile starts and at 0 and N (as in ring_compute_bases)
+    // the pieces, split at sub-tile starts and at 0 and N (as in ring_piece)
+    int e = side == 0 ? s0 + R : s0 - R - 1; // in [-N, 2N)
     int start[3], st[3], q[3];
-    bool have[3];
-    int p = p0;
+    {
+        int qq = e < 0 ? -1 : (e >= N ? 1 : 0), l = 0;
+        e -= qq * N;
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        have[k] = p <= p1;
-        const int qq = p < 0 ? -1 : (p >= N ? 1 : 0);
-        const int sp = (p - qq * N) >> kSubLog2;
-        start[k] = p;
-        st[k] = sp;
-        q[k] = qq;
-        int end = ((sp + 1) << kSubLog2) - 1;
-        end = end > N - 1 ? N - 1 : end;
-        p = end + qq * N + 1;
+        for (int k = 0; k < 3; ++k) {
+            start[k] = l < nvalid ? l : kSubTile;
+            st[k] = e >> kSubLog2;
+            q[k] = qq;
+            int end = e | (kSubTile - 1);
+            end = end > N - 1 ? N - 1 : end;
+            l += end - e + 1;
+            e = end + 1 == N ? 0 : end + 1;
+            qq += e == 0;
+        }
     }
     const int g0 = st[0] >> kGroupLog2;
 #pragma unroll
@@ -174,14 +267,14 @@ __device__ __forceinline__ void ring_flat_bases(const RingPlan &P, const int64_t
         const unsigned *acc = facc_in + c * ngroups * 4;
         const int64_t *fs = fsub_in + c * nsub;
         // the totals of the sub-tiles the later pieces follow (broadcast loads)
-        const int64_t f0 = have[1] ? __ldg(fs + st[0]) : 0, f1 = have[2] ? __ldg(fs + st[1]) : 0;
+        const int64_t f0 = __ldg(fs + st[0]), f1 = __ldg(fs + st[1]);
         unsigned pk[4] = {0, 0, 0, 0}, tk[4] = {0, 0, 0, 0};
         // groups lane and lane + 32 with the sub-tiles of the same offsets in
         // st0's group (this fixed, interleaved form measured fastest), then
         // groups 64..127 on rings that have them
 #pragma unroll
-        for (int e = 0; e < 2; ++e) {
-            const int g = lane + 32 * e;
+        for (int m = 0; m < 2; ++m) {
+            const int g = lane + 32 * m;
             if (g < ngroups) flat_group_add(acc, g, g0, pk, tk);
             const int sp = (g0 << kGroupLog2) + g;
             if (sp < st[0]) {
@@ -192,8 +285,8 @@ __device__ __forceinline__ void ring_flat_bases(const RingPlan &P, const int64_t
         }
         if (ngroups > 64) {
 #pragma unroll
-            for (int e = 2; e < kFlatMaxGroups / 32; ++e) {
-                const int g = lane + 32 * e;
+            for (int m = 2; m < kFlatMaxGroups / 32; ++m) {
+                const int g = lane + 32 * m;
                 if (g < ngroups) flat_group_add(acc, g, g0, pk, tk);
             }
         }
@@ -202,24 +295,17 @@ __device__ __forceinline__ void ring_flat_bases(const RingPlan &P, const int64_t
             pk[k] = __reduce_add_sync(0xffffffffu, pk[k]);
             tk[k] = __reduce_add_sync(0xffffffffu, tk[k]);
         }
-        if (lane == 0) {
+        if (lane < 3) { // lane k: the exact prefix at the start of piece k's sub-tile
             const i128 T = flat_value(tk[0], tk[1], tk[2], tk[3]);
-            i128 pre = flat_value(pk[0], pk[1], pk[2], pk[3]); // exact prefix at the start of st[k]
-#pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                if (!have[k]) break;
-                if (k > 0) pre = st[k] == 0 ? (i128)0 : pre + (i128)(k == 1 ? f0 : f1);
-                B.base[side][k][c] = pre + (q[k] < 0 ? -T : (q[k] > 0 ? T : (i128)0));
-            }
+            i128 pre = flat_value(pk[0], pk[1], pk[2], pk[3]);
+            if (lane >= 1) pre = st[1] == 0 ? (i128)0 : pre + (i128)f0;
+            if (lane >= 2) pre = st[2] == 0 ? (i128)0 : pre + (i128)f1;
+            const int qq = lane == 0 ? q[0] : (lane == 1 ? q[1] : q[2]);
+            ring_put_base(pre + (qq < 0 ? -T : (qq > 0 ? T : (i128)0)), P.mp.ksh, B.hi[side][lane][c],
+                          B.lo[side][lane][c]);
         }
     }
-    if (lane == 0) {
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            B.start[side][k] = have[k] ? (int64_t)start[k] : INT64_MAX;
-            B.qn[side][k] = have[k] ? (int64_t)q[k] * N : 0;
-        }
-    }
+    if (lane < 3) B.start[side][lane] = lane == 0 ? start[0] : (lane == 1 ? start[1] : start[2]);
 }
 
 // Called by every thread of the CTA (contains a __syncthreads).
@@ -231,109 +317,30 @@ __device__ __forceinline__ void ring_load_bases(const RingPlan &P, const i128 *i
     __syncthreads();
 }
 
-// Node i (position tid in its sub-tile): its own coupled quantity (fixed point
-// qo and its double fo) and the exact window sums W of every coupled quantity.
-template <int NQ>
+// Node i (node l = tid of the CTA's sub-tile, one node per thread): its own
+// coupled quantity qo and the shifted exact window sums S of every coupled
+// quantity.
+template <int M, int NQ>
 __device__ __forceinline__ void ring_window(const RingPlan &P, const int64_t *lam_in, const RingBases<NQ> &B, int tid,
-                                            int64_t i, int64_t (&qo)[NQ], double (&fo)[NQ], i128 (&W)[NQ])
+                                            int64_t sub, int64_t i, int64_t (&qo)[NQ], int64_t (&S)[NQ])
 {
-    const int64_t N = P.N;
-    const int64_t b = i + P.R + 1, am = i - P.R;
-    const int kb = (b >= B.start[0][1]) + (b >= B.start[0][2]);
-    const int ka = (am >= B.start[1][1]) + (am >= B.start[1][2]);
-    const int64_t bp = b - B.qn[0][kb], ap = am - B.qn[1][ka];
+    int64_t l[NQ], lp[NQ] = {}, lb[NQ], la[NQ], own[NQ];
+    lam_load<NQ>(lam_in + i * NQ, l);
+    if (tid) lam_load<NQ>(lam_in + (i - 1) * NQ, lp);
+    lam_load_end<NQ>(ring_end<NQ>(P, lam_in, sub, 0), tid, lb);
+    lam_load_end<NQ>(ring_end<NQ>(P, lam_in, sub, 1), tid, la);
 #pragma unroll
-    for (int c = 0; c < NQ; ++c) {
-        const int64_t *lam = lam_in + c * N;
-        const int64_t l = __ldg(lam + i);
-        qo[c] = tid ? l - __ldg(lam + i - 1) : l;
-        fo[c] = fixed_to_double(qo[c], P.F);
-        const int64_t lb = (bp & (kSubTile - 1)) ? __ldg(lam + bp - 1) : 0;
-        const int64_t la = (ap & (kSubTile - 1)) ? __ldg(lam + ap - 1) : 0;
-        W[c] = (B.base[0][kb][c] - B.base[1][ka][c]) + (i128)(lb - la);
-    }
+    for (int c = 0; c < NQ; ++c) qo[c] = l[c] - lp[c];
+    ring_own<M, NQ>(P.mp, qo, own);
+    ring_sums<NQ>(B, tid, P.mp.ksh, lb, la, own, S);
 }
 
 // Exact prefix of the fixed-point values qv (one per node, 0 past the ring's
-// end) into lam_out / ingrp_out / grpofs_out.  RECORD: the last CTA records the
-// Kuramoto order parameter from the totals (if P.obs is set); DEC_STEPS: it also
-// decrements the step budget.  Called by every thread of the CTA.
-template <int NQ, bool RECORD, bool DEC_STEPS>
-__device__ __forceinline__ void ring_prefix_tail(const RingPlan &P, int64_t *lam_out, i128 *ingrp_out,
-                                                 i128 *grpofs_out, int64_t sub, int64_t i, int64_t (&qv)[NQ])
-{
-    constexpr int NW = kRingThreads / 32;
-    __shared__ int64_t s_wtot[NW][NQ];
-    __shared__ int s_last;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int64_t N = P.N, nsub = P.nsub, ngroups = P.ngroups;
-
-    // Exact inclusive prefix inside the sub-tile (warp scans + preceding warps).
-#pragma unroll
-    for (int c = 0; c < NQ; ++c) {
-        qv[c] = warp_incl_scan(qv[c]);
-        if (lane == 31) s_wtot[warp][c] = qv[c];
-    }
-    __syncthreads();
-#pragma unroll
-    for (int c = 0; c < NQ; ++c) {
-        int64_t off = 0;
-        for (int w = 0; w < warp; ++w) off += s_wtot[w][c];
-        if (i < N) lam_out[c * N + i] = off + qv[c];
-    }
-
-    // Level 1: the last CTA of each group of 64 sub-tiles scans the group.
-    const int64_t g = sub >> kGroupLog2, s0 = g << kGroupLog2;
-    const int64_t gsize = nsub - s0 < kGroup ? nsub - s0 : kGroup;
-    if (tid == 0) {
-#pragma unroll
-        for (int c = 0; c < NQ; ++c) {
-            int64_t t = 0;
-            for (int w = 0; w < NW; ++w) t += s_wtot[w][c];
-            P.subtot[c * nsub + sub] = t;
-        }
-        __threadfence();
-        s_last = last_arrival(P.grp_ctr + g, (unsigned long long)gsize);
-    }
-    __syncthreads();
-    if (!s_last) return;
-    if (warp == 0) {
-#pragma unroll
-        for (int c = 0; c < NQ; ++c) {
-            const int64_t *st = P.subtot + c * nsub + s0;
-            const i128 v0 = 2 * lane < gsize ? (i128)__ldcg(st + 2 * lane) : (i128)0;
-            const i128 v1 = 2 * lane + 1 < gsize ? (i128)__ldcg(st + 2 * lane + 1) : (i128)0;
-            const i128 x = warp_incl_scan_i128(v0 + v1);
-            const i128 ex = x - v0 - v1;
-            i128 *ig = ingrp_out + c * nsub + s0;
-            if (2 * lane < gsize) st_i128(ig + 2 * lane, ex);
-            if (2 * lane + 1 < gsize) st_i128(ig + 2 * lane + 1, ex + v0);
-            if (lane == 31) st_i128(P.grptot + c * ngroups + g, x);
-        }
-        __threadfence();
-    }
-    __syncthreads();
-    if (tid == 0) s_last = last_arrival(P.top_ctr, (unsigned long long)ngroups);
-    __syncthreads();
-    if (!s_last) return;
-
-    // Level 2: the last group scans the group totals (and records the totals).
-    i128 total[NQ];
-#pragma unroll
-    for (int c = 0; c < NQ; ++c)
-        total[c] = block_exclusive_scan<8>(P.grptot + c * ngroups, grpofs_out + c * (ngroups + 1), ngroups);
-    if (RECORD && tid == 0 && P.obs) {
-        const double S = fixed_to_double(total[0], P.F);
-        const double C = fixed_to_double(total[NQ - 1], P.F);
-        const unsigned long long n = *P.obs_ctr;
-        P.obs[n % (unsigned long long)P.obs_cap] = sqrt(S * S + C * C) / (double)N;
-        *P.obs_ctr = n + 1;
-    }
-    if (DEC_STEPS && tid == 0 && P.steps_left) *P.steps_left -= 1;
-}
-
-// As ring_prefix_tail, with NPT adjacent nodes per thread (kSubTile / NPT
-// threads per CTA): node i0 + u of the thread holds qv[c][u].
+// end; NPT adjacent nodes per thread, kSubTile / NPT threads per CTA, node i0 + u
+// of the thread holds qv[u]) into lam_out / ingrp_out / grpofs_out.  RECORD: the
+// last CTA records the Kuramoto order parameter from the totals (if P.obs is
+// set); DEC_STEPS: it also decrements the step budget.  Called by every thread
+// of the CTA.
 //
 // One-pass output (flat): the sub-tile totals into fsub_out, their chunks into
 // the group accumulators facc_out, and CTA 0 clears facc_zero (the accumulators the next
@@ -342,7 +349,7 @@ __device__ __forceinline__ void ring_prefix_tail(const RingPlan &P, int64_t *lam
 template <int NQ, int NPT, bool RECORD, bool DEC_STEPS>
 __device__ __forceinline__ void ring_prefix_tail_n(const RingPlan &P, int64_t *lam_out, i128 *ingrp_out,
                                                    i128 *grpofs_out, int64_t sub, int64_t i0,
-                                                   const int64_t (&qv)[NQ][NPT], bool flat, bool tree,
+                                                   const int64_t (&qv)[NPT][NQ], bool flat, bool tree,
                                                    int64_t *fsub_out, unsigned *facc_out, unsigned *facc_zero)
 {
     constexpr int NW = kSubTile / NPT / 32;
@@ -353,44 +360,48 @@ __device__ __forceinline__ void ring_prefix_tail_n(const RingPlan &P, int64_t *l
 
     // Exact inclusive prefix inside the sub-tile: the thread's running sums, a
     // warp scan of the thread totals and the preceding warps' totals.
-    int64_t run[NQ][NPT], ex[NQ];
+    int64_t run[NPT][NQ], ex[NQ];
 #pragma unroll
     for (int c = 0; c < NQ; ++c) {
-        run[c][0] = qv[c][0];
+        run[0][c] = qv[0][c];
 #pragma unroll
-        for (int u = 1; u < NPT; ++u) run[c][u] = run[c][u - 1] + qv[c][u];
-        const int64_t incl = warp_incl_scan(run[c][NPT - 1]);
-        ex[c] = incl - run[c][NPT - 1];
+        for (int u = 1; u < NPT; ++u) run[u][c] = run[u - 1][c] + qv[u][c];
+        const int64_t incl = warp_incl_scan(run[NPT - 1][c]);
+        ex[c] = incl - run[NPT - 1][c];
         if (lane == 31) s_wtot[warp][c] = incl;
     }
     __syncthreads();
 #pragma unroll
-    for (int c = 0; c < NQ; ++c) {
-        int64_t off = ex[c];
-        for (int w = 0; w < warp; ++w) off += s_wtot[w][c];
+    for (int w = 0; w < NW - 1; ++w)
+        if (w < warp) {
 #pragma unroll
-        for (int u = 0; u < NPT; ++u)
-            if (i0 + u < N) lam_out[c * N + i0 + u] = off + run[c][u];
+            for (int c = 0; c < NQ; ++c) ex[c] += s_wtot[w][c];
+        }
+#pragma unroll
+    for (int u = 0; u < NPT; ++u) {
+#pragma unroll
+        for (int c = 0; c < NQ; ++c) run[u][c] += ex[c];
+        if (i0 + u < N) lam_store<NQ>(lam_out + (i0 + u) * NQ, run[u]);
     }
 
     if (flat) {
         const int64_t g = sub >> kGroupLog2;
-        if (tid == 0) {
-#pragma unroll
-            for (int c = 0; c < NQ; ++c) {
-                int64_t t = 0;
-                for (int w = 0; w < NW; ++w) t += s_wtot[w][c];
-                fsub_out[c * nsub + sub] = t;
-                unsigned *a = facc_out + (c * ngroups + g) * 4;
-#pragma unroll
-                for (int k = 0; k < 4; ++k) atomicAdd(a + k, flat_chunk(t, k));
-            }
+        if (tid < NQ * 4) { // one (component, chunk) per lane
+            const int c = tid >> 2, k = tid & 3;
+            int64_t t = 0;
+            for (int w = 0; w < NW; ++w) t += s_wtot[w][c];
+            if (k == 0) fsub_out[c * nsub + sub] = t;
+            atomicAdd(facc_out + (c * ngroups + g) * 4 + k, flat_chunk(t, k));
         }
         if (sub == 0)
             for (int64_t w = tid; w < NQ * ngroups * 4; w += blockDim.x) facc_zero[w] = 0u;
         if (!tree) {
             if ((RECORD && P.obs) || (DEC_STEPS && P.steps_left)) {
                 // the last CTA of the launch: totals from the accumulators
+                if (warp == 0) {
+                    __threadfence(); // the lanes' additions, before thread 0 counts the CTA in
+                    __syncwarp();
+                }
                 if (tid == 0) {
                     __threadfence();
                     s_last = last_arrival(P.flat_ctr, (unsigned long long)nsub);
@@ -472,6 +483,18 @@ __device__ __forceinline__ void ring_prefix_tail_n(const RingPlan &P, int64_t *l
     if (DEC_STEPS && tid == 0 && P.steps_left) *P.steps_left -= 1;
 }
 
+// One node per thread, two-level scan only.
+template <int NQ, bool RECORD, bool DEC_STEPS>
+__device__ __forceinline__ void ring_prefix_tail(const RingPlan &P, int64_t *lam_out, i128 *ingrp_out,
+                                                 i128 *grpofs_out, int64_t sub, int64_t i, const int64_t (&qv)[NQ])
+{
+    int64_t qv1[1][NQ];
+#pragma unroll
+    for (int c = 0; c < NQ; ++c) qv1[0][c] = qv[c];
+    ring_prefix_tail_n<NQ, 1, RECORD, DEC_STEPS>(P, lam_out, ingrp_out, grpofs_out, sub, i, qv1, false, true, nullptr,
+                                                 nullptr, nullptr);
+}
+
 // Buffers one stage reads and writes (chosen by the stage's parity).
 struct RingStageIO {
     const int64_t *lam_in;
@@ -522,8 +545,7 @@ __host__ __device__ __forceinline__ RingStageIO stage_io(const RingPlan &p)
 // gather works in three phases: load() issues the node's own global loads (they
 // need nothing shared), sync() makes the CTA's shared window bases visible (a
 // barrier every thread reaches), finish() combines them into the node's own
-// fixed-point coupled quantity, its window sums W, its link count and coupling
-// scale (see models.cuh).  The node's state loads are issued before the barrier
+// slope (the right-hand side from its window sums, see models.cuh).  The node's state loads are issued before the barrier
 // as well, so the CTA's start latency overlaps the bases' computation.
 template <int M, int STAGE, class Gather, bool FLAT_OK = false>
 __device__ __forceinline__ void stage_body(const RingPlan &P, const RingStageIO &a, const StepSize &h, int64_t sub,
@@ -563,14 +585,8 @@ __device__ __forceinline__ void stage_body(const RingPlan &P, const RingStageIO 
 #pragma unroll
             for (int v = 0; v < D; ++v) xn[v] = P.y[v * N + i];
         } else {
-            int64_t qo[NQ];
-            double fo[NQ];
-            i128 W[NQ];
-            int64_t wsize;
-            double cs;
-            gather.finish(tid, i, pre, qo, fo, W, wsize, cs);
             double k[D];
-            Mo::rhs(P.mp, P.F, fo, qo, W, X, Iext, k, wsize, cs);
+            gather.finish(tid, i, pre, X, Iext, k);
 #pragma unroll
             for (int v = 0; v < D; ++v) {
                 if (STAGE == 1) {
@@ -600,9 +616,9 @@ __device__ __forceinline__ void stage_body(const RingPlan &P, const RingStageIO 
     constexpr bool RECORD = (M == 0 || M == 3) && (STAGE == 0 || STAGE == 4);
     if constexpr (FLAT_OK) {
         if (P.flat) { // the one-pass prefix (both forms in the prologue)
-            int64_t qv1[NQ][1];
+            int64_t qv1[1][NQ];
 #pragma unroll
-            for (int c = 0; c < NQ; ++c) qv1[c][0] = qv[c];
+            for (int c = 0; c < NQ; ++c) qv1[0][c] = qv[c];
             ring_prefix_tail_n<NQ, 1, RECORD, STAGE == 4>(P, a.lam_out, a.ingrp_out, a.grpofs_out, sub, i, qv1, true,
                                                           STAGE == 0, a.fsub_out, a.facc_out, a.facc_zero);
             return;

@@ -413,13 +413,37 @@ void simk::model_constants(int model, const double *params, double K, ModelParam
     }
 }
 
-// A Kuramoto ring's shift of its exact window sums into int64 and the scale of
-// the cross product T on the grid 2^-(F - ksh - 3) (see ring_coupling).
-void simk::ring_coupling_constants(ModelParams &mp, int model, int F)
+// A ring's shift of its exact window sums into int64 (|S| < 2^62) and the power
+// of two its coupling constants carry for it: the Kuramoto models' cross product
+// T lies on the grid 2^-(F - ksh - 3) (see ring_coupling); FHN and HH have
+// |f| < 2^(54 - F), so |sum| <= wsize 2^54, and convert sums on 2^-(F - ksh).
+void simk::ring_coupling_constants(ModelParams &mp, int model, const double *params, int F)
 {
     const int lg = ceil_log2((uint64_t)mp.wsize);
-    mp.ksh = lg + F - 61 > 0 ? lg + F - 61 : 0;
-    mp.c[5] = std::ldexp(model == SIM_KS ? mp.c[1] : mp.c[0], mp.ksh + 3 - F);
+    if (model == SIM_KS || model == SIM_KSI) {
+        mp.ksh = lg + F - 61 > 0 ? lg + F - 61 : 0;
+        mp.c[5] = std::ldexp(model == SIM_KS ? mp.c[1] : mp.c[0], mp.ksh + 3 - F);
+        return;
+    }
+    mp.ksh = lg > 7 ? lg - 7 : 0;
+    mp.wsm = (uint64_t)mp.wsize << (56 - mp.ksh);
+    if (model != SIM_FHN) {
+        mp.c[7] = std::ldexp(mp.c[7], mp.ksh - F);
+        return;
+    }
+    // FHN: the integer bracket of Model<1>::rhs_ring needs its constants below
+    // 2^62, |a| < 64 (then both brackets stay below 2^9) and ksh = lg - 7 >= 0
+    mp.c[6] = std::ldexp(mp.c[0], -54);
+    mp.c[7] = std::ldexp(std::fma(-mp.c[0], params[0], 1.0) / params[0], -54); // the rest of 1/eps
+    mp.fx = lg >= 7 && std::fabs(mp.c[1]) < 64.0 && std::fabs(params[0]) > 1e-200 && std::fabs(params[0]) < 1e200;
+    mp.a54 = mp.fx ? (int64_t)std::llround(std::ldexp(mp.c[1], 54)) : 0;
+    const double sK[4] = {mp.c[2] / mp.c[0], mp.c[3] / mp.c[0], mp.c[4], mp.c[5]};
+    for (int i = 0; i < 4; ++i) {
+        const double v = std::ldexp(sK[i], mp.ksh + 67);
+        if (!(std::fabs(v) < 0x1p62)) mp.fx = 0;
+        else mp.kq[i] = (int64_t)std::llround(v);
+        mp.c[2 + i] = std::ldexp(mp.c[2 + i], mp.ksh - F);
+    }
 }
 
 // A lattice's rotation by -alpha (the ball's and disk's x pass rotate every
@@ -536,7 +560,7 @@ static int create_impl(sim_t *out, int model, int topology, int64_t N, int64_t r
         p.F = ring_F(model);
         p.lim = 54 - p.F;
         p.mp = mp;
-        if (model == SIM_KS || model == SIM_KSI) ring_coupling_constants(p.mp, model, p.F);
+        ring_coupling_constants(p.mp, model, params, p.F);
         p.y = reinterpret_cast<double *>(b + L.y);
         p.acc = reinterpret_cast<double *>(b + L.acc);
         p.xg[0] = reinterpret_cast<double *>(b + L.xg0);

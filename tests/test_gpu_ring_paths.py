@@ -1,0 +1,48 @@
+"""Edges of the ring kernels' dispatch rules: the cluster-resident kernel's slice
+sizes, and the FitzHugh-Nagumo slope in integer or FP64 arithmetic."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2410_19075_gb300 import inputs as I
+from _common import PARAMS, inputs_for
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("model", [0, 1, 2, 3])
+@pytest.mark.parametrize("N,R", [(129, 64), (257, 1), (1025, 256), (1921, 960), (4095, 2000), (4096, 2047)])
+def test_cluster_slices_equal_streaming_bitwise(model, N, R):
+    """Slice sizes with a ragged last slice and windows up to the whole ring; the
+    slope read after the run comes from the prefix form the cluster kernel leaves."""
+    from paper_2410_19075_gb300 import Network
+    y0, npar = inputs_for(model, 0, N, 11 + N)
+    outs = []
+    for streaming in (False, True):
+        with Network(model, 0, N, R, PARAMS[model](), streaming=streaming) as net:
+            if npar is not None:
+                net.set_node_param(npar)
+            net.set_state(y0)
+            net.step(19, 0.01)
+            outs.append((net.get_state(), net.observables(), net.rhs()))
+    for a, b in zip(*outs):
+        assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("R", [1, 31, 32, 63, 64, 1000])  # the integer form needs windows of 65 nodes
+@pytest.mark.parametrize("sigma,a", [(0.1, 0.5), (3.5, 0.5), (4.5, 0.5), (100.0, -2.0), (0.1, 63.9), (0.1, 64.0)])
+def test_fhn_slope_both_forms_match_oracle(R, sigma, a):
+    """sigma and a on both sides of the integer form's range (coupling constants
+    below 2^62, |a| < 64).  Both forms and the oracle round each term of the slope's
+    bracket to a few 2^-53 of its size; 1e-12 of the largest slope covers the
+    oracle's sum of up to 2000 terms."""
+    from paper_2410_19075_gb300 import Network
+    N = 5000
+    params = I.fhn_params(sigma=sigma, a=a)
+    y0, _ = inputs_for(1, 0, N, 5 + R)
+    q = np.arange(0, N, 7)
+    with Network(1, 0, N, R, params) as net:
+        net.set_state(y0)
+        k = net.rhs().reshape(2, N)[:, q]
+    ref = oracle.rhs_sampled(1, 0, N, R, params, y0, q)
+    assert np.abs(k - ref).max() < 1e-12 * max(1.0, np.abs(ref).max())
