@@ -3,15 +3,20 @@
 // For N <= kClusterMaxNodes the stage kernels of the streaming path are
 // launch-latency bound (a few CTAs per stage, four launches per RK4 step).  Here
 // one cluster of up to 16 CTAs (16 SMs) runs all stages of all steps of a call:
-//   * every CTA owns a contiguous slice of nodes; their y, acc and HH gates stay
-//     in registers for the whole call;
-//   * after each stage every CTA writes the fixed-point coupled quantities of
-//     its nodes into the shared memory of every CTA of the cluster (distributed
-//     shared memory), into the buffer of the next stage (double-buffered), and
-//     one cluster barrier per stage publishes them;
-//   * every CTA then builds the exact prefix of the whole ring in its own shared
-//     memory (int64 inside 256-node blocks, int128 block offsets) and gathers its
-//     nodes' window sums from it.
+//   * every CTA owns a contiguous slice of nodes, one per thread; their y, acc and
+//     HH gates stay in registers for the whole call;
+//   * after each stage every CTA builds the exact prefix lam of its slice in its own
+//     shared memory (warp scans; double-buffered) and sends its slice total to
+//     every CTA of the cluster (distributed shared memory); one cluster barrier
+//     per stage publishes both;
+//   * a node's window sum is then two 16-byte reads of lam, each in the shared memory
+//     of the CTA that owns that end of the window (its address is fixed for the
+//     call), plus the difference of the two slices' offsets, which every warp
+//     scans from the totals itself while those reads are in flight;
+//   * the order parameter of every step is recorded by one more warp of CTA 0,
+//     beside the stage that follows.
+// What bounds a stage is one dependent chain: barrier, remote reads, right-hand
+// side, sin/cos, scan.
 // The arithmetic (grid, exact sums, right-hand sides, RK4) is the streaming
 // path's, so the results are bit-for-bit the same.  At the end the cluster
 // writes y, the order parameters of every step, and the streaming path's
@@ -19,225 +24,251 @@
 #include <cooperative_groups.h>
 
 #include "internal.h"
+#include "ring_parts.cuh"
 
 namespace cg = cooperative_groups;
 
 namespace simk {
 
-constexpr int kClusterThreads = 256;
-constexpr int kClusterMaxNodesPerThread = 2;
+constexpr int kClusterMaxCtas = 16;
+constexpr int kClusterSlice = 512; // nodes of a CTA at most (two warps' worth of int64 headroom: 512 2^54 = 2^63)
+constexpr int kClusterThreadsMax = kClusterSlice + 32;
 
-// Byte offset of the int128 block offsets: after two Q buffers and the in-block
-// prefix (int64 each), rounded up to 16 bytes (int128 accesses need it).
+// Threads of a CTA that owns `per` nodes: one per node and the recording warp.
+static __host__ __device__ constexpr int cluster_threads(int per) { return (per + 31) / 32 * 32 + 32; }
+
 template <int NQ>
-__host__ __device__ constexpr size_t cluster_bofs_offset(int64_t N)
+__host__ __device__ constexpr size_t cluster_smem_bytes(int per)
 {
-    return ((size_t)(3 * NQ) * (size_t)N * sizeof(int64_t) + 15) / 16 * 16;
+    return sizeof(int64_t) * NQ * (size_t)(2 * per); // lam, two buffers
 }
 
+// Exact offsets of the cluster's slices from their totals, by one warp: lane r
+// holds the prefix in front of slice r as hi 2^sh + lo (ex_*), every lane the
+// ring's total (tot_*).
+template <int NQ> struct SliceOffsets {
+    int64_t ex_hi[NQ], tot_hi[NQ];
+    int ex_lo[NQ], tot_lo[NQ];
+};
 template <int NQ>
-__host__ __device__ constexpr size_t cluster_smem_bytes(int64_t N)
+__device__ __forceinline__ void slice_offsets(const int64_t (*tot)[NQ], int CL, int sh, SliceOffsets<NQ> &o)
 {
-    return cluster_bofs_offset<NQ>(N) + (size_t)NQ * ((N + 255) / 256 + 1) * sizeof(i128);
+    const int lane = threadIdx.x & 31, mask = (1 << sh) - 1;
+    int64_t t[NQ];
+#pragma unroll
+    for (int c = 0; c < NQ; ++c) t[c] = lane < CL ? tot[lane][c] : 0;
+#pragma unroll
+    for (int c = 0; c < NQ; ++c) {
+        const int64_t h = t[c] >> sh;
+        const int l = (int)t[c] & mask;
+        int64_t hi = h;
+        int lo = l;
+#pragma unroll
+        for (int d = 1; d < kClusterMaxCtas; d <<= 1) {
+            const int64_t h2 = __shfl_up_sync(0xffffffffu, hi, d);
+            const int l2 = __shfl_up_sync(0xffffffffu, lo, d);
+            if (lane >= d) {
+                hi += h2;
+                lo += l2;
+            }
+        }
+        o.ex_hi[c] = hi - h;
+        o.ex_lo[c] = lo - l;
+        o.tot_hi[c] = __shfl_sync(0xffffffffu, hi, kClusterMaxCtas - 1);
+        o.tot_lo[c] = __shfl_sync(0xffffffffu, lo, kClusterMaxCtas - 1);
+    }
+}
+
+// The prefix in front of slice r on copy q of the ring (-1, 0, 1).
+template <int NQ>
+__device__ __forceinline__ void slice_base(const SliceOffsets<NQ> &o, int r, int q, int64_t (&hi)[NQ], int (&lo)[NQ])
+{
+#pragma unroll
+    for (int c = 0; c < NQ; ++c) {
+        hi[c] = __shfl_sync(0xffffffffu, o.ex_hi[c], r) + q * o.tot_hi[c];
+        lo[c] = __shfl_sync(0xffffffffu, o.ex_lo[c], r) + q * o.tot_lo[c];
+    }
 }
 
 template <int M>
-__global__ void __launch_bounds__(kClusterThreads, 1)
-    ring_cluster_kernel(const RingPlan P, double dt, int64_t n_steps)
+__global__ void __launch_bounds__(kClusterThreadsMax, 1)
+    ring_cluster_kernel(const RingPlan P, const StepSize h, int per, int64_t n_steps)
 {
     using Mo = Model<M>;
-    constexpr int D = Mo::D, NQ = Mo::NQ, NX = Mo::NX, XOFF = D - NX, MPT = kClusterMaxNodesPerThread;
+    constexpr int D = Mo::D, NQ = Mo::NQ, NX = Mo::NX, XOFF = D - NX;
+    constexpr bool KURAMOTO = M == 0 || M == 3;
     cg::cluster_group cluster = cg::this_cluster();
     const int rank = (int)cluster.block_rank(), CL = (int)cluster.num_blocks();
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int64_t N = P.N, R = P.R, nb = (N + 255) / 256;
-    const int64_t per = (N + CL - 1) / CL, i0 = rank * per, i1 = i0 + per < N ? i0 + per : N;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = (int)(blockDim.x >> 5) - 1; // node warps
+    const int N = (int)P.N, R = (int)P.R, sh = P.mp.ksh, mask = (1 << sh) - 1;
+    const int i = rank * per + tid;
+    const bool recorder = warp == nwarps, live = !recorder && tid < per && i < N;
 
-    extern __shared__ __align__(16) unsigned char smem[];
-    int64_t *qbuf0 = reinterpret_cast<int64_t *>(smem);
-    int64_t *qbuf1 = qbuf0 + NQ * N;
-    int64_t *lam = qbuf1 + NQ * N;
-    i128 *bofs = reinterpret_cast<i128 *>(smem + cluster_bofs_offset<NQ>(N)); // NQ * (nb + 1)
+    extern __shared__ __align__(16) int64_t lam[]; // [2][per][NQ]
+    __shared__ __align__(16) int64_t s_tot[2][kClusterMaxCtas][NQ];
+    __shared__ int64_t s_wtot[kClusterThreadsMax / 32][NQ];
 
-    // own nodes: i = i0 + tid + k * blockDim
-    double y[MPT][D], acc[MPT][D], xs[MPT][NX > 0 ? NX : 1], iext[MPT];
-    int64_t qn[MPT][NQ];
-    bool ok = true;
+    // the node's window ends: slice, copy of the ring and address of lam (buffer 0)
+    int rk[2] = {0, 0}, qk[2] = {0, 0};
+    const int64_t *end[2] = {lam, lam};
 #pragma unroll
-    for (int k = 0; k < MPT; ++k) {
-        const int64_t i = i0 + tid + (int64_t)k * kClusterThreads;
-        iext[k] = 0.0;
-#pragma unroll
-        for (int v = 0; v < D; ++v) {
-            y[k][v] = i < i1 ? P.y[v * N + i] : 0.0;
-            acc[k][v] = 0.0;
+    for (int side = 0; side < 2; ++side) {
+        int e = side == 0 ? i + R : i - R - 1;
+        if (live) {
+            qk[side] = e < 0 ? -1 : (e >= N ? 1 : 0);
+            e -= qk[side] * N;
+            rk[side] = e / per;
+            end[side] = cluster.map_shared_rank(lam, rk[side]) + (e - rk[side] * per) * NQ;
         }
-#pragma unroll
-        for (int g = 0; g < NX; ++g) xs[k][g] = y[k][XOFF + g];
-        if (M == 2 && P.node_param && i < i1) iext[k] = P.node_param[i];
     }
 
-    // Q of f(x) for own nodes, written into `dst` of every CTA of the cluster
-    auto broadcast = [&](int64_t *dst) {
+    double y[D] = {}, acc[D] = {}, xs[NX > 0 ? NX : 1] = {}, iext = 0.0;
+    int64_t qn[NQ] = {};
+    bool ok = true;
+    if (live) {
 #pragma unroll
-        for (int k = 0; k < MPT; ++k) {
-            const int64_t i = i0 + tid + (int64_t)k * kClusterThreads;
-            if (i >= i1) continue;
-            for (int r = 0; r < CL; ++r) {
-                int64_t *remote = cluster.map_shared_rank(dst, r);
+        for (int v = 0; v < D; ++v) y[v] = P.y[(int64_t)v * N + i];
 #pragma unroll
-                for (int c = 0; c < NQ; ++c) remote[c * N + i] = qn[k][c];
-            }
-        }
-    };
+        for (int g = 0; g < NX; ++g) xs[g] = y[XOFF + g];
+        if (M == 2 && P.node_param) iext = P.node_param[i];
+        Mo::coupled_q(P.mp, y, P.F, P.lim, ok, qn);
+    }
 
-    // Exact prefix of a Q buffer: lam (inclusive inside 256-node blocks) and
-    // bofs (exclusive at block starts, bofs[nb] = total).  Each warp scans whole
-    // blocks (8 values per lane); warp 0 then scans the block totals.
-    auto build_prefix = [&](const int64_t *q) {
-        for (int64_t blk = warp; blk < (int64_t)NQ * nb; blk += kClusterThreads / 32) {
-            const int c = (int)(blk / nb);
-            const int64_t b = blk - (int64_t)c * nb;
-            const int64_t j0 = b * 256 + lane * 8;
-            int64_t v[8], run = 0;
+    // lam of the slice into buffer b and its total to every CTA, then the cluster barrier
+    auto publish = [&](int b) {
+        int64_t run[NQ];
 #pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                v[e] = j0 + e < N ? q[c * N + j0 + e] : 0;
-                run += v[e];
-                v[e] = run;
-            }
-            const int64_t incl = warp_incl_scan(run);
-            const int64_t off = incl - run;
-#pragma unroll
-            for (int e = 0; e < 8; ++e)
-                if (j0 + e < N) lam[c * N + j0 + e] = off + v[e];
-            if (lane == 31) bofs[c * (nb + 1) + b] = (i128)incl; // block total, scanned below
-        }
-        __syncthreads();
-        if (warp == 0) {
+        for (int c = 0; c < NQ; ++c) run[c] = qn[c];
+        if (!recorder) {
 #pragma unroll
             for (int c = 0; c < NQ; ++c) {
-                // nb <= 32 blocks (N <= 8192): one per lane
-                const i128 t = lane < nb ? bofs[c * (nb + 1) + lane] : (i128)0;
-                i128 x = t;
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const i128 u = shfl_up_i128(x, o);
-                    if (lane >= o) x += u;
-                }
-                __syncwarp();
-                if (lane < nb) bofs[c * (nb + 1) + lane] = x - t;
-                if (lane == 31) bofs[c * (nb + 1) + nb] = x;
+                run[c] = warp_incl_scan(run[c]);
+                if (lane == 31) s_wtot[warp][c] = run[c];
             }
         }
         __syncthreads();
-    };
-    auto prefix_at = [&](int c, int64_t p) -> i128 { // p in [-N, 2N)
-        i128 add = 0;
-        const i128 tot = bofs[c * (nb + 1) + nb];
-        if (p < 0) {
-            p += N;
-            add = -tot;
-        } else if (p >= N) {
-            p -= N;
-            add = tot;
+        if (live) {
+            for (int w = 0; w < warp; ++w)
+#pragma unroll
+                for (int c = 0; c < NQ; ++c) run[c] += s_wtot[w][c];
+            int64_t *o = lam + (b * per + tid) * NQ;
+#pragma unroll
+            for (int c = 0; c < NQ; ++c) o[c] = run[c];
         }
-        i128 v = bofs[c * (nb + 1) + (p >> 8)] + add;
-        if (p & 255) v += (i128)lam[c * N + p - 1];
-        return v;
+        if (recorder && lane < CL) {
+            int64_t *o = cluster.map_shared_rank(&s_tot[b][rank][0], lane);
+#pragma unroll
+            for (int c = 0; c < NQ; ++c) {
+                int64_t t = 0;
+                for (int w = 0; w < nwarps; ++w) t += s_wtot[w][c];
+                o[c] = t;
+            }
+        }
+        cluster.sync();
     };
-    auto record_order = [&]() {
-        if ((M == 0 || M == 3) && rank == 0 && tid == 0) {
-            const double S = fixed_to_double(bofs[nb], P.F);
-            const double C = fixed_to_double(bofs[(NQ - 1) * (nb + 1) + nb], P.F);
+    auto load_end = [&](int side, int b, int64_t (&v)[NQ]) {
+        const int64_t *p = end[side] + (b ? per * NQ : 0);
+        if constexpr (NQ == 2) {
+            const longlong2 w = *reinterpret_cast<const longlong2 *>(p);
+            v[0] = w.x;
+            v[1] = w.y;
+        } else v[0] = *p;
+    };
+    auto record_order = [&](const SliceOffsets<NQ> &o) { // the recording warp of CTA 0
+        if (KURAMOTO && rank == 0 && lane == 0) {
+            const double S = fixed_to_double(((i128)o.tot_hi[0] << sh) + o.tot_lo[0], P.F);
+            const double C = fixed_to_double(((i128)o.tot_hi[NQ - 1] << sh) + o.tot_lo[NQ - 1], P.F);
             const unsigned long long n = *P.obs_ctr;
             P.obs[n % (unsigned long long)P.obs_cap] = sqrt(S * S + C * C) / (double)N;
             *P.obs_ctr = n + 1;
         }
     };
 
-    // prologue: f(y) into buffer 0 (the observable of y was recorded when the
-    // state was set)
-#pragma unroll
-    for (int k = 0; k < MPT; ++k) {
-        Mo::coupled_q(P.mp, y[k], P.F, P.lim, ok, qn[k]);
-    }
-    broadcast(qbuf0);
-    cluster.sync();
-
+    // f(y) into buffer 0 (the observable of y was recorded when the state was set)
+    publish(0);
     int cur = 0; // buffer holding f of the current stage input
     for (int64_t step = 0; step < n_steps; ++step) {
 #pragma unroll 1
         for (int stage = 1; stage <= 4; ++stage) {
-            const int64_t *q = cur ? qbuf1 : qbuf0;
-            build_prefix(q);
-            if (stage == 1 && step > 0) record_order(); // order parameter of y after the previous step
+            if (!recorder) {
+                int64_t lb[NQ], la[NQ], hb[NQ], ha[NQ], S[NQ];
+                int lob[NQ], loa[NQ];
+                load_end(0, cur, lb);
+                load_end(1, cur, la);
+                SliceOffsets<NQ> o;
+                slice_offsets<NQ>(s_tot[cur], CL, sh, o);
+                slice_base<NQ>(o, rk[0], qk[0], hb, lob);
+                slice_base<NQ>(o, rk[1], qk[1], ha, loa);
+                if (live) {
 #pragma unroll
-            for (int k = 0; k < MPT; ++k) {
-                const int64_t i = i0 + tid + (int64_t)k * kClusterThreads;
-                if (i >= i1) continue;
-                int64_t qo[NQ], S[NQ];
-#pragma unroll
-                for (int c = 0; c < NQ; ++c) {
-                    qo[c] = q[c * N + i];
-                    const i128 W = prefix_at(c, i + R + 1) - prefix_at(c, i - R);
-                    S[c] = (int64_t)((Mo::OWN_OUT && !P.mp.include_self ? W - (i128)qo[c] : W) >> P.mp.ksh);
-                }
-                double kk[D], xn[D];
-                Mo::rhs_ring(P.mp, qo, S, xs[k], iext[k], kk);
-#pragma unroll
-                for (int v = 0; v < D; ++v) {
-                    if (stage == 1) {
-                        acc[k][v] = kk[v];
-                        xn[v] = y[k][v] + (0.5 * dt) * kk[v];
-                    } else if (stage == 2) {
-                        acc[k][v] = acc[k][v] + 2.0 * kk[v];
-                        xn[v] = y[k][v] + (0.5 * dt) * kk[v];
-                    } else if (stage == 3) {
-                        acc[k][v] = acc[k][v] + 2.0 * kk[v];
-                        xn[v] = y[k][v] + dt * kk[v];
-                    } else {
-                        y[k][v] = y[k][v] + (dt / 6.0) * (acc[k][v] + kk[v]);
-                        xn[v] = y[k][v];
+                    for (int c = 0; c < NQ; ++c) {
+                        const int64_t own = Mo::OWN_OUT && !P.mp.include_self ? qn[c] : 0;
+                        const int lo = lob[c] - loa[c] + ((int)lb[c] & mask) - ((int)la[c] & mask) - ((int)own & mask);
+                        S[c] = hb[c] - ha[c] + (lb[c] >> sh) - (la[c] >> sh) - (own >> sh) + (int64_t)(lo >> sh);
                     }
-                }
+                    double k[D], xn[D];
+                    Mo::rhs_ring(P.mp, qn, S, xs, iext, k);
 #pragma unroll
-                for (int g = 0; g < NX; ++g) xs[k][g] = xn[XOFF + g];
-                Mo::coupled_q(P.mp, xn, P.F, P.lim, ok, qn[k]);
+                    for (int v = 0; v < D; ++v) {
+                        if (stage == 1) {
+                            acc[v] = k[v];
+                            xn[v] = y[v] + h.half * k[v];
+                        } else if (stage == 4) {
+                            y[v] = y[v] + h.sixth * (acc[v] + k[v]);
+                            xn[v] = y[v];
+                        } else {
+                            acc[v] = acc[v] + 2.0 * k[v];
+                            xn[v] = y[v] + (stage == 2 ? h.half : h.dt) * k[v];
+                        }
+                    }
+#pragma unroll
+                    for (int g = 0; g < NX; ++g) xs[g] = xn[XOFF + g];
+                    Mo::coupled_q(P.mp, xn, P.F, P.lim, ok, qn);
+                }
+            } else if (KURAMOTO && stage == 1 && step > 0) { // R of y after the previous step
+                SliceOffsets<NQ> o;
+                slice_offsets<NQ>(s_tot[cur], CL, sh, o);
+                record_order(o);
             }
             cur ^= 1;
-            broadcast(cur ? qbuf1 : qbuf0);
-            cluster.sync();
+            publish(cur);
         }
     }
     if (!ok) raise_error(P.err, ERR_RANGE);
 
-    // results: y, the last order parameter, and the streaming path's prefix
-    // buffers of f(y) (buffer 0)
-    build_prefix(cur ? qbuf1 : qbuf0);
-    if (n_steps > 0) record_order();
+    // results: y, the last order parameter, and the streaming path's two-level
+    // prefix of f(y) (buffer 0): lam256(i) = P(i + 1) - P(start of i's 256-node
+    // sub-tile), the start's prefix read like a window end at e = start - 1
+    SliceOffsets<NQ> o;
+    slice_offsets<NQ>(s_tot[cur], CL, sh, o);
+    if (recorder && n_steps > 0) record_order(o);
+    if (!recorder) {
+        const int e = (i & ~(kSubTile - 1)) - 1, re = live && e >= 0 ? e / per : 0; // e < 0: prefix 0
+        int64_t hs[NQ], hi[NQ];
+        int los[NQ], lo[NQ];
+        slice_base<NQ>(o, re, 0, hs, los);
+        slice_base<NQ>(o, rank, 0, hi, lo);
+        if (live) {
+            const int64_t *ps = cluster.map_shared_rank(lam, re) + (cur * per + (e >= 0 ? e - re * per : 0)) * NQ;
+            const int64_t *pi = lam + (cur * per + tid) * NQ;
+            const int sub = i >> kSubLog2;
 #pragma unroll
-    for (int k = 0; k < MPT; ++k) {
-        const int64_t i = i0 + tid + (int64_t)k * kClusterThreads;
-        if (i >= i1) continue;
+            for (int v = 0; v < D; ++v) P.y[(int64_t)v * N + i] = y[v];
 #pragma unroll
-        for (int v = 0; v < D; ++v) P.y[v * N + i] = y[k][v];
-#pragma unroll
-        for (int c = 0; c < NQ; ++c) P.lam[0][i * NQ + c] = lam[c * N + i];
-    }
-    if (rank == 0) {
-        // one prefix group (nsub <= 64): in-group offsets are the block offsets
-        for (int64_t t = tid; t < (int64_t)NQ * nb; t += kClusterThreads) {
-            const int c = (int)(t / nb);
-            const int64_t b = t - (int64_t)c * nb;
-            P.ingrp[0][c * P.nsub + b] = bofs[c * (nb + 1) + b];
+            for (int c = 0; c < NQ; ++c) {
+                const i128 start = e >= 0 ? ((i128)hs[c] << sh) + los[c] + ps[c] : (i128)0;
+                const i128 here = ((i128)hi[c] << sh) + lo[c] + pi[c];
+                P.lam[0][(int64_t)i * NQ + c] = (int64_t)(here - start);
+                // one prefix group (at most 16 sub-tiles): in-group offsets are the sub-tile starts
+                if (!(i & (kSubTile - 1))) st_i128(P.ingrp[0] + c * P.nsub + sub, start);
+                if (i == 0) {
+                    st_i128(P.grpofs[0] + c * (P.ngroups + 1), 0);
+                    st_i128(P.grpofs[0] + c * (P.ngroups + 1) + 1, ((i128)o.tot_hi[c] << sh) + o.tot_lo[c]);
+                }
+            }
         }
-        if (tid < NQ) {
-            P.grpofs[0][tid * (P.ngroups + 1)] = 0;
-            P.grpofs[0][tid * (P.ngroups + 1) + 1] = bofs[tid * (nb + 1) + nb];
-        }
     }
-    cluster.sync(); // no CTA exits while others may still write its shared memory
+    cluster.sync(); // no CTA exits while others may still read its shared memory
 }
 
 static int g_max_cluster = 8; // 16 when the device can co-schedule it (set by configure)
@@ -248,40 +279,45 @@ int cluster_size_for(int64_t N)
     int cl = (int)((N + 127) / 128);
     if (cl < 2) cl = 2;
     if (cl > g_max_cluster) cl = g_max_cluster;
-    return (N + cl - 1) / cl <= (int64_t)kClusterThreads * kClusterMaxNodesPerThread ? cl : 0;
+    return (N + cl - 1) / cl <= (int64_t)kClusterSlice ? cl : 0;
 }
 
 template <int M>
-static cudaError_t configure_one(int64_t max_nodes)
+static cudaError_t configure_one()
 {
-    constexpr int NQ = Model<M>::NQ;
-    cudaError_t e = cudaFuncSetAttribute(ring_cluster_kernel<M>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)cluster_smem_bytes<NQ>(max_nodes));
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(ring_cluster_kernel<M>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    return e;
+    return cudaFuncSetAttribute(ring_cluster_kernel<M>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+}
+
+static cudaLaunchConfig_t cluster_config(int cl, int per, size_t smem, cudaStream_t s, cudaLaunchAttribute *attr)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)cl);
+    cfg.blockDim = dim3((unsigned)cluster_threads(per));
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    attr->id = cudaLaunchAttributeClusterDimension;
+    attr->val.clusterDim.x = (unsigned)cl;
+    attr->val.clusterDim.y = 1;
+    attr->val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cfg;
 }
 
 cudaError_t ring_cluster_configure()
 {
-    cudaError_t e = configure_one<0>(kClusterMaxNodes);
-    if (e == cudaSuccess) e = configure_one<1>(kClusterMaxNodes);
-    if (e == cudaSuccess) e = configure_one<2>(kClusterMaxNodes);
-    if (e == cudaSuccess) e = configure_one<3>(kClusterMaxNodes);
+    cudaError_t e = configure_one<0>();
+    if (e == cudaSuccess) e = configure_one<1>();
+    if (e == cudaSuccess) e = configure_one<2>();
+    if (e == cudaSuccess) e = configure_one<3>();
     if (e != cudaSuccess) return e;
-    // largest cluster the device can co-schedule with the largest shared-memory use
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(16);
-    cfg.blockDim = dim3(kClusterThreads);
-    cfg.dynamicSmemBytes = cluster_smem_bytes<2>(kClusterMaxNodes);
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 16;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    // largest cluster the device can co-schedule
+    cudaLaunchAttribute attr;
+    cudaLaunchConfig_t cfg = cluster_config(kClusterMaxCtas, (int)kClusterMaxNodes / kClusterMaxCtas,
+                                            cluster_smem_bytes<2>((int)kClusterMaxNodes / kClusterMaxCtas), nullptr, &attr);
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, ring_cluster_kernel<0>, &cfg) == cudaSuccess && n >= 1) g_max_cluster = 16;
+    if (cudaOccupancyMaxActiveClusters(&n, ring_cluster_kernel<0>, &cfg) == cudaSuccess && n >= 1)
+        g_max_cluster = kClusterMaxCtas;
     else g_max_cluster = 8;
     cudaGetLastError();
     return cudaSuccess;
@@ -290,20 +326,10 @@ cudaError_t ring_cluster_configure()
 template <int M>
 static cudaError_t launch_cluster(const RingPlan &p, double dt, int64_t n_steps, int cl, cudaStream_t s)
 {
-    constexpr int NQ = Model<M>::NQ;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)cl);
-    cfg.blockDim = dim3(kClusterThreads);
-    cfg.dynamicSmemBytes = cluster_smem_bytes<NQ>(p.N);
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)cl;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, ring_cluster_kernel<M>, p, dt, n_steps);
+    const int per = (int)((p.N + cl - 1) / cl);
+    cudaLaunchAttribute attr;
+    const cudaLaunchConfig_t cfg = cluster_config(cl, per, cluster_smem_bytes<Model<M>::NQ>(per), s, &attr);
+    return cudaLaunchKernelEx(&cfg, ring_cluster_kernel<M>, p, step_size(dt), per, n_steps);
 }
 
 cudaError_t ring_cluster_steps(const RingPlan &p, double dt, int64_t n_steps, cudaStream_t s)

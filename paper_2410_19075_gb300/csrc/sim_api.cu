@@ -50,6 +50,7 @@ namespace {
 
 constexpr int64_t kObsCap = 65536;
 constexpr int kGraphChunk = 16; // RK4 steps per captured graph
+constexpr int64_t kClusterSteps = 4096; // RK4 steps per launch of the cluster-resident kernel
 
 size_t align_up(size_t x, size_t a = 256) { return (x + a - 1) / a * a; }
 
@@ -890,6 +891,13 @@ int sim_step(sim_t h, int64_t n_steps, double dt)
         }
     }
     int64_t left = n_steps;
+    while (left > 0 && use_cluster(h)) { // one launch runs all the steps
+        const int64_t n = left < kClusterSteps ? left : kClusterSteps;
+        const cudaError_t e = ring_cluster_steps(h->ring, dt, n, h->stream);
+        if (e != cudaSuccess) return cuda_fail(e, "cluster launch");
+        left -= n;
+        h->steps_done += n;
+    }
     while (left > 0) {
         const int chunk = left >= kGraphChunk ? kGraphChunk : 1;
         cudaGraphExec_t ex;
