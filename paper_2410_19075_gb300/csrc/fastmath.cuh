@@ -41,22 +41,25 @@ namespace simk {
 // Tables (host-filled at handle creation; see sim_api.cu).
 constexpr int kSinTab = 1024;  // sin/cos(j pi/512), j in [0, 1024)
 constexpr int kExpTab = 64;    // 2^(j/64), j in [0, 64)
+constexpr int kExp2Tab = 256;  // 2^(j/256), j in [0, 256)
 
 struct MathTables {
     const double2 *sincos;     // (sin, cos) of j*pi/512
     const double *exp2j;       // 2^(j/64)
     const longlong2 *sincos_q; // (sin, cos) of j*pi/512 rounded onto the grid 2^-62
+    const unsigned long long *exp2q; // 2^(j/256) rounded onto the grid 2^-63
 };
 
 // The tables as one block of 64-bit words (host-filled in long double, uploaded
 // once per network or device): sincos (2 kSinTab doubles), exp2j (kExpTab
-// doubles), sincos_q (2 kSinTab int64).
-constexpr int kMathTableWords = 2 * kSinTab + kExpTab + 2 * kSinTab;
+// doubles), sincos_q (2 kSinTab int64), exp2q (kExp2Tab uint64).
+constexpr int kMathTableWords = 2 * kSinTab + kExpTab + 2 * kSinTab + kExp2Tab;
 __host__ __device__ inline MathTables math_tables_at(const void *block)
 {
     const double *d = static_cast<const double *>(block);
     return MathTables{reinterpret_cast<const double2 *>(d), d + 2 * kSinTab,
-                      reinterpret_cast<const longlong2 *>(d + 2 * kSinTab + kExpTab)};
+                      reinterpret_cast<const longlong2 *>(d + 2 * kSinTab + kExpTab),
+                      reinterpret_cast<const unsigned long long *>(d + 4 * kSinTab + kExpTab)};
 }
 
 // |x| as a float by truncating the mantissa (integer instructions; |x| must be

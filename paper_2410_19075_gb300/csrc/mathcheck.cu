@@ -22,6 +22,8 @@ void fill_math_tables(double *block)
         sincos_q[2 * j + 1] = (int64_t)llroundl(cosl(a) * 4611686018427387904.0L);
     }
     for (int j = 0; j < kExpTab; ++j) exp2j[j] = (double)exp2l((long double)j / 64.0L);
+    uint64_t *exp2q = reinterpret_cast<uint64_t *>(block + 4 * kSinTab + kExpTab);
+    for (int j = 0; j < kExp2Tab; ++j) exp2q[j] = (uint64_t)rintl(exp2l((long double)j / 256.0L) * 9223372036854775808.0L); // 2^63
 }
 
 __global__ void math_eval_kernel(int fn, const double *x, double *out, int64_t n, MathTables T)

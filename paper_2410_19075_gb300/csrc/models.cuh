@@ -7,6 +7,7 @@
 #pragma once
 #include "common.cuh"
 #include "fastmath.cuh"
+#include "hh_rates.cuh"
 
 namespace simk {
 
@@ -257,7 +258,8 @@ template <> struct Model<1> {
 //   dx/dt    = alpha_x(V) (1-x) - beta_x(V) x,   x in {m, h, n}
 // with CV = sum_{j in W(i)} (V_j - V_i) = W_V - wsize * Q(V_i), exact in fixed point.
 // c = {1/Cm, gNa, gK, gL, ENa, EK, EL, g/K}.  Coupled quantity V; the gates are
-// local variables.  Rates use the table-driven exp and reciprocal of fastmath.cuh.
+// local variables.  The rates come from integer arithmetic (hh_rates.cuh); 31
+// FP64 instructions per node are left.
 template <> struct Model<2> {
     static constexpr int D = 4, NQ = 1, NX = 3, F = 46;
     static constexpr bool OWN_OUT = false;
@@ -270,33 +272,27 @@ template <> struct Model<2> {
                                                const int64_t (&qo)[NQ], const i128 (&W)[NQ], const double *X,
                                                double Iext, double (&k)[D], int64_t wsize, double cs)
     {
-        slope(P, fo[0], cs * fixed_to_double_wide(W[0] - (i128)qo[0] * wsize, F_), X, Iext, k);
+        slope(P, qo[0], fo[0], cs * fixed_to_double_wide(W[0] - (i128)qo[0] * wsize, F_), X, Iext, k);
     }
     // Rings: c[7] carries 2^(ksh - F).
     __device__ __forceinline__ static void rhs_ring(const ModelParams &P, const int64_t (&qo)[NQ],
                                                     const int64_t (&S)[NQ], const double *X, double Iext,
                                                     double (&k)[D])
     {
-        slope(P, ll2double_scaled(qo[0], F), __ll2double_rn(S[0] - own_multiple(P, qo[0])), X, Iext, k);
+        slope(P, qo[0], ll2double_scaled(qo[0], F), __ll2double_rn(S[0] - own_multiple(P, qo[0])), X, Iext, k);
     }
-    __device__ __forceinline__ static void slope(const ModelParams &P, double V, double CV, const double *X,
+    __device__ __forceinline__ static void slope(const ModelParams &P, int64_t q, double V, double CV, const double *X,
                                                  double Iext, double (&k)[D])
     {
         const double m = X[0], h = X[1], n = X[2];
-        const MathTables &T = P.tab;
-        const double am = fast_x_over_1mexp(fma(V, 0.1, 4.0), T);                    // (V+40)/10
-        const double bm = 4.0 * fast_exp(fma(V, -1.0 / 18.0, -65.0 / 18.0), T);     // -(V+65)/18
-        const double ah = 0.07 * fast_exp(fma(V, -0.05, -3.25), T);                 // -(V+65)/20
-        const double bh = fast_rcp(1.0 + fast_exp(fma(V, -0.1, -3.5), T));          // -(V+35)/10
-        const double an = 0.1 * fast_x_over_1mexp(fma(V, 0.1, 5.5), T);             // (V+55)/10
-        const double bn = 0.125 * fast_exp(fma(V, -0.0125, -0.8125), T);            // -(V+65)/80
+        const HHRates r = hh_rates(q, P.tab);
         const double m3h = m * m * m * h, n4 = (n * n) * (n * n);
         const double I = Iext - P.c[1] * m3h * (V - P.c[4]) - P.c[2] * n4 * (V - P.c[5]) -
                          P.c[3] * (V - P.c[6]) + P.c[7] * CV;
         k[0] = I * P.c[0];
-        k[1] = am * (1.0 - m) - bm * m;
-        k[2] = ah * (1.0 - h) - bh * h;
-        k[3] = an * (1.0 - n) - bn * n;
+        k[1] = fma(-(r.am + r.bm), m, r.am); // alpha (1 - x) - beta x
+        k[2] = fma(-(r.ah + r.bh), h, r.ah);
+        k[3] = fma(-(r.an + r.bn), n, r.an);
     }
 };
 

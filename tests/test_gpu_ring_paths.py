@@ -11,7 +11,8 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("model", [0, 1, 2, 3])
-@pytest.mark.parametrize("N,R", [(129, 64), (257, 1), (1025, 256), (1921, 960), (4095, 2000), (4096, 2047)])
+@pytest.mark.parametrize("N,R", [(129, 64), (257, 1), (1025, 256), (1921, 960), (4095, 2000), (4096, 2047),
+                                 (5120, 700), (8191, 4095), (8192, 1)])
 def test_cluster_slices_equal_streaming_bitwise(model, N, R):
     """Slice sizes with a ragged last slice and windows up to the whole ring; the
     slope read after the run comes from the prefix form the cluster kernel leaves."""
@@ -46,3 +47,30 @@ def test_fhn_slope_both_forms_match_oracle(R, sigma, a):
         k = net.rhs().reshape(2, N)[:, q]
     ref = oracle.rhs_sampled(1, 0, N, R, params, y0, q)
     assert np.abs(k - ref).max() < 1e-12 * max(1.0, np.abs(ref).max())
+
+
+def test_hh_rates_over_the_voltage_range():
+    """The gates' slopes over |V| < 256 mV and next to the removable singularities at
+    -40 and -55 mV (series below 0.625 mV from them).  alpha - (alpha + beta) x cancels,
+    so the bound is 1e-14 of alpha + beta (the rates' error is below 2^-52 and the oracle's
+    libm and cancellation a few times that; 1 - exp(-x) at 0.06 loses four bits there)."""
+    from paper_2410_19075_gb300 import Network
+    rng = np.random.default_rng(9)
+    near = np.concatenate([s + d * sgn for s in (-40.0, -55.0) for sgn in (-1, 1)
+                           for d in [np.array([0.0, 1e-9, 0.624, 0.625, 0.626, 0.9])]])
+    V = np.concatenate([near, np.linspace(-255.9, 255.9, 1999), rng.uniform(-90, 50, 2000)])
+    N, R = V.size, 3
+    gates = rng.uniform(0.0, 1.0, 3 * N)
+    params = I.hh_params()
+    y0 = np.concatenate([V, gates])
+    for streaming in (False, True):
+        with Network(2, 0, N, R, params, streaming=streaming) as net:
+            net.set_state(y0)
+            k = net.rhs().reshape(4, N)
+        ref = oracle.rhs_sampled(2, 0, N, R, params, y0, np.arange(N))
+        zero, one = y0.copy(), y0.copy()
+        zero[N:], one[N:] = 0.0, 1.0
+        alpha = oracle.rhs_sampled(2, 0, N, R, params, zero, np.arange(N))[1:]
+        beta = -oracle.rhs_sampled(2, 0, N, R, params, one, np.arange(N))[1:]
+        assert (np.abs(k[1:] - ref[1:]) / (alpha + beta)).max() < 1e-14
+        assert np.abs(k[0] - ref[0]).max() < 1e-12 * np.abs(ref[0]).max()
