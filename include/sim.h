@@ -87,8 +87,8 @@ typedef enum {
 
 /* Creation flags. */
 #define SIM_FLAG_INCLUDE_SELF 1u /* count the node itself as one of its links */
-#define SIM_FLAG_STREAMING 2u    /* rings of <= 4096 nodes: use the multi-launch streaming kernels
-                                    instead of the thread-block-cluster kernel (same results) */
+#define SIM_FLAG_STREAMING 2u    /* rings of <= 8192 nodes (HH 5120): use the multi-launch streaming
+                                    kernels instead of the thread-block-cluster kernel (same results) */
 #define SIM_FLAG_LOW_MEMORY 4u   /* ball and disk lattices: keep one periodically extended row
                                     prefix (about 16 B per node) instead of one x-window array
                                     per chord half-width ((P+1) * 16 B per node, the default for

@@ -146,11 +146,14 @@ cudaError_t dp_launch(int ds, const DpGroup &g, cudaStream_t s);
 
 // Ring: f(y) -> lam[0], ofs[0] and the order parameter of y (Kuramoto).
 cudaError_t ring_prologue(const RingPlan &p, cudaStream_t s);
-// Small rings (N <= kClusterMaxNodes): all stages of n_steps RK4 steps in one
-// thread-block-cluster launch (ring_cluster.cu).  Same results as ring_step.
-constexpr int64_t kClusterMaxNodes = 4096;
+// Small rings (N <= kClusterMaxNodes, HH kClusterMaxNodesHH): all stages of n_steps
+// RK4 steps in one thread-block-cluster launch (ring_cluster.cu).  Same results
+// as ring_step.  Per RK4 step, cluster against streaming kernels: KS 10.2 / 21.8 us
+// at N = 5000 and 12.0 / 21.3 us at 8192 (512 nodes per CTA, the most a CTA takes);
+// HH 20.7 / 23.6 us at 5000, 30.5 / 23.1 us at 8192.
+constexpr int64_t kClusterMaxNodes = 8192, kClusterMaxNodesHH = 5120;
 cudaError_t ring_cluster_configure(); // per device, before the first cluster launch
-int cluster_size_for(int64_t N);      // CTAs of the cluster for a ring of N nodes (0: not eligible)
+int cluster_size_for(int model, int64_t N); // CTAs of the cluster for a ring of N nodes (0: not eligible)
 cudaError_t ring_cluster_steps(const RingPlan &p, double dt, int64_t n_steps, cudaStream_t s);
 
 // Ring: stage 1 only with dt = 0, so acc receives f(y) and y is untouched.

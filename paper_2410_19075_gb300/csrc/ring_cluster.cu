@@ -259,7 +259,7 @@ __global__ void __launch_bounds__(kClusterThreadsMax, 1)
                 const i128 start = e >= 0 ? ((i128)hs[c] << sh) + los[c] + ps[c] : (i128)0;
                 const i128 here = ((i128)hi[c] << sh) + lo[c] + pi[c];
                 P.lam[0][(int64_t)i * NQ + c] = (int64_t)(here - start);
-                // one prefix group (at most 16 sub-tiles): in-group offsets are the sub-tile starts
+                // one prefix group (at most 32 sub-tiles): in-group offsets are the sub-tile starts
                 if (!(i & (kSubTile - 1))) st_i128(P.ingrp[0] + c * P.nsub + sub, start);
                 if (i == 0) {
                     st_i128(P.grpofs[0] + c * (P.ngroups + 1), 0);
@@ -273,9 +273,9 @@ __global__ void __launch_bounds__(kClusterThreadsMax, 1)
 
 static int g_max_cluster = 8; // 16 when the device can co-schedule it (set by configure)
 
-int cluster_size_for(int64_t N)
+int cluster_size_for(int model, int64_t N)
 {
-    if (N > kClusterMaxNodes) return 0;
+    if (N > (model == 2 ? kClusterMaxNodesHH : kClusterMaxNodes)) return 0;
     int cl = (int)((N + 127) / 128);
     if (cl < 2) cl = 2;
     if (cl > g_max_cluster) cl = g_max_cluster;
@@ -334,7 +334,7 @@ static cudaError_t launch_cluster(const RingPlan &p, double dt, int64_t n_steps,
 
 cudaError_t ring_cluster_steps(const RingPlan &p, double dt, int64_t n_steps, cudaStream_t s)
 {
-    const int cl = cluster_size_for(p.N);
+    const int cl = cluster_size_for(p.model, p.N);
     if (cl == 0) return cudaErrorInvalidValue;
     cudaError_t e;
     switch (p.model) {

@@ -296,7 +296,7 @@ int check_device_error(sim_t h)
 
 bool use_cluster(sim_t h)
 {
-    return h->topo == SIM_RING && !(h->flags & SIM_FLAG_STREAMING) && cluster_size_for(h->N) > 0;
+    return h->topo == SIM_RING && !(h->flags & SIM_FLAG_STREAMING) && cluster_size_for(h->model, h->N) > 0;
 }
 
 cudaError_t launch_steps(sim_t h, int64_t n, double dt, cudaStream_t s)
