@@ -89,10 +89,10 @@ typedef enum {
 #define SIM_FLAG_INCLUDE_SELF 1u /* count the node itself as one of its links */
 #define SIM_FLAG_STREAMING 2u    /* rings of <= 8192 nodes (HH 5120): use the multi-launch streaming
                                     kernels instead of the thread-block-cluster kernel (same results) */
-#define SIM_FLAG_LOW_MEMORY 4u   /* ball and disk lattices: keep one periodically extended row
-                                    prefix (about 16 B per node) instead of one x-window array
-                                    per chord half-width ((P+1) * 16 B per node, the default for
-                                    P >= 5 when it stays within 8 GiB), at two loads per chord
+#define SIM_FLAG_LOW_MEMORY 4u   /* ball lattices: keep one periodically extended row prefix (about
+                                    16 B per node, what disks always keep) instead of one x-window
+                                    array per chord half-width ((P+1) * 16 B per node, the default
+                                    for P >= 5 when it stays within 8 GiB), at two loads per chord
                                     instead of one; the results are the same bits */
 
 /* Bytes of device memory sim_create() allocates for this network with flags 0
@@ -172,7 +172,7 @@ int sim_step(sim_t h, int64_t n_steps, double dt);
  * with a kernel of kind k, launches_by_kind[k] their number (4 entries each):
  * kind 0 = the fused stage kernel of a ring or link matrix (one per stage; the
  * whole call for the cluster-resident small-ring kernel), the x pass of a ball
- * or disk, or the cube's order-parameter total (once per step), 1 = the y pass
+ * or disk, or a lattice's order-parameter total (once per step), 1 = the y pass
  * of the cube, 2 = the node pass of a lattice (the cube's elementwise RK4 pass
  * fused with the next stage's x pass, the chord gather of the ball and disk),
  * 3 = the z-window pass of the cube.  The

@@ -179,7 +179,7 @@ struct LatticePlan {
     int64_t *sx;      // cube: 2 * nodes window sums along x (SoA); ball, disk: per row,
                       // rs (sin, cos) pairs of the periodically extended inclusive
                       // prefix E(x), x in [-P-1, N1+P-1], stored at x + P + 1
-    int64_t rs;       // ball, disk: row stride of sx in (sin, cos) pairs, N1 + 2P + 1
+    int64_t rs;       // ball, disk: row stride of sx in (sin, cos) pairs (lattice_row_stride)
     int wmode;        // ball, disk: sx holds, for w = 0..P, nodes (sin, cos) pairs of the
                       // x-window sums S_w (one load per chord) instead of the row prefixes
     int64_t *sxy;     // cube box sums over x and y: 2 components, i-block-major (tiled passes)
@@ -192,8 +192,12 @@ struct LatticePlan {
     double *obs;
     int64_t obs_cap;
     unsigned long long *obs_ctr;
-    const int4 *chords; // ball/disk: (dy, dz, w, 0) chords of the window
-    int nchords;
+    // ball/disk: the reads (row shift, plane shift, half-width, 0) of the windows of a
+    // thread's block of lattice_gather_nodes nodes together (lattice_gather_kernel), by the set of nodes
+    // that add them: the reads of set m (bit jj + 2 kk = node (j + jj, k + kk)) end at
+    // op_end[m] and start at op_end[m - 1]
+    const int4 *ops;
+    int nops, op_end[16];
     const int *skip;    // if set and nonzero, the x, y and gather passes of stage 1 return at once
                         // (a finished Dormand-Prince run); nullptr for every other use
 };
@@ -236,6 +240,8 @@ cudaError_t lattice_configure(); // once per process, before the first launch
 int64_t lattice_order_blocks(int topo, int64_t N1); // CTAs of the order-parameter passes (sliding-window grid)
 int64_t lattice_sxy_elems(int64_t N1); // cube: xy-window sums (both layouts of the y pass's output)
 int64_t lattice_partial_blocks(int topo, int64_t N1); // order-parameter partials to allocate (every grid)
+int64_t lattice_row_stride(int64_t N1, int64_t P, bool wmode);
+int lattice_gather_nodes(int topo, int64_t N1); // nodes per thread of the ball and disk gather
 int64_t lattice_sx_elems(int topo, int64_t N1, int64_t P, bool wmode); // int64 elements of sx
 constexpr int64_t kLatticeWindowBudget = int64_t(8) << 30; // bytes of the per-w window arrays
 cudaError_t lattice_prologue(const LatticePlan &p, cudaStream_t s);
@@ -264,7 +270,7 @@ void ring_coupling_constants(ModelParams &mp, int model, const double *params, i
 // Per-kernel timing of sim_step_timed: while set on the launching host thread,
 // every stage-kernel launch of ring_step, graph_step, lattice_step and
 // ring_cluster_steps records an event of its kind right after itself (kinds:
-// 0 fused ring / link-matrix stage kernel, lattice x pass or the cube's
+// 0 fused ring / link-matrix stage kernel, lattice x pass or a lattice's
 // order-parameter total, 1 cube y pass, 2 lattice node pass (cube node pass
 // fused with the next x pass, ball / disk gather), 3 cube z-window pass).  Never set during a stream capture.
 struct KernelMarks {

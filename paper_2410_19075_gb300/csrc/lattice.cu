@@ -18,16 +18,17 @@
 //           Batched cubes use sliding windows along j and k instead, the z pass
 //           fused with the node update.
 // Ball and disk, per RK4 stage:
-//   x pass  for every half-width w = 0..P the x-window sums S_w(i) of Q(f) along
-//           every row, sin and cos interleaved; or, when those P+1 arrays would
-//           exceed the memory budget (or SIM_FLAG_LOW_MEMORY), the inclusive row
-//           prefix E(x) extended periodically by P + 1 entries on the left and P
-//           on the right (wrapping int64);
+//   x pass  balls of P >= 5: for every half-width w = 0..P the x-window sums S_w(i) of
+//           Q(f) along every row, sin and cos interleaved; otherwise, and when those
+//           P+1 arrays would exceed the memory budget (or SIM_FLAG_LOW_MEMORY), the
+//           inclusive row prefix E(x) extended periodically by P + 1 entries on the
+//           left and P on the right (wrapping int64);
 //   gather  W = sum over the chords of the window, one per (dy, dz) (ball) or dy
 //           (disk): the row segment |dx| <= w = floor(sqrt(P^2 - dy^2 - dz^2)),
 //           read as S_w (one 16-byte load) or E(i + w) - E(i - w - 1) (two),
-//           O(P^2) resp. O(P) reads per node, fused with the right-hand side and
-//           RK4 update.
+//           O(P^2) resp. O(P) reads per node, up to four neighbouring nodes per thread
+//           sharing the reads their windows have in common, fused with the right-hand side
+//           and RK4 update.
 #include <algorithm>
 
 #include "internal.h"
@@ -38,7 +39,8 @@ constexpr int kRowWarpsMax = 8;       // x pass: one warp per row
 constexpr int kColThreads = 128;      // cube y and z passes: threads per CTA along i
 constexpr int64_t kColTarget = 152 * 1024; // cube y and z passes: columns are split into
                                            // segments until about this many threads run
-constexpr int kGatherThreads = 256;   // ball/disk gather: one node per thread
+constexpr int kGatherThreads = 128;   // ball/disk gather: a block of rows x planes of nodes per thread
+constexpr int kGatherOps = 512;       // ball/disk gather: reads of the window held in shared memory at a time
 constexpr size_t kRowSmemMax = 220 * 1024;
 
 // i-columns per tile: shared memory 2 (N1 + 1) BI 8 bytes stays below ~76 KB
@@ -98,14 +100,17 @@ __device__ __forceinline__ void lattice_rotated_q(const LatticePlan &p, int64_t 
 }
 
 // x pass: one warp per row.  pre(p) = sum_{m<p} Q'(f(m)) for p in [0, N1] is built
-// in shared memory (stride N1 + 1 per component).  With Pe(p) = pre(p mod N1) +
-// floor(p / N1) pre(N1) the periodic extension:
-//   MODE 0 (cube)        SX(i) = Pe(i+P+1) - Pe(i-P), sin and cos in two arrays;
+// in shared memory.  With Pe(p) = pre(p mod N1) + floor(p / N1) pre(N1) the
+// periodic extension:
+//   MODE 0 (cube)        SX(i) = Pe(i+P+1) - Pe(i-P), sin and cos in two arrays
+//                        (pre0/pre1, stride N1 + 1 per component);
 //   MODE 1 (ball, disk,  the extended inclusive prefix E(x) = Pe(x+1),
 //           low memory)  x in [-P-1, N1+P-1], (sin, cos) pairs, modulo 2^64;
-//   MODE 2 (ball, disk)  for every half-width w = 0..P the window sums
+//   MODE 2 (ball)        for every half-width w = 0..P the window sums
 //                        S_w(i) = Pe(i+w+1) - Pe(i-w), (sin, cos) pairs, one
-//                        array of nodes pairs per w.
+//                        array of rows per w.
+// Modes 1 and 2 build Pe on [-P, N1 + P] as (sin, cos) pairs (lattice_ext_row) where
+// that fits in shared memory; longer rows (disks only, mode 1) use pre0/pre1.
 // One row of the x pass (one warp; pre0/pre1 its shared prefix rows).
 // IBLK (cube, the tiled passes): SX in the plane-wise i-block-major layout
 // [k][i-block][j][ii] (cube_sx_index), which each y tile reads as one
@@ -171,19 +176,7 @@ __device__ __forceinline__ void lattice_x_scan_out(const LatticePlan &p, int64_t
         pre1[0] = 0;
     }
     __syncwarp();
-    if (MODE == 2) {
-        const int64_t t0 = pre0[N1], t1 = pre1[N1];
-        longlong2 *__restrict__ o = reinterpret_cast<longlong2 *>(p.sx) + row * N1;
-        for (int64_t w = 0; w <= P; ++w, o += nodes) {
-            for (int64_t i = lane; i < N1; i += 32) {
-                int64_t b = i + w + 1, a = i - w;
-                int64_t s0 = 0, s1 = 0;
-                if (b > N1) { b -= N1; s0 += t0; s1 += t1; }
-                if (a < 0) { a += N1; s0 += t0; s1 += t1; } // Pe(a) = pre(a+N1) - total
-                o[i] = make_longlong2(s0 + pre0[b] - pre0[a], s1 + pre1[b] - pre1[a]);
-            }
-        }
-    } else if (MODE == 1) {
+    if (MODE == 1) {
         // E(x) = Pe(x + 1) for x in [-P-1, N1+P-1], at slot x + P + 1
         const uint64_t t0 = (uint64_t)pre0[N1], t1 = (uint64_t)pre1[N1];
         longlong2 *__restrict__ o = reinterpret_cast<longlong2 *>(p.sx) + row * p.rs;
@@ -254,6 +247,91 @@ __device__ __forceinline__ void lattice_x_row(const LatticePlan &p, int64_t row,
 {
     lattice_x_fill<MODE>(p, row, pre0, pre1);
     lattice_x_scan_out<MODE, IBLK>(p, row, pre0, pre1);
+}
+
+// Ball and disk: the row's extended prefix in shared memory, ext[p + P] = Pe(p)
+// for p in [-P, N1 + P], then the outputs read straight from it: a window sum is
+// two 16-byte shared loads and no wrap test (36 -> 24 us for seven windows of
+// 10^6 nodes; the wrapped form took 20 of its 27 instructions per window).
+// Lanes own an odd number of adjacent slots, so their 16-byte accesses do not
+// share banks.
+template <int MODE>
+__device__ __forceinline__ void lattice_ext_row(const LatticePlan &p, int64_t row, longlong2 *ext)
+{
+    const int lane = threadIdx.x & 31, n1 = (int)p.N1, P = (int)p.P;
+    const longlong2 *__restrict__ fr = reinterpret_cast<const longlong2 *>(p.f) + row * n1;
+    longlong2 *pre = ext + P; // pre[q] = Pe(q)
+    for (int mb = lane; mb < n1; mb += 32 * 4) { // 4 loads in flight per lane
+        longlong2 v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) v[u] = mb + 32 * u < n1 ? __ldg(fr + mb + 32 * u) : make_longlong2(0, 0);
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (mb + 32 * u < n1) {
+                int64_t qs, qc;
+                lattice_rotated_q(p, v[u].x, v[u].y, qs, qc);
+                pre[mb + 32 * u + 1] = make_longlong2(qs, qc);
+            }
+    }
+    __syncwarp();
+    const int per = ((n1 + 31) >> 5) | 1;
+    const int m0 = min(lane * per, n1) + 1, m1 = min(m0 + per, n1 + 1);
+    uint64_t r0 = 0, r1 = 0; // wrapping sums
+    for (int m = m0; m < m1; ++m) {
+        const longlong2 v = pre[m];
+        r0 += (uint64_t)v.x;
+        r1 += (uint64_t)v.y;
+    }
+    const uint64_t i0 = (uint64_t)warp_incl_scan((int64_t)r0), i1 = (uint64_t)warp_incl_scan((int64_t)r1);
+    uint64_t e0 = i0 - r0, e1 = i1 - r1;
+    for (int m = m0; m < m1; ++m) {
+        const longlong2 v = pre[m];
+        e0 += (uint64_t)v.x;
+        e1 += (uint64_t)v.y;
+        pre[m] = make_longlong2((long long)e0, (long long)e1);
+    }
+    if (lane == 0) pre[0] = make_longlong2(0, 0);
+    const uint64_t t0 = __shfl_sync(0xffffffffu, i0, 31), t1 = __shfl_sync(0xffffffffu, i1, 31); // the row's total
+    __syncwarp();
+    for (int q = lane; q < P; q += 32) { // 2P + 1 <= N1: both extensions read pre[0..N1]
+        const longlong2 lo = pre[q - P + n1], hi = pre[q + 1];
+        pre[q - P] = make_longlong2((long long)((uint64_t)lo.x - t0), (long long)((uint64_t)lo.y - t1));
+        pre[n1 + q + 1] = make_longlong2((long long)((uint64_t)hi.x + t0), (long long)((uint64_t)hi.y + t1));
+    }
+    __syncwarp();
+    longlong2 *__restrict__ sx = reinterpret_cast<longlong2 *>(p.sx);
+    if (MODE == 1) {
+        longlong2 *__restrict__ o = sx + row * p.rs;
+        for (int e = lane; e < (int)p.rs; e += 32) o[e] = ext[e];
+    } else {
+        longlong2 *__restrict__ o = sx + row * p.rs;
+        const int64_t warray = p.nodes / n1 * p.rs;
+        for (int w = 0; w <= P; ++w, o += warray)
+#pragma unroll 4
+            for (int i = lane; i < n1; i += 32) {
+                const longlong2 hi = pre[i + w + 1], lo = pre[i - w];
+                o[i] = make_longlong2((long long)((uint64_t)hi.x - (uint64_t)lo.x),
+                                      (long long)((uint64_t)hi.y - (uint64_t)lo.y));
+            }
+    }
+    __syncwarp();
+}
+
+template <int MODE>
+__global__ void __launch_bounds__(32 * kRowWarpsMax) lattice_ext_kernel(LatticePlan p)
+{
+    if (p.skip && *(const volatile int *)p.skip) return;
+    extern __shared__ __align__(16) longlong2 ext_mem[];
+    const int warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+    const int64_t rows = p.nodes / p.N1, row = (int64_t)blockIdx.x * nwarps + warp;
+    if (row < rows) lattice_ext_row<MODE>(p, row, ext_mem + warp * (p.N1 + 2 * p.P + 1)); // uniform over the warp
+}
+
+// Warps per CTA of lattice_ext_kernel (0: the row's extension does not fit).
+static int ext_warps(int64_t N1, int64_t P)
+{
+    const int64_t w = (int64_t)(kRowSmemMax / (sizeof(longlong2) * (size_t)(N1 + 2 * P + 1)));
+    return (int)(w > kRowWarpsMax ? kRowWarpsMax : w);
 }
 
 template <int MODE>
@@ -450,10 +528,18 @@ __device__ void lattice_record_order(const LatticePlan &p, i128 ps, i128 pc, uns
 }
 
 // The order parameter from the partials of a previous launch of nblk CTAs (the
-// cube's fused node pass, whose CTAs only store their partials): CTA g adds up
+// cube's fused node pass and the ball's and disk's gather, whose CTAs only store
+// their partials): CTA g adds up
 // its slice of them into the pair nblk + g, and the last of the kOrderCtas CTAs
 // to finish (arrival counter tile_ctr) adds those up.
 constexpr int kOrderCtas = 128, kOrderThreads = 256;
+constexpr unsigned kOrderInline = 1024; // gathers of at most this many CTAs: their last CTA records R itself
+                                        // (one launch less; with more CTAs the fences cost more than the launch)
+static unsigned order_grid(unsigned nblk) // one CTA per 64 partials, up to kOrderCtas
+{
+    const unsigned g = (nblk + 63) / 64;
+    return g < 1 ? 1u : g > (unsigned)kOrderCtas ? (unsigned)kOrderCtas : g;
+}
 __global__ void __launch_bounds__(kOrderThreads) lattice_order_kernel(LatticePlan p, unsigned nblk)
 {
     if (p.skip && *(const volatile int *)p.skip) return;
@@ -783,6 +869,33 @@ __global__ void __launch_bounds__(kTileThreads) cube_y_tile_kernel(LatticePlan p
     }
 }
 
+// A node's coupling term to cpl (KM = -1), or its whole slope to acc for a
+// right-hand-side evaluation of model KM (the stage input's own variables are y).
+template <int KM>
+__device__ __forceinline__ void lattice_write_slope(const LatticePlan &p, int64_t n, double c)
+{
+    if constexpr (KM < 0) {
+        p.cpl[n] = c;
+    } else {
+        constexpr int D = Model<KM>::D, NX = Model<KM>::NX, XOFF = D - NX;
+        double X[NX > 0 ? NX : 1], k[D];
+#pragma unroll
+        for (int g = 0; g < NX; ++g) X[g] = p.y[(XOFF + g) * p.nodes + n];
+        Model<KM>::rhs_from_coupling(p.mp, c, X, k);
+#pragma unroll
+        for (int v = 0; v < D; ++v) p.acc[v * p.nodes + n] = k[v];
+    }
+}
+
+// Ball and disk: from the rotated window sums and the node's own (sin, cos).
+template <int KM>
+__device__ __forceinline__ void lattice_write_coupling(const LatticePlan &p, int64_t n, int64_t W0, int64_t W1)
+{
+    const longlong2 f = reinterpret_cast<const longlong2 *>(p.f)[n];
+    const int64_t f62[2] = {f.x, f.y};
+    lattice_write_slope<KM>(p, n, lattice_coupling_term(p.mp, f62, W0, W1));
+}
+
 // Tiled cube z pass, split in two kernels per stage:
 //   window pass  CTA (ib, j) scans the xy-window sums of its columns along k and
 //                writes every node's coupling term (lattice_coupling_term, the
@@ -802,6 +915,7 @@ __global__ void __launch_bounds__(kTileThreads) cube_y_tile_kernel(LatticePlan p
 // plane per iteration 0.860 ms; 512 threads (at most 42 registers) 0.884 ms.
 constexpr int kZThreads = 384, kZAhead = 3, kZBlocks = 3; // kZAhead: planes of own (sin, cos) in flight
 
+template <int KM> // -1: coupling terms; a model: the slopes of a right-hand-side evaluation
 __global__ void __launch_bounds__(kZThreads, kZBlocks) cube_zw_tile_kernel(LatticePlan p)
 {
     if (p.skip && *(const volatile int *)p.skip) return;
@@ -820,7 +934,6 @@ __global__ void __launch_bounds__(kZThreads, kZBlocks) cube_zw_tile_kernel(Latti
     const uint64_t *col0 = tile + ii, *col1 = tile + cstride + ii;
     const uint64_t t0 = col0[(unsigned)N1 << lg], t1 = col1[(unsigned)N1 << lg];
     const longlong2 *__restrict__ fp = reinterpret_cast<const longlong2 *>(p.f) + base + ii; // (sin, cos) pairs
-    double *__restrict__ cpl = p.cpl + base + ii;
     int64_t f[kZAhead + 1][2]; // own (sin, cos) of the planes a, a + rstep, ...
 #pragma unroll
     for (int d = 0; d < kZAhead; ++d) {
@@ -837,8 +950,9 @@ __global__ void __launch_bounds__(kZThreads, kZBlocks) cube_zw_tile_kernel(Latti
         f[kZAhead][1] = v.y;
         int64_t t62[2];
         own_phase_turned(p.mp, f[0], t62);
-        cpl[(unsigned)a * plane] = lattice_coupling_term(p.mp, t62, cube_tile_window(col0, N1, P, lg, a, t0),
-                                                         cube_tile_window(col1, N1, P, lg, a, t1));
+        lattice_write_slope<KM>(p, base + ii + (unsigned)a * plane,
+                                lattice_coupling_term(p.mp, t62, cube_tile_window(col0, N1, P, lg, a, t0),
+                                                      cube_tile_window(col1, N1, P, lg, a, t1)));
 #pragma unroll
         for (int d = 0; d < kZAhead; ++d) {
             f[d][0] = f[d + 1][0];
@@ -959,51 +1073,157 @@ __global__ void __launch_bounds__(kColThreads)
     cube_z_col<M, STAGE>(p, h, bx, j, seg, (unsigned)lb, (unsigned)(nbx * p.N1 * col_segments(p.N1)));
 }
 
-// ball / disk gather: one node per thread; the window is the union of the chords
-// (dy, dz, w) of the plan's table.  WMODE: one load per chord, the x-window sum
-// S_w of the chord's row; otherwise two, the difference of the row's extended
-// prefix at both ends (wrapping arithmetic; every chord sum and the window sum
-// itself are exact either way, so both give the same bits).
-template <int M, int STAGE, bool WMODE>
-__global__ void __launch_bounds__(kGatherThreads) lattice_gather_kernel(LatticePlan p, const StepSize h)
+// ball / disk gather: a thread gathers the window sums of kGatherTj x TK nodes (j,
+// j + 1; k, k + 1; disks one plane) at column i.  The plan's table lists the reads
+// of all its windows together, (row shift a from row j - P, plane shift z from plane
+// k - P, half-width w) in the order of the set of nodes that add them: a row segment
+// that several of the windows share is read once (69 reads per node for the 113
+// chords of P = 6, 89 with two nodes per thread).  WMODE: one load per read, the
+// x-window sum S_w of the row; otherwise two, the difference of the row's
+// extended prefix at both ends (wrapping arithmetic; every chord sum and the
+// window sum itself are exact either way, so both give the same bits).  Per CTA the
+// reads' offsets are put into shared memory with the plane's wrap resolved (two
+// reads per 16-byte shared load), so that a read costs a thread the row's wrap, one
+// multiply-add and the load.  Rows of window arrays are padded to 8 pairs, and
+// threads run over the padded columns, so that 8 lanes read one 128-byte line.
+// What bounds it: the L1 data array (16 B per read, and about as much again for the
+// lines that arrive from L2).  N1 = 100, P = 6, per stage: one node per thread, with
+// both wraps and 64-bit addresses formed per chord, took 36 instructions per chord
+// and 152 us; two nodes per thread 88 us; now 84 us.
+template <bool WMODE>
+__device__ __forceinline__ void gather_read(const longlong2 *base, int j0, int n1, unsigned rowlen, unsigned aw,
+                                            unsigned off, uint64_t (&v)[2])
 {
-    if (STAGE == 1 && p.skip && *(const volatile int *)p.skip) return; // stage 1 records nothing
-    const int64_t N1 = p.N1, nodes = p.nodes;
-    const int64_t n = (int64_t)blockIdx.x * kGatherThreads + threadIdx.x;
+    const unsigned jj = (unsigned)j0 + (aw & 0xffffu), jw = min(jj, jj - (unsigned)n1); // row mod N1
+    const longlong2 *r = base + (size_t)(off + jw * rowlen);
+    if (WMODE) {
+        const longlong2 x = __ldg(r);
+        v[0] = (uint64_t)x.x;
+        v[1] = (uint64_t)x.y;
+    } else {
+        const int w = (int)(aw >> 16);
+        const longlong2 hi = __ldg(r + w), lo = __ldg(r - w - 1);
+        v[0] = (uint64_t)hi.x - (uint64_t)lo.x;
+        v[1] = (uint64_t)hi.y - (uint64_t)lo.y;
+    }
+}
+
+// The reads [q, e) of the chunk, which the nodes of the set MASK add.
+template <int MASK, int NB, bool WMODE>
+__device__ __forceinline__ void gather_class(const uint2 *s_op, int q, int e, const longlong2 *base, int j0, int n1,
+                                             unsigned rowlen, uint64_t (&W)[NB][2])
+{
+    auto add = [&](const uint64_t (&x)[2]) {
+#pragma unroll
+        for (int b = 0; b < NB; ++b)
+            if (MASK >> b & 1) {
+                W[b][0] += x[0];
+                W[b][1] += x[1];
+            }
+    };
+    if ((q & 1) && q < e) { // to an even read
+        const uint2 o = s_op[q++];
+        uint64_t x[2];
+        gather_read<WMODE>(base, j0, n1, rowlen, o.x, o.y, x);
+        add(x);
+    }
+#pragma unroll (WMODE ? 3 : 2) // measured: 3 reads ahead cost the two-load form registers
+    for (; q + 1 < e; q += 2) {
+        const uint4 o = *reinterpret_cast<const uint4 *>(s_op + q);
+        uint64_t x[2], y[2];
+        gather_read<WMODE>(base, j0, n1, rowlen, o.x, o.y, x);
+        gather_read<WMODE>(base, j0, n1, rowlen, o.z, o.w, y);
+#pragma unroll
+        for (int b = 0; b < NB; ++b)
+            if (MASK >> b & 1) {
+                W[b][0] += x[0] + y[0];
+                W[b][1] += x[1] + y[1];
+            }
+    }
+    if (q < e) {
+        const uint2 o = s_op[q];
+        uint64_t x[2];
+        gather_read<WMODE>(base, j0, n1, rowlen, o.x, o.y, x);
+        add(x);
+    }
+}
+template <int MASK, int NB, bool WMODE>
+__device__ __forceinline__ void gather_classes(const int *start, int c0, int n, const uint2 *s_op,
+                                               const longlong2 *base, int j0, int n1, unsigned rowlen,
+                                               uint64_t (&W)[NB][2])
+{
+    if constexpr (MASK < (1 << NB)) {
+        const int q = max(start[MASK - 1] - c0, 0), e = min(start[MASK] - c0, n);
+        if (q < e) gather_class<MASK, NB, WMODE>(s_op, q, e, base, j0, n1, rowlen, W);
+        gather_classes<MASK + 1, NB, WMODE>(start, c0, n, s_op, base, j0, n1, rowlen, W);
+    }
+}
+
+// STAGE 1-4: the RK4 stage; 0: the prologue (no gather); 5: the slopes into acc (a
+// right-hand-side evaluation).  NB nodes per thread (LatticePlan::nb).
+template <int M, int STAGE, bool WMODE, int NB>
+__global__ void __launch_bounds__(kGatherThreads, 7) lattice_gather_kernel(LatticePlan p, const StepSize h)
+{
+    if (STAGE == 5 && p.skip && *(const volatile int *)p.skip) return;
+    constexpr int TJ = NB > 1 ? 2 : 1, TK = NB > 2 ? 2 : 1; // rows and planes of a thread's block
+    const int n1 = (int)p.N1, P = (int)p.P, tid = threadIdx.x;
+    const unsigned cols = (unsigned)(n1 + 7) & ~7u, t = blockIdx.x * kGatherThreads + tid, jp = t / cols;
+    const int i = (int)(t - jp * cols), j = TJ * (int)jp, k = TK * blockIdx.y;
+    const bool live = i < n1 && j < n1;
+    uint64_t W[NB][2] = {};
+    if (STAGE > 0) {
+        // a read: row shift a | w << 16, and the element offset of its plane (and S_w array)
+        __shared__ __align__(16) uint2 s_op[kGatherOps];
+        __shared__ int s_start[1 << NB];
+        const unsigned rowlen = (unsigned)p.rs;
+        const unsigned warray = WMODE ? (unsigned)(p.nodes / n1) * rowlen : 0u; // one S_w
+        const bool ball = TK > 1 || p.dims == 3;
+        const int j0 = j < P ? j - P + n1 : j - P, k0 = ball ? (k < P ? k - P + n1 : k - P) : 0;
+        const longlong2 *base = reinterpret_cast<const longlong2 *>(p.sx) + (live ? i : 0) + (WMODE ? 0 : P + 1);
+        const int nops = p.nops;
+        if (tid < (1 << NB)) s_start[tid] = p.op_end[tid];
+        for (int c0 = 0; c0 < nops; c0 += kGatherOps) {
+            const int n = min(kGatherOps, nops - c0);
+            if (c0) __syncthreads();
+            for (int q = tid; q < n; q += kGatherThreads) {
+                const int4 op = __ldg(p.ops + c0 + q); // (a, z, w, 0)
+                const int kk = k0 + op.y;
+                const unsigned kw = ball ? (unsigned)(kk >= n1 ? kk - n1 : kk) : 0u;
+                s_op[q] = make_uint2((unsigned)op.x | (unsigned)op.z << 16, kw * (unsigned)n1 * rowlen + (unsigned)op.z * warray);
+            }
+            __syncthreads();
+            if (live) gather_classes<1, NB, WMODE>(s_start, c0, n, s_op, base, j0, n1, rowlen, W);
+        }
+    }
     i128 ps = 0, pc = 0;
     bool ok = true;
-    if (n < nodes) {
-        const int i = (int)(n % N1), j = (int)((n / N1) % N1), k = p.dims == 3 ? (int)(n / (N1 * N1)) : 0;
-        const int n1 = (int)N1;
-        uint64_t w0 = 0, w1 = 0;
-        if (STAGE > 0) {
-            const longlong2 *__restrict__ E =
-                reinterpret_cast<const longlong2 *>(p.sx) + (WMODE ? (int64_t)i : (int64_t)(i + p.P + 1));
-            const int nch = p.nchords;
-#pragma unroll 4
-            for (int c = 0; c < nch; ++c) {
-                const int4 ch = __ldg(p.chords + c); // (dy, dz, w, 0)
-                int jj = j + ch.x, kk = k + ch.y;
-                jj += jj < 0 ? n1 : 0;
-                jj -= jj >= n1 ? n1 : 0;
-                kk += kk < 0 ? n1 : 0;
-                kk -= kk >= n1 ? n1 : 0;
-                if (WMODE) {
-                    const longlong2 v = __ldg(E + (int64_t)ch.z * nodes + (int64_t)(kk * n1 + jj) * N1);
-                    w0 += (uint64_t)v.x;
-                    w1 += (uint64_t)v.y;
-                } else {
-                    const longlong2 *r = E + (int64_t)(kk * n1 + jj) * p.rs;
-                    const longlong2 b = __ldg(r + ch.z), a = __ldg(r - ch.z - 1);
-                    w0 += (uint64_t)b.x - (uint64_t)a.x;
-                    w1 += (uint64_t)b.y - (uint64_t)a.y;
-                }
+    if (live) {
+#pragma unroll 1
+        for (int kk = 0; kk < TK; ++kk) {
+            if (TK > 1 && k + kk >= n1) break;
+            const int64_t node = ((int64_t)(k + kk) * n1 + j) * n1 + i;
+#pragma unroll
+            for (int u = 0; u < TJ; ++u) {
+                if (u && j + 1 >= n1) break;
+                const int64_t w0 = (int64_t)(kk ? W[NB - TJ + u][0] : W[u][0]), w1 = (int64_t)(kk ? W[NB - TJ + u][1] : W[u][1]);
+                if (STAGE == 5) lattice_write_coupling<M>(p, node + u * n1, w0, w1);
+                else lattice_node<M, STAGE>(p, node + u * n1, w0, w1, h, ok, ps, pc);
             }
         }
-        lattice_node<M, STAGE>(p, n, (int64_t)w0, (int64_t)w1, h, ok, ps, pc);
     }
     if (!ok) raise_error(p.err, ERR_RANGE);
-    if (STAGE == 0 || STAGE == 4) lattice_record_order(p, ps, pc, blockIdx.x, gridDim.x, p.done_ctr);
+    if (STAGE == 0 || STAGE == 4) { // the order parameter's partials
+        const unsigned bid = blockIdx.y * gridDim.x + blockIdx.x, nblk = gridDim.x * gridDim.y;
+        if (nblk <= kOrderInline) { // the last CTA adds them up
+            lattice_record_order(p, ps, pc, bid, nblk, p.done_ctr);
+            return;
+        }
+        cta_sum_pair(ps, pc); // lattice_order_kernel adds them up
+        if (tid == 0) {
+            st_i128(p.partial + 2 * (int64_t)bid, ps);
+            st_i128(p.partial + 2 * (int64_t)bid + 1, pc);
+        }
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -1013,16 +1233,37 @@ static dim3 tile_grid(int64_t N1)
     return dim3((unsigned)((N1 + BI - 1) / BI), (unsigned)N1, 1);
 }
 
-static unsigned gather_grid(const LatticePlan &p)
+// Nodes per thread of the gather: 4 (rows j, j + 1 of planes k, k + 1) or 2 (rows j,
+// j + 1) where the lattice still fills the chip with so few threads.  RK4 step of a
+// ball with P = 4, in us, by nodes per thread 4 / 2 / 1: N1 = 40 79 / 59 / 50, 50
+// 90 / 71 / -, 64 106 / 97, 72 121 / 173, 100 275 / 327.
+int lattice_gather_nodes(int topo, int64_t N1)
 {
-    return (unsigned)((p.nodes + kGatherThreads - 1) / kGatherThreads);
+    if (topo == 3) return N1 >= 400 ? 2 : 1;
+    return N1 >= 72 ? 4 : N1 >= 48 ? 2 : 1;
+}
+
+// Ball and disk gather: CTAs over (padded column, row or row pair), times planes or
+// pairs of them.
+static dim3 gather_grid(int topo, int64_t N1)
+{
+    const int64_t nb = lattice_gather_nodes(topo, N1), tj = nb > 1 ? 2 : 1, tk = nb > 2 ? 2 : 1;
+    const int64_t n = (N1 + 7) / 8 * 8 * ((N1 + tj - 1) / tj);
+    return dim3((unsigned)((n + kGatherThreads - 1) / kGatherThreads), topo == 3 ? 1u : (unsigned)((N1 + tk - 1) / tk), 1);
+}
+
+// Row stride of sx in (sin, cos) pairs: window arrays have rows padded to 8 pairs,
+// row prefixes their extension.
+int64_t lattice_row_stride(int64_t N1, int64_t P, bool wmode)
+{
+    return wmode ? (N1 + 7) / 8 * 8 : N1 + 2 * P + 1;
 }
 
 int64_t lattice_sx_elems(int topo, int64_t N1, int64_t P, bool wmode)
 {
     if (topo == 1) return lattice_sxy_elems(N1); // both layouts of the x pass's output
     const int64_t rows = topo == 3 ? N1 : N1 * N1;
-    return wmode ? 2 * (P + 1) * rows * N1 : 2 * rows * (N1 + 2 * P + 1);
+    return 2 * (wmode ? P + 1 : 1) * rows * lattice_row_stride(N1, P, wmode);
 }
 
 int64_t lattice_sxy_elems(int64_t N1)
@@ -1034,7 +1275,7 @@ int64_t lattice_sxy_elems(int64_t N1)
 int64_t lattice_partial_blocks(int topo, int64_t N1)
 {
     const int64_t a = lattice_order_blocks(topo, N1);
-    if (topo != 1) return a;
+    if (topo != 1) return a + kOrderCtas;
     // the fused node pass (one row per warp) and the order kernel's second level
     const int64_t b = (N1 * N1 + nodex_warps(N1) - 1) / nodex_warps(N1) + kOrderCtas;
     return a > b ? a : b;
@@ -1043,8 +1284,8 @@ int64_t lattice_partial_blocks(int topo, int64_t N1)
 int64_t lattice_order_blocks(int topo, int64_t N1)
 {
     if (topo == 1) return ((N1 + kColThreads - 1) / kColThreads) * N1 * col_segments(N1);
-    const int64_t nodes = topo == 3 ? N1 * N1 : N1 * N1 * N1;
-    return (nodes + kGatherThreads - 1) / kGatherThreads;
+    const dim3 g = gather_grid(topo, N1);
+    return (int64_t)g.x * g.y;
 }
 
 cudaError_t lattice_configure()
@@ -1055,15 +1296,18 @@ cudaError_t lattice_configure()
         e = cudaFuncSetAttribute(lattice_x_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)kRowSmemMax);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(lattice_x_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)kRowSmemMax);
-    if (e == cudaSuccess)
         e = cudaFuncSetAttribute(cube_batch_x_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)kRowSmemMax);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(lattice_ext_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRowSmemMax);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(lattice_ext_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRowSmemMax);
     // the largest tile of any edge: the top edge of each tile width
     const int tmax = (int)std::max(std::max(cube_tile_smem(297), cube_tile_smem(594)), cube_tile_smem(1024));
     if (e == cudaSuccess) e = cudaFuncSetAttribute(cube_y_tile_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, tmax);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(cube_zw_tile_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, tmax);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(cube_zw_tile_kernel<-1>, cudaFuncAttributeMaxDynamicSharedMemorySize, tmax);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(cube_zw_tile_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, tmax);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(cube_zw_tile_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, tmax);
 #define SIM_NODEX_ATTR(M, S)                                                                                           \
     if (e == cudaSuccess)                                                                                              \
         e = cudaFuncSetAttribute(cube_nodex_kernel<M, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRowSmemMax);
@@ -1131,12 +1375,30 @@ static size_t x_smem(const LatticePlan &p)
 
 static cudaError_t launch_x(const LatticePlan &p, cudaStream_t s)
 {
-    const int w = row_warps(p.N1);
-    if (p.topo == 1) lattice_x_kernel<0><<<x_grid(p), 32 * w, x_smem(p), s>>>(p);
-    else if (p.wmode) lattice_x_kernel<2><<<x_grid(p), 32 * w, x_smem(p), s>>>(p);
+    const int w = row_warps(p.N1), we = p.topo == 1 ? 0 : ext_warps(p.N1, p.P);
+    if (we > 0) {
+        const unsigned grid = (unsigned)((p.nodes / p.N1 + we - 1) / we);
+        const size_t smem = sizeof(longlong2) * (size_t)we * (size_t)(p.N1 + 2 * p.P + 1);
+        if (p.wmode) lattice_ext_kernel<2><<<grid, 32 * we, smem, s>>>(p);
+        else lattice_ext_kernel<1><<<grid, 32 * we, smem, s>>>(p);
+    } else if (p.topo == 1) lattice_x_kernel<0><<<x_grid(p), 32 * w, x_smem(p), s>>>(p);
     else lattice_x_kernel<1><<<x_grid(p), 32 * w, x_smem(p), s>>>(p);
     const cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) kernel_mark(s, 0);
+    return e;
+}
+
+// The cube's y and z-window passes: every node's coupling term (KM = -1) or slope
+// of model KM from the x sums.
+template <int KM>
+static cudaError_t launch_cube_windows(const LatticePlan &p, cudaStream_t s)
+{
+    cube_y_tile_kernel<<<tile_grid(p.N1), kTileThreads, cube_tile_smem(p.N1), s>>>(p);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    kernel_mark(s, 1);
+    cube_zw_tile_kernel<KM><<<tile_grid(p.N1), kZThreads, cube_tile_smem(p.N1), s>>>(p);
+    if ((e = cudaGetLastError()) == cudaSuccess) kernel_mark(s, 3);
     return e;
 }
 
@@ -1146,15 +1408,8 @@ static cudaError_t launch_x(const LatticePlan &p, cudaStream_t s)
 template <int M, int STAGE>
 static cudaError_t launch_cube_stage(const LatticePlan &p, double dt, cudaStream_t s)
 {
-    cudaError_t e = cudaSuccess;
-    if (STAGE > 0) {
-        cube_y_tile_kernel<<<tile_grid(p.N1), kTileThreads, cube_tile_smem(p.N1), s>>>(p);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        kernel_mark(s, 1);
-        cube_zw_tile_kernel<<<tile_grid(p.N1), kZThreads, cube_tile_smem(p.N1), s>>>(p);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        kernel_mark(s, 3);
-    }
+    cudaError_t e = STAGE > 0 ? launch_cube_windows<-1>(p, s) : cudaSuccess;
+    if (e != cudaSuccess) return e;
     const int w = nodex_warps(p.N1);
     const int64_t rows = p.nodes / p.N1;
     const unsigned nblk = (unsigned)((rows + w - 1) / w);
@@ -1163,7 +1418,30 @@ static cudaError_t launch_cube_stage(const LatticePlan &p, double dt, cudaStream
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     kernel_mark(s, 2);
     if (STAGE == 0 || STAGE == 4) {
-        lattice_order_kernel<<<kOrderCtas, kOrderThreads, 0, s>>>(p, nblk);
+        lattice_order_kernel<<<order_grid(nblk), kOrderThreads, 0, s>>>(p, nblk);
+        if ((e = cudaGetLastError()) == cudaSuccess) kernel_mark(s, 0);
+    }
+    return e;
+}
+
+template <int M, int STAGE>
+static cudaError_t launch_gather(const LatticePlan &p, double dt, cudaStream_t s)
+{
+    const dim3 grid = gather_grid(p.topo, p.N1);
+    const StepSize h = step_size(dt);
+    const int nb = lattice_gather_nodes(p.topo, p.N1);
+    const bool wm = STAGE > 0 && p.wmode;
+    if (nb == 4 && wm) lattice_gather_kernel<M, STAGE, true, 4><<<grid, kGatherThreads, 0, s>>>(p, h);
+    else if (nb == 4) lattice_gather_kernel<M, STAGE, false, 4><<<grid, kGatherThreads, 0, s>>>(p, h);
+    else if (nb == 2 && wm) lattice_gather_kernel<M, STAGE, true, 2><<<grid, kGatherThreads, 0, s>>>(p, h);
+    else if (nb == 2) lattice_gather_kernel<M, STAGE, false, 2><<<grid, kGatherThreads, 0, s>>>(p, h);
+    else if (wm) lattice_gather_kernel<M, STAGE, true, 1><<<grid, kGatherThreads, 0, s>>>(p, h);
+    else lattice_gather_kernel<M, STAGE, false, 1><<<grid, kGatherThreads, 0, s>>>(p, h);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    kernel_mark(s, 2);
+    if ((STAGE == 0 || STAGE == 4) && grid.x * grid.y > kOrderInline) {
+        lattice_order_kernel<<<order_grid(grid.x * grid.y), kOrderThreads, 0, s>>>(p, grid.x * grid.y);
         if ((e = cudaGetLastError()) == cudaSuccess) kernel_mark(s, 0);
     }
     return e;
@@ -1174,13 +1452,8 @@ static cudaError_t launch_cube_stage(const LatticePlan &p, double dt, cudaStream
 template <int M, int STAGE>
 static cudaError_t launch_gather_stage(const LatticePlan &p, double dt, cudaStream_t s)
 {
-    cudaError_t e = STAGE > 0 ? launch_x(p, s) : cudaSuccess;
-    if (e != cudaSuccess) return e;
-    if (p.wmode && STAGE > 0)
-        lattice_gather_kernel<M, STAGE, true><<<gather_grid(p), kGatherThreads, 0, s>>>(p, step_size(dt));
-    else lattice_gather_kernel<M, STAGE, false><<<gather_grid(p), kGatherThreads, 0, s>>>(p, step_size(dt));
-    if ((e = cudaGetLastError()) == cudaSuccess && STAGE > 0) kernel_mark(s, 2);
-    return e;
+    const cudaError_t e = STAGE > 0 ? launch_x(p, s) : cudaSuccess;
+    return e != cudaSuccess ? e : launch_gather<M, STAGE>(p, dt, s);
 }
 
 template <int M>
@@ -1215,14 +1488,14 @@ cudaError_t lattice_prologue(const LatticePlan &p, cudaStream_t s)
     return launch_any(0, p, 0.0, s);
 }
 
-// k = f(y) into acc (stage 1 with dt = 0, from the stored (sin, cos) of y).
+// k = f(y) into acc, from the stored (sin, cos) of y (y may be a stage input that
+// has no x sums yet).
 cudaError_t lattice_rhs(const LatticePlan &p, cudaStream_t s)
 {
-    if (p.topo == 1) {
-        const cudaError_t e = launch_x(p, s); // y may be a stage input that has no x sums yet
-        if (e != cudaSuccess) return e;
-    }
-    return launch_any(1, p, 0.0, s);
+    const cudaError_t e = launch_x(p, s);
+    if (e != cudaSuccess) return e;
+    if (p.topo == 1) return p.model == 3 ? launch_cube_windows<3>(p, s) : launch_cube_windows<0>(p, s);
+    return p.model == 3 ? launch_gather<3, 5>(p, 0.0, s) : launch_gather<0, 5>(p, 0.0, s);
 }
 
 cudaError_t lattice_step(const LatticePlan &p, double dt, cudaStream_t s)

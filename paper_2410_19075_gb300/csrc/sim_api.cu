@@ -90,6 +90,45 @@ std::vector<int4> chords_of(int topo, int64_t P, int64_t *count)
     return out;
 }
 
+// The reads of the windows of a block of nb nodes (4: rows j, j + 1 of planes k, k + 1;
+// 2: rows j, j + 1; 1) of a ball or disk together, as (row shift from row j - P, plane
+// shift from plane k - P, half-width, 0): see LatticePlan::ops.
+std::vector<int4> gather_ops(int topo, int64_t P, int nb, LatticePlan &p)
+{
+    int64_t count = 0;
+    const int tk = nb > 2 ? 2 : 1, tj = nb > 1 ? 2 : 1, rows = 2 * (int)P + 1, np = topo == SIM_BALL3D ? rows : 1;
+    std::vector<int> w((size_t)np * rows, -1); // half-width at (plane shift, dy + P)
+    for (const int4 &c : chords_of(topo, P, &count))
+        w[(size_t)(np > 1 ? c.y + (int)P : 0) * rows + c.x + (int)P] = c.z;
+    std::vector<std::vector<int4>> by_set(16);
+    for (int z = 0; z < np + tk - 1; ++z)
+        for (int a = 0; a < rows + tj - 1; ++a) {
+            int wb[4] = {-1, -1, -1, -1}; // the half-width node b of the block reads there
+            for (int b = 0; b < nb; ++b) {
+                const int zz = z - (b >> 1), aa = a - (b & 1); // nb <= 4: bit 0 the row, bit 1 the plane
+                if (zz >= 0 && zz < np && aa >= 0 && aa < rows) wb[b] = w[(size_t)zz * rows + aa];
+            }
+            for (int b = 0; b < nb; ++b) {
+                if (wb[b] < 0) continue;
+                int set = 0;
+                bool first = true;
+                for (int c = 0; c < nb; ++c)
+                    if (wb[c] == wb[b]) {
+                        set |= 1 << c;
+                        first = first && c >= b;
+                    }
+                if (first) by_set[set].push_back(make_int4(a, z, wb[b], 0));
+            }
+        }
+    std::vector<int4> out;
+    for (int m = 0; m < 16; ++m) {
+        out.insert(out.end(), by_set[m].begin(), by_set[m].end());
+        p.op_end[m] = (int)out.size();
+    }
+    p.nops = (int)out.size();
+    return out;
+}
+
 int64_t window_of(int topo, int64_t R)
 {
     if (topo == SIM_RING) return 2 * R + 1;
@@ -156,16 +195,18 @@ struct Layout {
     size_t f, xs, sx, sxy, cpl, partial, chords, ctrs, obs, tabs;
 };
 
-// Ball and disk: one x-window array per chord half-width (one load per chord
-// instead of two) for radii of 5 and more, when the arrays fit the budget.
-// Measured on the 100^3 ball: 8% faster at P = 6 and 19% on 200^3 at P = 8;
-// at P <= 4 the extra x-pass writes cost as much as the loads they save.
+// Ball: one x-window array per chord half-width (one load per read instead of two)
+// for radii of 5 and more, when the arrays fit the budget.  Measured per RK4 step,
+// window arrays against row prefixes: 100^3 P = 5 380 / 376 us, P = 6 441 / 479,
+// P = 8 618 / 711; 150^3 P = 5 1106 / 1201, P = 6 1328 / 1500; 200^3 P = 8 4547 / 4989.
+// At P <= 4 the extra x-pass writes cost more than the loads they save, and so they
+// do on disks at every radius (1000^2 P = 30: 654 / 356 us; 2500^2 P = 60: 8398 /
+// 3611), whose P + 1 arrays serve only 2P + 1 reads per node.
 constexpr int64_t kWindowMinRadius = 5;
 bool lattice_wmode(int topo, int64_t N, int64_t R, unsigned flags)
 {
-    if (topo != SIM_BALL3D && topo != SIM_DISK2D) return false;
-    if ((flags & SIM_FLAG_LOW_MEMORY) || R < kWindowMinRadius) return false;
-    return (R + 1) * 16 * nodes_of(topo, N) <= kLatticeWindowBudget;
+    if (topo != SIM_BALL3D || (flags & SIM_FLAG_LOW_MEMORY) || R < kWindowMinRadius) return false;
+    return 8 * lattice_sx_elems(topo, N, R, true) <= kLatticeWindowBudget;
 }
 
 Layout layout_of(int model, int topo, int64_t N, int64_t R, unsigned flags = 0)
@@ -210,7 +251,7 @@ Layout layout_of(int model, int topo, int64_t N, int64_t R, unsigned flags = 0)
         L.sxy = take(topo == SIM_CUBE3D ? sizeof(int64_t) * lattice_sxy_elems(N) : 0);
         L.cpl = take(topo == SIM_CUBE3D ? sizeof(double) * n : 0);
         L.partial = take(sizeof(i128) * 2 * nblk);
-        L.chords = take(topo == SIM_CUBE3D ? 0 : sizeof(int4) * (2 * R + 1) * (2 * R + 1));
+        L.chords = take(topo == SIM_CUBE3D ? 0 : sizeof(int4) * 4 * (2 * R + 2) * (topo == SIM_DISK2D ? 1 : 2 * R + 2));
     }
     L.ctrs = take(64);
     L.obs = take(sizeof(double) * kObsCap);
@@ -254,7 +295,7 @@ struct sim_handle {
     Layout L;
     RingPlan ring{};
     LatticePlan lat{};
-    std::vector<int4> chords; // host copy (the upload reads it asynchronously)
+    std::vector<int4> gather_ops; // host copy (the upload reads it asynchronously)
     unsigned *err = nullptr;
     unsigned long long *obs_ctr = nullptr;
     double *obs = nullptr;
@@ -617,8 +658,8 @@ static int create_impl(sim_t *out, int model, int topology, int64_t N, int64_t r
         p.f = reinterpret_cast<int64_t *>(b + L.f);
         p.xs = reinterpret_cast<double *>(b + L.xs);
         p.sx = reinterpret_cast<int64_t *>(b + L.sx);
-        p.rs = N + 2 * radius + 1;
         p.wmode = lattice_wmode(topology, N, radius, flags) ? 1 : 0;
+        p.rs = lattice_row_stride(N, radius, p.wmode != 0);
         p.sxy = reinterpret_cast<int64_t *>(b + L.sxy);
         p.cpl = reinterpret_cast<double *>(b + L.cpl);
         p.partial = reinterpret_cast<i128 *>(b + L.partial);
@@ -628,16 +669,12 @@ static int create_impl(sim_t *out, int model, int topology, int64_t N, int64_t r
         p.obs = h->obs;
         p.obs_cap = kObsCap;
         p.obs_ctr = h->obs_ctr;
-        p.chords = nullptr;
-        p.nchords = 0;
+        p.ops = nullptr;
         if (topology != SIM_CUBE3D) {
-            int64_t cnt = 0;
-            const std::vector<int4> ch = chords_of(topology, radius, &cnt);
-            h->chords = ch;
-            p.chords = reinterpret_cast<const int4 *>(b + L.chords);
-            p.nchords = (int)ch.size();
-            e = cudaMemcpyAsync(b + L.chords, h->chords.data(), sizeof(int4) * ch.size(), cudaMemcpyHostToDevice,
-                                h->stream);
+            h->gather_ops = gather_ops(topology, radius, lattice_gather_nodes(topology, N), p);
+            p.ops = reinterpret_cast<const int4 *>(b + L.chords);
+            e = cudaMemcpyAsync(b + L.chords, h->gather_ops.data(), sizeof(int4) * h->gather_ops.size(),
+                                cudaMemcpyHostToDevice, h->stream);
         }
         static std::once_flag lat_once;
         static cudaError_t lat_err = cudaSuccess;
@@ -928,7 +965,7 @@ int sim_step_timed(sim_t h, int64_t n_steps, double dt, double *ms_by_kind, int6
             h->pfx = 2;
         }
     }
-    const int per_step = use_cluster(h) ? 1 : h->topo == SIM_CUBE3D ? 13 : is_lattice(h->topo) ? 8 : 4;
+    const int per_step = use_cluster(h) ? 1 : h->topo == SIM_CUBE3D ? 13 : is_lattice(h->topo) ? 9 : 4;
     const int cap = (int)(use_cluster(h) ? 1 : per_step * n_steps);
     std::vector<cudaEvent_t> ev(cap + 1, nullptr);
     std::vector<unsigned char> kind(cap, 0);
