@@ -122,10 +122,10 @@ __global__ void __launch_bounds__(kRingThreads, DpMinBlocks<M>::value)
                     acc = c_dp_a[1][0] * k[v];
                 } else {
                     Q.k[DS][q] = k[v];
-                    acc = c_dp_a[DS][0] * k1[q];
+                    acc = dp_sum2(c_dp_a[DS][0], k1[q], c_dp_a[DS][1], DS == 2 ? k[v] : Q.k[2][q]);
 #pragma unroll
-                    for (int j = 1; j < DS - 1; ++j) acc += c_dp_a[DS][j] * Q.k[j + 1][q];
-                    acc += c_dp_a[DS][DS - 1] * k[v];
+                    for (int j = 2; j < DS - 1; ++j) acc = fma(c_dp_a[DS][j], Q.k[j + 1][q], acc);
+                    if (DS > 2) acc = fma(c_dp_a[DS][DS - 1], k[v], acc);
                 }
                 xn[v] = y[q] + h * acc;
                 if (DS == 6) y5[q] = xn[v];
@@ -141,10 +141,10 @@ __global__ void __launch_bounds__(kRingThreads, DpMinBlocks<M>::value)
             for (int v = 0; v < D; ++v) {
                 const int64_t q = v * N + i;
                 Q.k[cur ^ 1][q] = k[v];
-                double e = c_dp_e[0] * k1[q];
+                double e = dp_sum2(c_dp_e[0], k1[q], c_dp_e[2], Q.k[3][q]);
 #pragma unroll
-                for (int j = 2; j <= 5; ++j) e += c_dp_e[j] * Q.k[j + 1][q];
-                e += c_dp_e[6] * k[v];
+                for (int j = 3; j <= 5; ++j) e = fma(c_dp_e[j], Q.k[j + 1][q], e);
+                e = fma(c_dp_e[6], k[v], e);
                 e *= h;
                 const double sc = atol + rtol * fmax(fabs(y[q]), fabs(y5[q]));
                 const double r = e / sc;
@@ -185,8 +185,7 @@ __global__ void __launch_bounds__(kRingThreads, DpMinBlocks<M>::value)
             double th = (to - t) / h;
             th = th > 1.0 ? 1.0 : th;
             const double a0 = y[i], a1 = y5[i], f0 = k1[i], f1 = k[0];
-            const double ph = (1.0 - th) * a0 + th * a1 +
-                              th * (th - 1.0) * ((1.0 - 2.0 * th) * (a1 - a0) + (th - 1.0) * h * f0 + th * h * f1);
+            const double ph = dp_hermite(th, h, a0, a1, f0, f1);
             int64_t s62, c62;
             fixed_sincos(ph, P.mp.tab, s62, c62, ok);
             ss = q62_to(s62, P.F);

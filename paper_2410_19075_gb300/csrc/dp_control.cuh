@@ -21,6 +21,18 @@ __constant__ double c_dp_a[7][6] = {
 __constant__ double c_dp_e[7] = {71.0 / 57600.0, 0.0, -71.0 / 16695.0, 71.0 / 1920.0, -17253.0 / 339200.0,
                                  22.0 / 525.0, -1.0 / 40.0};
 
+// The roundings of the tableau sums, fixed so that every kernel gives the same
+// bits: the first two products in one FMA, every further one in an FMA of its own.
+__device__ __forceinline__ double dp_sum2(double a, double x, double b, double y) { return fma(a, x, __dmul_rn(b, y)); }
+
+// Hermite interpolant of the phase at t + th h from the step's ends (a0, a1) and slopes (f0, f1).
+__device__ __forceinline__ double dp_hermite(double th, double h, double a0, double a1, double f0, double f1)
+{
+    const double u = th - 1.0, p = dp_sum2(-u, a0, th, a1);
+    const double q = fma(__dmul_rn(th, h), f1, dp_sum2(fma(-2.0, th, 1.0), a1 - a0, __dmul_rn(u, h), f0));
+    return fma(__dmul_rn(th, u), q, p);
+}
+
 // Step-size controller: safety factor, smallest and largest factor per step.
 constexpr double kDpSafe = 0.9, kDpFacMin = 0.2, kDpFacMax = 10.0;
 

@@ -24,13 +24,12 @@
 #include <cooperative_groups.h>
 
 #include "internal.h"
-#include "ring_parts.cuh"
+#include "ring_slices.cuh"
 
 namespace cg = cooperative_groups;
 
 namespace simk {
 
-constexpr int kClusterMaxCtas = 16;
 constexpr int kClusterSlice = 512; // nodes of a CTA at most (two warps' worth of int64 headroom: 512 2^54 = 2^63)
 constexpr int kClusterThreadsMax = kClusterSlice + 32;
 
@@ -43,53 +42,6 @@ __host__ __device__ constexpr size_t cluster_smem_bytes(int per)
     return sizeof(int64_t) * NQ * (size_t)(2 * per); // lam, two buffers
 }
 
-// Exact offsets of the cluster's slices from their totals, by one warp: lane r
-// holds the prefix in front of slice r as hi 2^sh + lo (ex_*), every lane the
-// ring's total (tot_*).
-template <int NQ> struct SliceOffsets {
-    int64_t ex_hi[NQ], tot_hi[NQ];
-    int ex_lo[NQ], tot_lo[NQ];
-};
-template <int NQ>
-__device__ __forceinline__ void slice_offsets(const int64_t (*tot)[NQ], int CL, int sh, SliceOffsets<NQ> &o)
-{
-    const int lane = threadIdx.x & 31, mask = (1 << sh) - 1;
-    int64_t t[NQ];
-#pragma unroll
-    for (int c = 0; c < NQ; ++c) t[c] = lane < CL ? tot[lane][c] : 0;
-#pragma unroll
-    for (int c = 0; c < NQ; ++c) {
-        const int64_t h = t[c] >> sh;
-        const int l = (int)t[c] & mask;
-        int64_t hi = h;
-        int lo = l;
-#pragma unroll
-        for (int d = 1; d < kClusterMaxCtas; d <<= 1) {
-            const int64_t h2 = __shfl_up_sync(0xffffffffu, hi, d);
-            const int l2 = __shfl_up_sync(0xffffffffu, lo, d);
-            if (lane >= d) {
-                hi += h2;
-                lo += l2;
-            }
-        }
-        o.ex_hi[c] = hi - h;
-        o.ex_lo[c] = lo - l;
-        o.tot_hi[c] = __shfl_sync(0xffffffffu, hi, kClusterMaxCtas - 1);
-        o.tot_lo[c] = __shfl_sync(0xffffffffu, lo, kClusterMaxCtas - 1);
-    }
-}
-
-// The prefix in front of slice r on copy q of the ring (-1, 0, 1).
-template <int NQ>
-__device__ __forceinline__ void slice_base(const SliceOffsets<NQ> &o, int r, int q, int64_t (&hi)[NQ], int (&lo)[NQ])
-{
-#pragma unroll
-    for (int c = 0; c < NQ; ++c) {
-        hi[c] = __shfl_sync(0xffffffffu, o.ex_hi[c], r) + q * o.tot_hi[c];
-        lo[c] = __shfl_sync(0xffffffffu, o.ex_lo[c], r) + q * o.tot_lo[c];
-    }
-}
-
 template <int M>
 __global__ void __launch_bounds__(kClusterThreadsMax, 1)
     ring_cluster_kernel(const RingPlan P, const StepSize h, int per, int64_t n_steps)
@@ -100,7 +52,7 @@ __global__ void __launch_bounds__(kClusterThreadsMax, 1)
     cg::cluster_group cluster = cg::this_cluster();
     const int rank = (int)cluster.block_rank(), CL = (int)cluster.num_blocks();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = (int)(blockDim.x >> 5) - 1; // node warps
-    const int N = (int)P.N, R = (int)P.R, sh = P.mp.ksh, mask = (1 << sh) - 1;
+    const int N = (int)P.N, R = (int)P.R, sh = P.mp.ksh;
     const int i = rank * per + tid;
     const bool recorder = warp == nwarps, live = !recorder && tid < per && i < N;
 
@@ -200,12 +152,7 @@ __global__ void __launch_bounds__(kClusterThreadsMax, 1)
                 slice_base<NQ>(o, rk[0], qk[0], hb, lob);
                 slice_base<NQ>(o, rk[1], qk[1], ha, loa);
                 if (live) {
-#pragma unroll
-                    for (int c = 0; c < NQ; ++c) {
-                        const int64_t own = Mo::OWN_OUT && !P.mp.include_self ? qn[c] : 0;
-                        const int lo = lob[c] - loa[c] + ((int)lb[c] & mask) - ((int)la[c] & mask) - ((int)own & mask);
-                        S[c] = hb[c] - ha[c] + (lb[c] >> sh) - (la[c] >> sh) - (own >> sh) + (int64_t)(lo >> sh);
-                    }
+                    slice_sums<M, NQ>(P.mp, lb, la, hb, ha, lob, loa, qn, S);
                     double k[D], xn[D];
                     Mo::rhs_ring(P.mp, qn, S, xs, iext, k);
 #pragma unroll
@@ -272,6 +219,7 @@ __global__ void __launch_bounds__(kClusterThreadsMax, 1)
 }
 
 static int g_max_cluster = 8; // 16 when the device can co-schedule it (set by configure)
+int cluster_max_ctas() { return g_max_cluster; }
 
 int cluster_size_for(int model, int64_t N)
 {

@@ -508,6 +508,14 @@ void simk::lattice_rotation(LatticePlan &p, double alpha)
     p.mp.c[5] = std::ldexp(p.model == SIM_KS ? p.mp.c[1] : p.mp.c[0], -(p.F - 2));
 }
 
+static cudaError_t ensure_cluster_configured()
+{
+    static std::once_flag once;
+    static cudaError_t err = cudaSuccess;
+    std::call_once(once, [] { err = ring_cluster_configure(); });
+    return err;
+}
+
 extern "C" {
 
 size_t sim_workspace_bytes(int model, int topology, int64_t N, int64_t radius)
@@ -637,10 +645,7 @@ static int create_impl(sim_t *out, int model, int topology, int64_t N, int64_t r
             p.flat_ctr = ctrs + 3;
         }
         if (N <= kClusterMaxNodes && !(flags & SIM_FLAG_STREAMING)) {
-            static std::once_flag cl_once;
-            static cudaError_t cl_err = cudaSuccess;
-            std::call_once(cl_once, [] { cl_err = ring_cluster_configure(); });
-            if (cl_err != cudaSuccess) h->flags |= SIM_FLAG_STREAMING; // fall back to the streaming kernels
+            if (ensure_cluster_configured() != cudaSuccess) h->flags |= SIM_FLAG_STREAMING; // fall back to the streaming kernels
         }
     } else {
         LatticePlan &p = h->lat;
@@ -1503,6 +1508,7 @@ static_assert(kDpStatusSteps == SIM_ESTEPS && kDpStatusSmall == SIM_ESMALL, "sta
 namespace {
 
 constexpr int kDpGraphAttempts = 16; // attempted steps per captured graph
+constexpr int kDpClusterAttempts = 256; // attempted steps per launch of the cluster-resident kernel
 constexpr int kDpMaxOutPerStep = 8;  // the step is capped at this many output intervals
 
 int64_t dp_n_out(double t0, double t_end, double out_dt)
@@ -1662,10 +1668,20 @@ int dp_run(const std::vector<sim_t> &mem, const sim_dp5_opts *opts, sim_dp5_stat
     // Device tables of the run: plans, work items per model group, control
     // words, the members' error words and the counter of unfinished members.
     std::vector<std::vector<int>> by_model(4);
+    std::map<std::pair<int, int>, std::vector<int>> resident; // (model, CTAs) -> small rings, each run in one cluster
     std::vector<int> lat_members;
+    int n_rings = 0;
+    for (int i = 0; i < n; ++i) n_rings += mem[i]->topo == SIM_RING;
+    if (n_rings && ensure_cluster_configured() != cudaSuccess) n_rings = 0; // streaming kernels only
     for (int i = 0; i < n; ++i) {
-        if (mem[i]->topo == SIM_RING) by_model[mem[i]->model].push_back(i);
-        else lat_members.push_back(i);
+        const sim_t h = mem[i];
+        if (h->topo != SIM_RING) {
+            lat_members.push_back(i);
+            continue;
+        }
+        const int cl = n_rings && !(h->flags & SIM_FLAG_STREAMING) ? dp_cluster_size(h->model, h->N, n_rings) : 0;
+        if (cl) resident[{h->model, cl}].push_back(i);
+        else by_model[h->model].push_back(i);
     }
     std::vector<DpPlan> plans;
     std::vector<int> inst_of_item, plan_member;
@@ -1684,6 +1700,17 @@ int dp_run(const std::vector<sim_t> &mem, const sim_dp5_opts *opts, sim_dp5_stat
             sp.n_items += h->ring.nsub;
         }
         spans.push_back(sp);
+    }
+    struct Resident { int model, cl, first_plan, n; int64_t n_max; };
+    std::vector<Resident> clusters;
+    for (const auto &kv : resident) {
+        Resident r{kv.first.first, kv.first.second, (int)plans.size(), (int)kv.second.size(), 0};
+        for (int i : kv.second) {
+            plans.push_back(mem[i]->dp);
+            plan_member.push_back(i);
+            r.n_max = std::max(r.n_max, mem[i]->N);
+        }
+        clusters.push_back(r);
     }
     std::vector<unsigned *> errs(n);
     for (int i = 0; i < n; ++i) errs[i] = mem[i]->err;
@@ -1771,9 +1798,29 @@ int dp_run(const std::vector<sim_t> &mem, const sim_dp5_opts *opts, sim_dp5_stat
         e = ring_prologue(mem[graph_idx[q]]->ring, s); // R(t0)
         if (e == cudaSuccess) e = graph_dp_start(gplans[q], s);
     }
+    auto run_clusters = [&](int first) {
+        for (const Resident &r : clusters)
+            if (e == cudaSuccess)
+                e = dp_cluster_launch(r.model, reinterpret_cast<const DpPlan *>(tb + o_plans) + r.first_plan, r.n, r.cl,
+                                      r.n_max, kDpClusterAttempts, first, s);
+    };
+    run_clusters(1);
     if (e != cudaSuccess) return finish(cuda_fail(e, "Dormand-Prince start"));
+    long long max_att = 0;
+    for (int i = 0; i < n; ++i) max_att = opts[i].max_attempts > max_att ? opts[i].max_attempts : max_att;
+    int h_rem = remaining;
+    const bool only_clusters = groups.empty() && lplans.empty() && gplans.empty();
+    if (only_clusters) { // further launches while a ring has attempts left
+        const long long max_launches = max_att / kDpClusterAttempts + 2;
+        for (long long r = 0; r < max_launches && h_rem > 0; ++r) {
+            if (r) run_clusters(0);
+            if (e == cudaSuccess) e = cudaMemcpyAsync(&h_rem, d_rem, sizeof(int), cudaMemcpyDeviceToHost, s);
+            if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+            if (e != cudaSuccess) return finish(cuda_fail(e, "Dormand-Prince attempts"));
+        }
+    }
     // Attempts in captured graphs until every member is done.
-    if (remaining > 0) {
+    if (remaining > 0 && !only_clusters) {
         e = cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking);
         if (e == cudaSuccess) e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
         if (e != cudaSuccess) return finish(cuda_fail(e, "Dormand-Prince capture"));
@@ -1796,18 +1843,16 @@ int dp_run(const std::vector<sim_t> &mem, const sim_dp5_opts *opts, sim_dp5_stat
         e = cudaGraphInstantiate(&ex, graph, 0);
         cudaGraphDestroy(graph);
         if (e != cudaSuccess) return finish(cuda_fail(e, "cudaGraphInstantiate"));
-        long long max_att = 0;
-        for (int i = 0; i < n; ++i) max_att = opts[i].max_attempts > max_att ? opts[i].max_attempts : max_att;
         const long long max_replays = max_att / kDpGraphAttempts + 2;
-        int h_rem = remaining;
         for (long long r = 0; r < max_replays && h_rem > 0; ++r) {
-            e = cudaGraphLaunch(ex, s);
+            if (r) run_clusters(0);
+            if (e == cudaSuccess) e = cudaGraphLaunch(ex, s);
             if (e == cudaSuccess) e = cudaMemcpyAsync(&h_rem, d_rem, sizeof(int), cudaMemcpyDeviceToHost, s);
             if (e == cudaSuccess) e = cudaStreamSynchronize(s);
             if (e != cudaSuccess) return finish(cuda_fail(e, "Dormand-Prince attempts"));
         }
-        if (h_rem > 0) status = fail(SIM_EDEVICE, "Dormand-Prince run did not finish within its attempt budget");
     }
+    if (h_rem > 0) status = fail(SIM_EDEVICE, "Dormand-Prince run did not finish within its attempt budget");
     // State back in the handles' buffers with the prefix of f(y) for the RK4
     // path, the control words and the OR of the members' error words.
     for (const DpGroup &g : groups)
