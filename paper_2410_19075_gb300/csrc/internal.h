@@ -56,7 +56,8 @@ struct RingPlan {
     // unsigned, and t >> 54 signed) in 32-bit words, exact because no sum of
     // chunks over at most 8192 sub-tiles reaches 2^31; the next kernel's CTAs
     // sum those themselves, so no CTA waits for the last one of its launch.
-    int flat;             // plain stage kernels only (batched members keep the two-level scan)
+    int flat;             // plain stage kernels (batched members keep the two-level scan) and link matrices of
+                          // at most kGraphFlatSubs sub-tiles
     int npt;              // nodes per thread of the stage kernels: 2 (128 threads per sub-tile;
                           // not HH) or 1 (256); set by sim_create and the autotuner
     int64_t *fsub[2];     // NQ * nsub each: sub-tile totals (same parity as lam)
@@ -64,6 +65,8 @@ struct RingPlan {
     unsigned long long *flat_ctr; // arrival counter of the one-pass kernels that record or count steps
 };
 
+constexpr int kGraphFlatSubs = 512; // link matrices: sub-tiles up to which every CTA scans all totals (N <= 131072);
+                                    // 1024 cost smaller networks 8% and gained 1% at 200000 nodes
 constexpr int kFlatMaxGroups = 128; // lanes sum four groups each; 8192 sub-tiles keep chunk sums below 2^31
 
 // Ring members of one model in a batch: device tables of the batched launch.
@@ -164,6 +167,7 @@ int cluster_max_ctas();               // 8 or 16
 int cluster_size_for(int model, int64_t N); // CTAs of the cluster for a ring of N nodes (0: not eligible)
 cudaError_t ring_cluster_steps(const RingPlan &p, double dt, int64_t n_steps, cudaStream_t s);
 
+cudaError_t ring_clear_slot(const RingPlan &p, int slot, cudaStream_t s); // zero a one-pass accumulator slot
 // Ring: stage 1 only with dt = 0, so acc receives f(y) and y is untouched.
 cudaError_t ring_rhs(const RingPlan &p, cudaStream_t s);
 // Ring: one RK4 step, 4 fused stage kernels.

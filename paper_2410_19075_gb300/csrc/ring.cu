@@ -317,11 +317,16 @@ cudaError_t ring_prologue(const RingPlan &p, cudaStream_t s)
     return launch_any(0, p, 0.0, s);
 }
 
+cudaError_t ring_clear_slot(const RingPlan &p, int slot, cudaStream_t s)
+{
+    return cudaMemsetAsync(p.facc[slot], 0, flat_slot_bytes(p), s);
+}
+
 cudaError_t ring_rhs(const RingPlan &p, cudaStream_t s)
 {
     cudaError_t e = launch_any(1, p, 0.0, s);
     // a stage 1 on its own leaves slot 1 filled; the next RK4 step adds into it
-    if (e == cudaSuccess && p.flat) e = cudaMemsetAsync(p.facc[1], 0, flat_slot_bytes(p), s);
+    if (e == cudaSuccess && p.flat) e = ring_clear_slot(p, 1, s);
     return e;
 }
 

@@ -222,11 +222,8 @@ __global__ void __launch_bounds__(DpShape<M>::NT, 2)
         SliceOffsets<NQ> o;
         offsets(o);
         if (KURAMOTO && rank == 0 && tid == 0 && P.obs) {
-            const double S = fixed_to_double(((i128)o.tot_hi[0] << sh) + o.tot_lo[0], P.F);
-            const double C = fixed_to_double(((i128)o.tot_hi[NQ - 1] << sh) + o.tot_lo[NQ - 1], P.F);
-            const unsigned long long n = *P.obs_ctr;
-            P.obs[n % (unsigned long long)P.obs_cap] = sqrt(S * S + C * C) / (double)N;
-            *P.obs_ctr = n + 1;
+            ring_record_order(P, ((i128)o.tot_hi[0] << sh) + o.tot_lo[0],
+                              ((i128)o.tot_hi[NQ - 1] << sh) + o.tot_lo[NQ - 1]);
         }
         if (!s_ctl.done) {
 #pragma unroll

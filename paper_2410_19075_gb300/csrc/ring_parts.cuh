@@ -337,6 +337,15 @@ __device__ __forceinline__ void ring_window(const RingPlan &P, const int64_t *la
     ring_sums<NQ>(B, tid, P.mp.ksh, lb, la, own, S);
 }
 
+// The Kuramoto order parameter from the ring's exact totals, recorded by one thread.
+__device__ __forceinline__ void ring_record_order(const RingPlan &P, i128 s, i128 c)
+{
+    const double S = fixed_to_double(s, P.F), C = fixed_to_double(c, P.F);
+    const unsigned long long n = *P.obs_ctr;
+    P.obs[n % (unsigned long long)P.obs_cap] = sqrt(S * S + C * C) / (double)P.N;
+    *P.obs_ctr = n + 1;
+}
+
 // Exact prefix of the fixed-point values qv (one per node, 0 past the ring's
 // end; NPT adjacent nodes per thread, kSubTile / NPT threads per CTA, node i0 + u
 // of the thread holds qv[u]) into lam_out / ingrp_out / grpofs_out.  RECORD: the
@@ -421,13 +430,7 @@ __device__ __forceinline__ void ring_prefix_tail_n(const RingPlan &P, int64_t *l
                         for (int k = 0; k < 4; ++k) tk[k] = __reduce_add_sync(0xffffffffu, tk[k]);
                         total[c] = flat_value(tk[0], tk[1], tk[2], tk[3]);
                     }
-                    if (RECORD && lane == 0 && P.obs) {
-                        const double S = fixed_to_double(total[0], P.F);
-                        const double C = fixed_to_double(total[NQ - 1], P.F);
-                        const unsigned long long n = *P.obs_ctr;
-                        P.obs[n % (unsigned long long)P.obs_cap] = sqrt(S * S + C * C) / (double)N;
-                        *P.obs_ctr = n + 1;
-                    }
+                    if (RECORD && lane == 0 && P.obs) ring_record_order(P, total[0], total[NQ - 1]);
                     if (DEC_STEPS && lane == 0 && P.steps_left) *P.steps_left -= 1;
                 }
             }
@@ -451,6 +454,7 @@ __device__ __forceinline__ void ring_prefix_tail_n(const RingPlan &P, int64_t *l
     __syncthreads();
     if (!s_last) return;
     if (warp == 0) {
+        i128 total[NQ]; // of the group, in lane 31
 #pragma unroll
         for (int c = 0; c < NQ; ++c) {
             const int64_t *st = P.subtot + c * nsub + s0;
@@ -461,10 +465,24 @@ __device__ __forceinline__ void ring_prefix_tail_n(const RingPlan &P, int64_t *l
             i128 *ig = ingrp_out + c * nsub + s0;
             if (2 * lane < gsize) st_i128(ig + 2 * lane, e);
             if (2 * lane + 1 < gsize) st_i128(ig + 2 * lane + 1, e + v0);
-            if (lane == 31) st_i128(P.grptot + c * ngroups + g, x);
+            total[c] = x;
+            if (lane == 31 && ngroups > 1) st_i128(P.grptot + c * ngroups + g, x);
+        }
+        if (ngroups == 1) { // the ring's total: no second level
+            if (lane == 31) {
+#pragma unroll
+                for (int c = 0; c < NQ; ++c) {
+                    st_i128(grpofs_out + 2 * c, 0);
+                    st_i128(grpofs_out + 2 * c + 1, total[c]);
+                }
+                if (RECORD && P.obs) ring_record_order(P, total[0], total[NQ - 1]);
+                if (DEC_STEPS && P.steps_left) *P.steps_left -= 1;
+            }
+            return;
         }
         __threadfence();
     }
+    if (ngroups == 1) return;
     __syncthreads();
     if (tid == 0) s_last = last_arrival(P.top_ctr, (unsigned long long)ngroups);
     __syncthreads();
@@ -475,13 +493,7 @@ __device__ __forceinline__ void ring_prefix_tail_n(const RingPlan &P, int64_t *l
 #pragma unroll
     for (int c = 0; c < NQ; ++c)
         total[c] = block_exclusive_scan<8>(P.grptot + c * ngroups, grpofs_out + c * (ngroups + 1), ngroups);
-    if (RECORD && tid == 0 && P.obs) {
-        const double S = fixed_to_double(total[0], P.F);
-        const double C = fixed_to_double(total[NQ - 1], P.F);
-        const unsigned long long n = *P.obs_ctr;
-        P.obs[n % (unsigned long long)P.obs_cap] = sqrt(S * S + C * C) / (double)N;
-        *P.obs_ctr = n + 1;
-    }
+    if (RECORD && tid == 0 && P.obs) ring_record_order(P, total[0], total[NQ - 1]);
     if (DEC_STEPS && tid == 0 && P.steps_left) *P.steps_left -= 1;
 }
 

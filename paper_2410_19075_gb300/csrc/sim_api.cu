@@ -858,7 +858,7 @@ int sim_create_graph(sim_t *out, int model, int64_t N, const int64_t *row_ptr, c
         return cuda_fail(e, "link matrix upload");
     }
     GraphPlan &g = h->graph;
-    h->ring.flat = 0; // the link-matrix kernels read the two-level prefix
+    if (h->ring.nsub > kGraphFlatSubs) h->ring.flat = 0; // the link-matrix kernels read the two-level prefix
     g.r = h->ring;
     g.runs = reinterpret_cast<const int2 *>(b + o_runs);
     g.nruns = (int)T.runs.size();

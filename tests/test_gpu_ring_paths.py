@@ -74,3 +74,27 @@ def test_hh_rates_over_the_voltage_range():
         beta = -oracle.rhs_sampled(2, 0, N, R, params, one, np.arange(N))[1:]
         assert (np.abs(k[1:] - ref[1:]) / (alpha + beta)).max() < 1e-14
         assert np.abs(k[0] - ref[0]).max() < 1e-12 * np.abs(ref[0]).max()
+
+
+@pytest.mark.parametrize("N", [5, 255, 256, 257, 16385, 131072, 131073])
+@pytest.mark.parametrize("model", [0, 1])
+def test_link_matrix_prefix_forms(model, N):
+    """A ring written as rows, on both sides of the size (512 sub-tiles) up to which every
+    CTA scans the sub-tile totals itself, against the ring kernels: both add the same exact
+    sums, and convert them with roundings of 2^-53 of the slope's terms (1e-12)."""
+    from paper_2410_19075_gb300 import Network
+    R = 2
+    cols = (np.arange(N)[:, None] + np.array([d for d in range(-R, R + 1) if d])) % N
+    y0, _ = inputs_for(model, 0, N, 3 + N)
+    outs = []
+    for rows in (False, True):
+        net = (Network.from_links(model, N, np.arange(N + 1) * 2 * R, cols.ravel(), PARAMS[model]()) if rows
+               else Network(model, 0, N, R, PARAMS[model](), streaming=True))
+        net.set_state(y0)
+        k = net.rhs()
+        net.step(3, 0.01)
+        outs.append((k, net.get_state(), net.observables(), net.dp5(t_end=0.1, rtol=1e-6, atol=1e-6, h0=0.01)["status"],
+                     net.get_state()))
+        net.close()
+    for a, b in zip(*outs):
+        assert np.abs(np.asarray(a) - np.asarray(b)).max(initial=0.0) < 1e-12 * max(1.0, np.abs(outs[0][0]).max())
