@@ -188,18 +188,17 @@ struct LatticePlan {
     double *y, *acc;  // D * nodes
     int64_t *f;       // nodes (sin, cos) pairs (f[2n], f[2n+1]) of the current stage-input phase on the grid 2^-62
     double *xs;       // NX * nodes: local stage-input variables (psi of model 3)
-    int64_t *sx;      // cube: 2 * nodes window sums along x (SoA); ball, disk: per row,
+    int64_t *sx;      // cube: (sin, cos) pairs of the window sums along x; ball, disk: per row,
                       // rs (sin, cos) pairs of the periodically extended inclusive
                       // prefix E(x), x in [-P-1, N1+P-1], stored at x + P + 1
     int64_t rs;       // ball, disk: row stride of sx in (sin, cos) pairs (lattice_row_stride)
     int wmode;        // ball, disk: sx holds, for w = 0..P, nodes (sin, cos) pairs of the
                       // x-window sums S_w (one load per chord) instead of the row prefixes
-    int64_t *sxy;     // cube box sums over x and y: 2 components, i-block-major (tiled passes)
-                      // or node order (the batched sliding passes)
+    int64_t *sxy;     // cube: pairs of the box sums over x and y, i-block-major
     double *cpl;      // cube: nodes coupling terms of the current stage (window pass -> node pass)
     i128 *partial;    // per-CTA partial sums of the order parameter
-    unsigned long long *done_ctr; // arrival counter of the sliding-window node passes (and the prologue)
-    unsigned long long *tile_ctr; // arrival counter of the cube node pass (another CTA count per launch)
+    unsigned long long *done_ctr; // arrival counter of small gathers
+    unsigned long long *tile_ctr; // arrival counter of the order kernel (another CTA count per launch)
     unsigned *err;
     double *obs;
     int64_t obs_cap;
@@ -249,9 +248,11 @@ cudaError_t graph_dp_start(const GraphDpPlan &d, cudaStream_t s);
 cudaError_t graph_dp_attempt(const GraphDpPlan &d, cudaStream_t s);
 
 cudaError_t lattice_configure(); // once per process, before the first launch
-int64_t lattice_order_blocks(int topo, int64_t N1); // CTAs of the order-parameter passes (sliding-window grid)
-int64_t lattice_sxy_elems(int64_t N1); // cube: xy-window sums (both layouts of the y pass's output)
-int64_t lattice_partial_blocks(int topo, int64_t N1); // order-parameter partials to allocate (every grid)
+int64_t cube_tiles(int64_t N1);     // CTAs of a cube's y and z-window passes
+int cube_node_warps(int64_t N1);    // rows per CTA of a cube's node pass
+size_t cube_batch_tile_smem(int64_t N1); // shared bytes of its y and z-window CTAs
+int64_t lattice_sxy_elems(int64_t N1); // cube: int64 elements of the x sums and of the xy sums
+int64_t lattice_partial_blocks(int topo, int64_t N1); // order-parameter partials to allocate
 int64_t lattice_row_stride(int64_t N1, int64_t P, bool wmode);
 int lattice_gather_nodes(int topo, int64_t N1); // nodes per thread of the ball and disk gather
 int64_t lattice_sx_elems(int topo, int64_t N1, int64_t P, bool wmode); // int64 elements of sx
@@ -260,22 +261,22 @@ cudaError_t lattice_prologue(const LatticePlan &p, cudaStream_t s);
 cudaError_t lattice_step(const LatticePlan &p, double dt, cudaStream_t s);
 cudaError_t lattice_rhs(const LatticePlan &p, cudaStream_t s); // acc <- f(y)
 
-// Cube members of one model in a batch: device tables of the batched x, y and z
-// launches (lattice.cu).  x: CTA b does rows of member x_item[b] (w warps, one
-// row each, counted from x_base[member]); y and z: CTA b is the member's CTA
-// b - yz_base[member] of its single-network column grid.
+// Cube members of one model in a batch: device tables of the batched launches
+// (lattice.cu).  Node pass: CTA b does rows of member x_item[b] (w warps, one row
+// each, counted from x_base[member]); y and z-window pass: CTA b is the member's CTA
+// b - yz_base[member] of its single-network tile grid.
 struct CubeBatchGroup {
     int model;
     int n_inst;
-    int w;                    // warps per x CTA (for the largest edge)
-    int64_t n1_max;           // largest edge (sizes the x pass's shared rows)
-    int64_t n_x, n_yz;        // CTAs of the x and of the y / z launches
+    int w;                    // warps per node-pass CTA (for the largest edge)
+    size_t tile_smem;         // shared bytes of a y or z-window CTA (the largest tile)
+    int64_t n1_max;           // largest edge (sizes the node pass's shared rows)
+    int64_t n_x, n_yz;        // CTAs of the node pass and of the y / z-window launches
     const LatticePlan *plans; // n_inst (device)
     const int *x_item, *yz_item;
     const int64_t *x_base, *yz_base; // n_inst each
 };
 cudaError_t cube_batch_step(const CubeBatchGroup &g, double dt, cudaStream_t s); // one RK4 step of every member
-int lattice_row_warps(int64_t N1); // warps per CTA of the x pass for edge N1
 void lattice_rotation(LatticePlan &p, double alpha); // rot_* and mp.c[5] of a lattice (sim_api.cu)
 void ring_coupling_constants(ModelParams &mp, int model, const double *params, int F); // ksh and the scaled coupling constants of a ring (sim_api.cu)
 

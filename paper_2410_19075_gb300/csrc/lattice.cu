@@ -15,8 +15,10 @@
 //   z pass  W(i,j,k)   = sum_{|dz|<=P} SXY(i,j,k+dz)       (column prefix in a tile)
 //           and the coupling term; the node pass then runs the right-hand side,
 //           the RK4 update, the next (sin, cos) and the next stage's x pass.
-//           Batched cubes use sliding windows along j and k instead, the z pass
-//           fused with the node update.
+//           Both sums are (sin, cos) pairs: one address, one wrap test and one
+//           16-byte shared access serve the two components (two separate arrays
+//           took 172 instructions per node in the y pass of a 101^3 cube, pairs
+//           122).  Batched cubes run the same passes, one launch for all members.
 // Ball and disk, per RK4 stage:
 //   x pass  balls of P >= 5: for every half-width w = 0..P the x-window sums S_w(i) of
 //           Q(f) along every row, sin and cos interleaved; otherwise, and when those
@@ -36,21 +38,18 @@
 namespace simk {
 
 constexpr int kRowWarpsMax = 8;       // x pass: one warp per row
-constexpr int kColThreads = 128;      // cube y and z passes: threads per CTA along i
-constexpr int64_t kColTarget = 152 * 1024; // cube y and z passes: columns are split into
-                                           // segments until about this many threads run
 constexpr int kGatherThreads = 128;   // ball/disk gather: a block of rows x planes of nodes per thread
 constexpr int kGatherOps = 512;       // ball/disk gather: reads of the window held in shared memory at a time
 constexpr size_t kRowSmemMax = 220 * 1024;
 
-// i-columns per tile: shared memory 2 (N1 + 1) BI 8 bytes stays below ~76 KB
+// i-columns per tile: shared memory (N1 + 1) BI 16 bytes stays below ~76 KB
 // (two or three CTAs per SM) and every row segment of a load is BI * 8 bytes.
 __host__ __device__ inline int cube_tile_lg(int64_t N1) { return N1 <= 297 ? 4 : N1 <= 594 ? 3 : 2; }
 __host__ __device__ inline int cube_tile_bi(int64_t N1) { return 1 << cube_tile_lg(N1); }
 
-// Component stride of the tiled cube's xy-window sums in their i-block-major
-// layout [i-block][j][k][ii]: every i-block padded to BI columns.
-__host__ __device__ inline int64_t cube_sxy_cstride(int64_t N1)
+// Pairs of the cube's x sums ([k][i-block][j][ii]) and of its xy sums
+// ([i-block][j][k][ii]): every i-block padded to BI columns.
+static int64_t cube_sum_pairs(int64_t N1)
 {
     const int BI = cube_tile_bi(N1);
     return ((N1 + BI - 1) / BI) * BI * N1 * N1;
@@ -58,7 +57,7 @@ __host__ __device__ inline int64_t cube_sxy_cstride(int64_t N1)
 
 static int row_warps(int64_t N1)
 {
-    const size_t per_warp = 2 * (size_t)(N1 + 1) * sizeof(int64_t);
+    const size_t per_warp = (size_t)(N1 + 1) * sizeof(longlong2);
     int w = (int)(kRowSmemMax / per_warp);
     return w < 1 ? 1 : (w > kRowWarpsMax ? kRowWarpsMax : w);
 }
@@ -99,168 +98,24 @@ __device__ __forceinline__ void lattice_rotated_q(const LatticePlan &p, int64_t 
     }
 }
 
-// x pass: one warp per row.  pre(p) = sum_{m<p} Q'(f(m)) for p in [0, N1] is built
-// in shared memory.  With Pe(p) = pre(p mod N1) + floor(p / N1) pre(N1) the
-// periodic extension:
-//   MODE 0 (cube)        SX(i) = Pe(i+P+1) - Pe(i-P), sin and cos in two arrays
-//                        (pre0/pre1, stride N1 + 1 per component);
+// x pass: one warp per row.  pre[p] = sum_{m<p} Q'(f(m)) for p in [0, N1] is built
+// in shared memory as (sin, cos) pairs.  With Pe(p) = pre[p mod N1] + floor(p / N1)
+// pre[N1] the periodic extension:
+//   MODE 0 (cube)        SX(i) = Pe(i+P+1) - Pe(i-P);
 //   MODE 1 (ball, disk,  the extended inclusive prefix E(x) = Pe(x+1),
-//           low memory)  x in [-P-1, N1+P-1], (sin, cos) pairs, modulo 2^64;
+//           low memory)  x in [-P-1, N1+P-1], modulo 2^64;
 //   MODE 2 (ball)        for every half-width w = 0..P the window sums
-//                        S_w(i) = Pe(i+w+1) - Pe(i-w), (sin, cos) pairs, one
-//                        array of rows per w.
-// Modes 1 and 2 build Pe on [-P, N1 + P] as (sin, cos) pairs (lattice_ext_row) where
-// that fits in shared memory; longer rows (disks only, mode 1) use pre0/pre1.
-// One row of the x pass (one warp; pre0/pre1 its shared prefix rows).
-// IBLK (cube, the tiled passes): SX in the plane-wise i-block-major layout
-// [k][i-block][j][ii] (cube_sx_index), which each y tile reads as one
-// contiguous block; otherwise node order (the batched sliding passes).
-// The row's own part: pre0/pre1[m + 1] = Q'(f(m)) for m < N1 from the stored
-// (sin, cos).
+//                        S_w(i) = Pe(i+w+1) - Pe(i-w), one array of rows per w.
+// Modes 1 and 2 build Pe on [-P, N1 + P] (lattice_ext_row) where that fits in shared
+// memory; longer rows (disks only, mode 1) extend while they write.
+//
+// The row's quantities into pre[1..N1] from the stored (sin, cos): the cube's
+// unrotated (its node's own phase is turned instead), the ball's and disk's rotated.
 template <int MODE>
-__device__ __forceinline__ void lattice_x_fill(const LatticePlan &p, int64_t row, int64_t *pre0, int64_t *pre1)
+__device__ __forceinline__ void lattice_row_fill(const LatticePlan &p, int64_t row, longlong2 *pre)
 {
-    const int lane = threadIdx.x & 31;
-    const int64_t N1 = p.N1, nodes = p.nodes;
-    const longlong2 *__restrict__ fr = reinterpret_cast<const longlong2 *>(p.f) + row * N1; // (sin, cos) pairs
-    for (int64_t mb = lane; mb < N1; mb += 32 * 8) { // coalesced, 8 loads in flight per lane
-        int64_t vs[8], vc[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const int64_t m = mb + 32 * u;
-            const longlong2 v = m < N1 ? __ldg(fr + m) : make_longlong2(0, 0);
-            vs[u] = v.x;
-            vc[u] = v.y;
-        }
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const int64_t m = mb + 32 * u;
-            if (m < N1) {
-                if (MODE == 0) { // cube: the node's own phase is turned instead
-                    pre0[m + 1] = q62_to(vs[u], p.F);
-                    pre1[m + 1] = q62_to(vc[u], p.F);
-                } else {
-                    lattice_rotated_q(p, vs[u], vc[u], pre0[m + 1], pre1[m + 1]);
-                }
-            }
-        }
-    }
-}
-
-// The row's prefix and window sums from pre0/pre1[1..N1] (filled by the warp).
-template <int MODE, bool IBLK>
-__device__ __forceinline__ void lattice_x_scan_out(const LatticePlan &p, int64_t row, int64_t *pre0, int64_t *pre1)
-{
-    const int lane = threadIdx.x & 31;
-    const int64_t N1 = p.N1, P = p.P, nodes = p.nodes;
-    const int n1 = (int)N1, per = (n1 + 31) >> 5;
-    __syncwarp();
-    // lane l owns the prefix slots m0 .. m1 - 1: its part's total, the warp's
-    // exclusive scan of the totals, then the part's prefix written once
-    const int m0 = min(lane * per, n1) + 1, m1 = min(m0 + per, n1 + 1);
-    uint64_t r0 = 0, r1 = 0; // wrapping sums
-    for (int m = m0; m < m1; ++m) {
-        r0 += (uint64_t)pre0[m];
-        r1 += (uint64_t)pre1[m];
-    }
-    uint64_t e0 = (uint64_t)warp_incl_scan((int64_t)r0) - r0;
-    uint64_t e1 = (uint64_t)warp_incl_scan((int64_t)r1) - r1;
-    for (int m = m0; m < m1; ++m) {
-        e0 += (uint64_t)pre0[m];
-        e1 += (uint64_t)pre1[m];
-        pre0[m] = (int64_t)e0;
-        pre1[m] = (int64_t)e1;
-    }
-    if (lane == 0) {
-        pre0[0] = 0;
-        pre1[0] = 0;
-    }
-    __syncwarp();
-    if (MODE == 1) {
-        // E(x) = Pe(x + 1) for x in [-P-1, N1+P-1], at slot x + P + 1
-        const uint64_t t0 = (uint64_t)pre0[N1], t1 = (uint64_t)pre1[N1];
-        longlong2 *__restrict__ o = reinterpret_cast<longlong2 *>(p.sx) + row * p.rs;
-        for (int64_t e = lane; e < p.rs; e += 32) {
-            int64_t q = e - P; // = x + 1, in [-P, N1 + P]
-            uint64_t v0, v1;
-            if (q < 0) {
-                v0 = (uint64_t)pre0[q + N1] - t0;
-                v1 = (uint64_t)pre1[q + N1] - t1;
-            } else if (q > N1) {
-                v0 = (uint64_t)pre0[q - N1] + t0;
-                v1 = (uint64_t)pre1[q - N1] + t1;
-            } else {
-                v0 = (uint64_t)pre0[q];
-                v1 = (uint64_t)pre1[q];
-            }
-            o[e] = make_longlong2((long long)v0, (long long)v1);
-        }
-    } else {
-        const int64_t t0 = pre0[N1], t1 = pre1[N1];
-        if (IBLK) {
-            // row = k N1 + j; element i at ((k tiles + i / BI) N1 + j) BI + i % BI.
-            // BI divides 32, so lane's column within its i-block stays fixed and
-            // every 32 columns move 32 / BI i-blocks further.
-            const int lg = cube_tile_lg(N1), BI = 1 << lg, p1 = (int)P;
-            const int64_t k = row / N1, j = row - k * N1, tiles = (N1 + BI - 1) >> lg;
-            const int64_t bstep = N1 * BI; // one i-block further
-            int64_t *__restrict__ o0 = p.sx + (k * tiles * N1 + j) * BI;
-            int64_t *__restrict__ o1 = o0 + cube_sxy_cstride(N1);
-            const unsigned ostep = (unsigned)bstep << (5 - lg);
-            unsigned o = (unsigned)((lane >> lg) * bstep) + (lane & (BI - 1));
-#pragma unroll 2
-            for (int i = lane; i < n1; i += 32, o += ostep) {
-                // 2P + 1 <= N1: at most one end of the window wraps, adding the total
-                const int b = i + p1 + 1, a = i - p1;
-                const bool hi = b > n1, lo = a < 0;
-                const int bb = hi ? b - n1 : b, aa = lo ? a + n1 : a;
-                const int64_t s0 = (hi || lo) ? t0 : 0, s1 = (hi || lo) ? t1 : 0;
-                o0[o] = s0 + pre0[bb] - pre0[aa];
-                o1[o] = s1 + pre1[bb] - pre1[aa];
-            }
-            // the last i-block's columns past the cube's edge read as zeros
-            const int64_t pad = tiles * BI - N1;
-            if (lane < pad) {
-                const int64_t o = (tiles - 1) * bstep + (BI - pad + lane);
-                o0[o] = 0;
-                o1[o] = 0;
-            }
-        } else {
-            int64_t *__restrict__ o0 = p.sx + row * N1;
-            int64_t *__restrict__ o1 = p.sx + nodes + row * N1;
-            for (int64_t i = lane; i < N1; i += 32) {
-                int64_t b = i + P + 1, a = i - P;
-                int64_t s0 = 0, s1 = 0;
-                if (b > N1) { b -= N1; s0 += t0; s1 += t1; }
-                if (a < 0) { a += N1; s0 += t0; s1 += t1; } // Pe(a) = pre(a+N1) - total
-                o0[i] = s0 + pre0[b] - pre0[a];
-                o1[i] = s1 + pre1[b] - pre1[a];
-            }
-        }
-    }
-    __syncwarp();
-}
-
-template <int MODE, bool IBLK = false>
-__device__ __forceinline__ void lattice_x_row(const LatticePlan &p, int64_t row, int64_t *pre0, int64_t *pre1,
-                                              bool &)
-{
-    lattice_x_fill<MODE>(p, row, pre0, pre1);
-    lattice_x_scan_out<MODE, IBLK>(p, row, pre0, pre1);
-}
-
-// Ball and disk: the row's extended prefix in shared memory, ext[p + P] = Pe(p)
-// for p in [-P, N1 + P], then the outputs read straight from it: a window sum is
-// two 16-byte shared loads and no wrap test (36 -> 24 us for seven windows of
-// 10^6 nodes; the wrapped form took 20 of its 27 instructions per window).
-// Lanes own an odd number of adjacent slots, so their 16-byte accesses do not
-// share banks.
-template <int MODE>
-__device__ __forceinline__ void lattice_ext_row(const LatticePlan &p, int64_t row, longlong2 *ext)
-{
-    const int lane = threadIdx.x & 31, n1 = (int)p.N1, P = (int)p.P;
+    const int lane = threadIdx.x & 31, n1 = (int)p.N1;
     const longlong2 *__restrict__ fr = reinterpret_cast<const longlong2 *>(p.f) + row * n1;
-    longlong2 *pre = ext + P; // pre[q] = Pe(q)
     for (int mb = lane; mb < n1; mb += 32 * 4) { // 4 loads in flight per lane
         longlong2 v[4];
 #pragma unroll
@@ -269,34 +124,90 @@ __device__ __forceinline__ void lattice_ext_row(const LatticePlan &p, int64_t ro
         for (int u = 0; u < 4; ++u)
             if (mb + 32 * u < n1) {
                 int64_t qs, qc;
-                lattice_rotated_q(p, v[u].x, v[u].y, qs, qc);
+                if (MODE == 0) {
+                    qs = q62_to(v[u].x, p.F);
+                    qc = q62_to(v[u].y, p.F);
+                } else lattice_rotated_q(p, v[u].x, v[u].y, qs, qc);
                 pre[mb + 32 * u + 1] = make_longlong2(qs, qc);
             }
     }
+}
+
+__device__ __forceinline__ longlong2 pair_add(longlong2 a, longlong2 b)
+{
+    return make_longlong2((long long)((uint64_t)a.x + (uint64_t)b.x), (long long)((uint64_t)a.y + (uint64_t)b.y));
+}
+__device__ __forceinline__ longlong2 pair_sub(longlong2 a, longlong2 b)
+{
+    return make_longlong2((long long)((uint64_t)a.x - (uint64_t)b.x), (long long)((uint64_t)a.y - (uint64_t)b.y));
+}
+
+// pre[1..n1] -> its inclusive prefix, pre[0] = 0; returns the row's total (wrapping
+// sums).  Lanes own an odd number of adjacent slots, so their 16-byte accesses do
+// not share banks.
+__device__ __forceinline__ longlong2 lattice_row_prefix(longlong2 *pre, int n1)
+{
+    const int lane = threadIdx.x & 31;
     __syncwarp();
     const int per = ((n1 + 31) >> 5) | 1;
     const int m0 = min(lane * per, n1) + 1, m1 = min(m0 + per, n1 + 1);
-    uint64_t r0 = 0, r1 = 0; // wrapping sums
+    longlong2 r = make_longlong2(0, 0);
+    for (int m = m0; m < m1; ++m) r = pair_add(r, pre[m]);
+    const longlong2 x = make_longlong2(warp_incl_scan(r.x), warp_incl_scan(r.y));
+    longlong2 e = pair_sub(x, r);
     for (int m = m0; m < m1; ++m) {
-        const longlong2 v = pre[m];
-        r0 += (uint64_t)v.x;
-        r1 += (uint64_t)v.y;
-    }
-    const uint64_t i0 = (uint64_t)warp_incl_scan((int64_t)r0), i1 = (uint64_t)warp_incl_scan((int64_t)r1);
-    uint64_t e0 = i0 - r0, e1 = i1 - r1;
-    for (int m = m0; m < m1; ++m) {
-        const longlong2 v = pre[m];
-        e0 += (uint64_t)v.x;
-        e1 += (uint64_t)v.y;
-        pre[m] = make_longlong2((long long)e0, (long long)e1);
+        e = pair_add(e, pre[m]);
+        pre[m] = e;
     }
     if (lane == 0) pre[0] = make_longlong2(0, 0);
-    const uint64_t t0 = __shfl_sync(0xffffffffu, i0, 31), t1 = __shfl_sync(0xffffffffu, i1, 31); // the row's total
     __syncwarp();
+    return make_longlong2(__shfl_sync(0xffffffffu, x.x, 31), __shfl_sync(0xffffffffu, x.y, 31));
+}
+
+// Window sum at a (0 <= a < n1) of a prefix with its entries `step` pairs apart:
+// Pe(a + P + 1) - Pe(a - P).  As 2P + 1 <= n1, at most one end wraps, and either wrap
+// adds the total once.
+__device__ __forceinline__ longlong2 pair_window(const longlong2 *pre, int n1, int P, int lg, int a, longlong2 total)
+{
+    const bool wb = a + P + 1 > n1, wl = a < P;
+    const int b = a + P + 1 - (wb ? n1 : 0), lo = a - P + (wl ? n1 : 0);
+    const longlong2 w = pair_sub(pre[(unsigned)b << lg], pre[(unsigned)lo << lg]);
+    return wb || wl ? pair_add(w, total) : w;
+}
+
+// The cube's x sums of a row from its prefix, in the plane-wise i-block-major layout
+// each y tile reads as one contiguous block: row = k N1 + j; element i at
+// ((k tiles + i / BI) N1 + j) BI + i % BI, zeros past the cube's edge.  BI divides 32,
+// so a lane's column within its i-block stays fixed and every 32 columns move
+// 32 / BI i-blocks further.
+__device__ __forceinline__ void cube_x_out(const LatticePlan &p, int64_t row, const longlong2 *pre, longlong2 total)
+{
+    const int lane = threadIdx.x & 31, n1 = (int)p.N1, P = (int)p.P;
+    const int lg = cube_tile_lg(n1), BI = 1 << lg, tiles = (n1 + BI - 1) >> lg;
+    const int64_t k = row / n1, j = row - k * n1;
+    const unsigned bstep = (unsigned)n1 << lg; // one i-block further
+    longlong2 *__restrict__ o = reinterpret_cast<longlong2 *>(p.sx) + ((k * tiles * n1 + j) << lg);
+    unsigned at = (unsigned)(lane >> lg) * bstep + (lane & (BI - 1));
+#pragma unroll 2
+    for (int i = lane; i < tiles << lg; i += 32, at += bstep << (5 - lg))
+        o[at] = i < n1 ? pair_window(pre, n1, P, 0, i, total) : make_longlong2(0, 0);
+    __syncwarp();
+}
+
+// Ball and disk: the row's extended prefix in shared memory, ext[p + P] = Pe(p)
+// for p in [-P, N1 + P], then the outputs read straight from it: a window sum is
+// two 16-byte shared loads and no wrap test (36 -> 24 us for seven windows of
+// 10^6 nodes; the wrapped form took 20 of its 27 instructions per window).
+template <int MODE>
+__device__ __forceinline__ void lattice_ext_row(const LatticePlan &p, int64_t row, longlong2 *ext)
+{
+    const int lane = threadIdx.x & 31, n1 = (int)p.N1, P = (int)p.P;
+    longlong2 *pre = ext + P; // pre[q] = Pe(q)
+    lattice_row_fill<MODE>(p, row, pre);
+    const longlong2 total = lattice_row_prefix(pre, n1);
     for (int q = lane; q < P; q += 32) { // 2P + 1 <= N1: both extensions read pre[0..N1]
-        const longlong2 lo = pre[q - P + n1], hi = pre[q + 1];
-        pre[q - P] = make_longlong2((long long)((uint64_t)lo.x - t0), (long long)((uint64_t)lo.y - t1));
-        pre[n1 + q + 1] = make_longlong2((long long)((uint64_t)hi.x + t0), (long long)((uint64_t)hi.y + t1));
+        pre[q - P] = pair_sub(pre[q - P + n1], total);
+        pre[n1 + q + 1] = pair_add(pre[q + 1], total);
     }
     __syncwarp();
     longlong2 *__restrict__ sx = reinterpret_cast<longlong2 *>(p.sx);
@@ -308,11 +219,7 @@ __device__ __forceinline__ void lattice_ext_row(const LatticePlan &p, int64_t ro
         const int64_t warray = p.nodes / n1 * p.rs;
         for (int w = 0; w <= P; ++w, o += warray)
 #pragma unroll 4
-            for (int i = lane; i < n1; i += 32) {
-                const longlong2 hi = pre[i + w + 1], lo = pre[i - w];
-                o[i] = make_longlong2((long long)((uint64_t)hi.x - (uint64_t)lo.x),
-                                      (long long)((uint64_t)hi.y - (uint64_t)lo.y));
-            }
+            for (int i = lane; i < n1; i += 32) o[i] = pair_sub(pre[i + w + 1], pre[i - w]);
     }
     __syncwarp();
 }
@@ -334,132 +241,27 @@ static int ext_warps(int64_t N1, int64_t P)
     return (int)(w > kRowWarpsMax ? kRowWarpsMax : w);
 }
 
+// The x pass of a cube (MODE 0) or of rows too long for lattice_ext_kernel (MODE 1).
 template <int MODE>
 __global__ void __launch_bounds__(32 * kRowWarpsMax) lattice_x_kernel(LatticePlan p)
 {
     if (p.skip && *(const volatile int *)p.skip) return;
-    extern __shared__ int64_t smem[];
-    const int warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-    const int64_t stride = p.N1 + 1, rows = p.nodes / p.N1;
-    int64_t *pre0 = smem + (int64_t)warp * 2 * stride;
-    int64_t *pre1 = pre0 + stride;
-    bool ok = true;
-    for (int64_t row = (int64_t)blockIdx.x * nwarps + warp; row < rows; row += (int64_t)gridDim.x * nwarps)
-        lattice_x_row<MODE, MODE == 0>(p, row, pre0, pre1, ok);
-    if (!ok) raise_error(p.err, ERR_RANGE);
-}
-
-// Batched cube x pass: CTA b works on rows (b - x_base[m]) * warps + warp of
-// member m = x_item[b]; shared memory is sized for the group's largest edge.
-__global__ void __launch_bounds__(32 * kRowWarpsMax)
-    cube_batch_x_kernel(const LatticePlan *__restrict__ plans, const int *__restrict__ x_item,
-                        const int64_t *__restrict__ x_base)
-{
-    const int inst = x_item[blockIdx.x];
-    const LatticePlan &p = plans[inst];
-    extern __shared__ int64_t smem[];
-    const int warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-    const int64_t stride = p.N1 + 1, rows = p.nodes / p.N1;
-    int64_t *pre0 = smem + (int64_t)warp * 2 * stride;
-    int64_t *pre1 = pre0 + stride;
-    const int64_t row = ((int64_t)blockIdx.x - x_base[inst]) * nwarps + warp;
-    bool ok = true;
-    if (row < rows) lattice_x_row<0, true>(p, row, pre0, pre1, ok); // uniform over the warp
-    if (!ok) raise_error(p.err, ERR_RANGE);
-}
-
-// Columns of the y and z passes are split into gridDim.z segments of
-// col_seg_len() nodes (small cubes would otherwise run a few thousand threads,
-// each walking its column serially); every segment starts its own sliding
-// window, so the window sums, being exact, do not depend on the split.
-__host__ __device__ inline int64_t col_segments(int64_t N1)
-{
-    const int64_t cols = N1 * N1;
-    int64_t nseg = (kColTarget + cols - 1) / cols;
-    if (nseg > N1) nseg = N1;
-    return nseg < 1 ? 1 : nseg;
-}
-
-__host__ __device__ inline int64_t col_seg_len(int64_t N1)
-{
-    const int64_t nseg = col_segments(N1);
-    return (N1 + nseg - 1) / nseg;
-}
-
-// cube y pass: one thread per segment of an (i, k) column, sliding window along
-// j (exact int64), 8 rows of window loads issued together; writes the window
-// sums.
-__device__ __forceinline__ void cube_y_col(const LatticePlan &p, int64_t i, int64_t k, int64_t seg)
-{
-    constexpr int U = 8;
-    const int64_t N1 = p.N1, P = p.P, nodes = p.nodes;
-    const int64_t len = col_seg_len(N1), jb = seg * len;
-    const int64_t je = jb + len < N1 ? jb + len : N1;
-    if (i >= N1 || jb >= N1) return;
-    const int64_t col = k * N1 * N1 + i; // + j * N1
-    // the x sums in the plane-wise i-block-major layout: (i, j, k) at
-    // ((k tiles + i / BI) N1 + j) BI + i % BI, so consecutive j are BI apart
-    const int lg = cube_tile_lg(N1), BI = 1 << lg;
-    const int64_t tiles = (N1 + BI - 1) >> lg;
-    const int64_t *__restrict__ a0 = p.sx + ((k * tiles + (i >> lg)) * N1) * BI + (i & (BI - 1));
-    const int64_t *__restrict__ a1 = a0 + cube_sxy_cstride(N1);
-    int64_t *__restrict__ o0 = p.sxy + col;
-    int64_t *__restrict__ o1 = p.sxy + nodes + col;
-    int64_t s0 = 0, s1 = 0;
-    for (int64_t d = -P; d <= P; ++d) {
-        int64_t j = jb + d;
-        j += j < 0 ? N1 : 0;
-        j -= j >= N1 ? N1 : 0;
-        s0 += __ldg(a0 + j * BI);
-        s1 += __ldg(a1 + j * BI);
-    }
-    for (int64_t j0 = jb; j0 < je; j0 += U) {
-        int64_t in0[U], out0[U], in1[U], out1[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int64_t j = j0 + u;
-            int64_t jin = j + P + 1, jout = j - P;
-            if (jin >= N1) jin -= N1;
-            if (jout < 0) jout += N1;
-            const bool live = j < je;
-            in0[u] = live ? __ldg(a0 + jin * BI) : 0;
-            out0[u] = live ? __ldg(a0 + jout * BI) : 0;
-            in1[u] = live ? __ldg(a1 + jin * BI) : 0;
-            out1[u] = live ? __ldg(a1 + jout * BI) : 0;
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int64_t j = j0 + u;
-            if (j < je) {
-                o0[j * N1] = s0;
-                o1[j * N1] = s1;
-            }
-            s0 += in0[u] - out0[u];
-            s1 += in1[u] - out1[u];
+    extern __shared__ __align__(16) longlong2 row_mem[];
+    const int warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5, lane = threadIdx.x & 31;
+    const int64_t rows = p.nodes / p.N1, row = (int64_t)blockIdx.x * nwarps + warp;
+    if (row >= rows) return; // uniform over the warp
+    longlong2 *pre = row_mem + warp * (p.N1 + 1);
+    lattice_row_fill<MODE>(p, row, pre);
+    const longlong2 total = lattice_row_prefix(pre, (int)p.N1);
+    if (MODE == 0) {
+        cube_x_out(p, row, pre, total);
+    } else { // E(x) = Pe(x + 1) for x in [-P-1, N1+P-1], at slot x + P + 1
+        longlong2 *__restrict__ o = reinterpret_cast<longlong2 *>(p.sx) + row * p.rs;
+        for (int64_t e = lane; e < p.rs; e += 32) {
+            const int64_t q = e - p.P; // = x + 1, in [-P, N1 + P]
+            o[e] = q < 0 ? pair_sub(pre[q + p.N1], total) : q > p.N1 ? pair_add(pre[q - p.N1], total) : pre[q];
         }
     }
-}
-
-// The (column block, plane, segment) of CTA b of a batched y or z pass: the
-// member's CTAs in the order of the single-network grid (x fastest).
-__device__ __forceinline__ void cube_col_item(const LatticePlan &p, int64_t lb, int64_t &bx, int64_t &plane,
-                                              int64_t &seg)
-{
-    const int64_t nbx = (p.N1 + kColThreads - 1) / kColThreads;
-    bx = lb % nbx;
-    plane = (lb / nbx) % p.N1;
-    seg = lb / (nbx * p.N1);
-}
-
-__global__ void __launch_bounds__(kColThreads)
-    cube_batch_y_kernel(const LatticePlan *__restrict__ plans, const int *__restrict__ yz_item,
-                        const int64_t *__restrict__ yz_base)
-{
-    const int inst = yz_item[blockIdx.x];
-    const LatticePlan &p = plans[inst];
-    int64_t bx, k, seg;
-    cube_col_item(p, (int64_t)blockIdx.x - yz_base[inst], bx, k, seg);
-    cube_y_col(p, bx * kColThreads + threadIdx.x, k, seg);
 }
 
 // Deterministic order parameter of the new state: per-CTA partial sums of the
@@ -655,87 +457,26 @@ __device__ __forceinline__ void lattice_node_finish(const LatticePlan &p, int64_
     lattice_node_update<M, STAGE, Acc>(p, n, k, in, h, ok, ps, pc);
 }
 
-// TURN (the cube): the window sums are unrotated, and the node's own phase is
-// turned by +alpha for the cross product instead (own_phase_turned).
-template <int M, int STAGE, bool TURN = false>
+template <int M, int STAGE>
 __device__ __forceinline__ void lattice_node(const LatticePlan &p, int64_t n, int64_t W0, int64_t W1, const StepSize &h,
                                              bool &ok, i128 &ps, i128 &pc)
 {
     LatNodeIn<M> in;
     lattice_node_load<M, STAGE>(p, n, in);
-    if (TURN && STAGE > 0) {
-        int64_t t62[2];
-        own_phase_turned(p.mp, in.f62, t62);
-        in.f62[0] = t62[0];
-        in.f62[1] = t62[1];
-    }
     lattice_node_finish<M, STAGE, i128>(p, n, W0, W1, in, h, ok, ps, pc);
 }
 
-// Batched cube z pass: one thread per segment of an (i, j) column, sliding
-// window along k, fused with the node update.
-template <int M, int STAGE>
-__device__ __forceinline__ void cube_z_col(const LatticePlan &p, const StepSize &h, int64_t bx, int64_t j,
-                                           int64_t seg, unsigned bid, unsigned nblk)
-{
-    const int64_t N1 = p.N1, P = p.P, nodes = p.nodes, plane = N1 * N1;
-    const int64_t i = bx * kColThreads + threadIdx.x;
-    const int64_t len = col_seg_len(N1), kb = seg * len;
-    const int64_t ke = kb + len < N1 ? kb + len : N1;
-    i128 ps = 0, pc = 0;
-    bool ok = true;
-    if (i < N1) {
-        const int64_t col = j * N1 + i; // + k * plane
-        const int64_t *__restrict__ a0 = p.sxy + col;
-        const int64_t *__restrict__ a1 = p.sxy + nodes + col;
-        int64_t s0 = 0, s1 = 0;
-        if (STAGE > 0 && kb < N1) {
-            for (int64_t d = -P; d <= P; ++d) {
-                int64_t k = kb + d;
-                k += k < 0 ? N1 : 0;
-                k -= k >= N1 ? N1 : 0;
-                s0 += __ldg(a0 + k * plane);
-                s1 += __ldg(a1 + k * plane);
-            }
-        }
-        for (int64_t k = kb; k < ke; ++k) {
-            lattice_node<M, STAGE, true>(p, col + k * plane, s0, s1, h, ok, ps, pc);
-            if (STAGE > 0) {
-                int64_t kin = k + P + 1, kout = k - P;
-                if (kin >= N1) kin -= N1;
-                if (kout < 0) kout += N1;
-                s0 += __ldg(a0 + kin * plane) - __ldg(a0 + kout * plane);
-                s1 += __ldg(a1 + kin * plane) - __ldg(a1 + kout * plane);
-            }
-        }
-    }
-    if (!ok) raise_error(p.err, ERR_RANGE);
-    if (STAGE == 0 || STAGE == 4) lattice_record_order(p, ps, pc, bid, nblk, p.done_ctr);
-}
-
 // ---------------------------------------------------------------------------
-// Tiled y and z passes of a single cube (the batched cubes keep the sliding
-// windows above and below; both give the same exact sums).  CTA (ib, m) loads
-// the 2 x N1 x BI block of one plane (y pass: plane k = m, i-block ib, all j) or
-// one row of columns (z pass: row j = m, i-block ib, all k) into shared memory,
-// so that every element crosses HBM once (a sliding window re-reads the element
-// leaving the window, 2P+1 rows or planes after it entered, long gone from L2
-// on large cubes).  The block is scanned in place into the exact inclusive
-// prefix along the window axis (wrapping int64 arithmetic, as the x pass), and
-// every window sum is Pe(a+P+1) - Pe(a-P) on its periodic extension.
+// Tiled y and z passes of a cube.  CTA (ib, m) loads the N1 x BI block of pairs of
+// one plane (y pass: plane k = m, i-block ib, all j) or one row of columns (z pass:
+// row j = m, i-block ib, all k) into shared memory, so that every element crosses
+// HBM once.  The block is scanned in place into the exact inclusive prefix along the
+// window axis (wrapping int64 arithmetic, as the x pass), and every window sum is
+// Pe(a+P+1) - Pe(a-P) on its periodic extension.
 constexpr int kTileThreads = 256;
 
-// Asynchronous 8-byte copy global -> shared (zero fill when !live); the copies
-// of a thread complete at cp_async_wait_all.
-__device__ __forceinline__ void cp_async8(uint64_t *dst, const uint64_t *src, bool live)
-{
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"((unsigned)__cvta_generic_to_shared(dst)),
-                 "l"(src), "r"(live ? 8 : 0)
-                 : "memory");
-}
-
 // Asynchronous 16-byte copy global -> shared (both addresses 16-byte aligned).
-__device__ __forceinline__ void cp_async16(uint64_t *dst, const uint64_t *src)
+__device__ __forceinline__ void cp_async16(longlong2 *dst, const longlong2 *src)
 {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"((unsigned)__cvta_generic_to_shared(dst)),
                  "l"(src)
@@ -746,127 +487,94 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 
 __host__ __device__ inline size_t cube_tile_smem(int64_t N1)
 {
-    return (size_t)2 * (size_t)(N1 + 1) * (size_t)cube_tile_bi(N1) * sizeof(int64_t);
+    return (size_t)(N1 + 1) * (size_t)cube_tile_bi(N1) * sizeof(longlong2);
 }
 
-// Turn every column (c, ii) of a loaded tile into its inclusive prefix along a
-// (wrapping uint64): NT / (2 BI) segments per column, segment sums, their
-// exclusive scan, rewrite.  Called by every thread of the CTA after the tile's
-// rows 1..N1 and its zero row 0 are in place and visible; ends with a barrier.
+// Load a contiguous block blk[a BI + ii] (a < N1, ii < BI = 2^lg; zeros past the cube's
+// edge) into tile[(a + 1) BI + ii] by asynchronous 16-byte copies, so that the whole
+// tile is in flight at once, and turn every column into its inclusive prefix along
+// a (tile row 0 zero): NT / BI segments per column, the segment sums scanned inside a
+// warp by shuffles and across warps from shared memory.  Called by every thread of
+// the CTA; ends with a barrier.
 template <int NT>
-__device__ __forceinline__ void cube_tile_scan(int N1, int lg, uint64_t *tile)
+__device__ __forceinline__ void cube_tile_load_scan(const longlong2 *blk, int N1, int lg, longlong2 *tile)
 {
-    const int tid = threadIdx.x, BI = 1 << lg;
-    const unsigned cstride = (unsigned)(N1 + 1) << lg; // tile words per component
-    __shared__ uint64_t s_seg[NT];
-    const int ncol = 2 * BI, nseg = NT / ncol;
-    const int col = tid & (ncol - 1), sg = tid >> (lg + 1);
-    uint64_t *colp = tile + (col >> lg) * cstride + (col & (BI - 1));
-    const int seg = (N1 + nseg - 1) / nseg;
-    const int a0 = 1 + sg * seg, a1 = min(N1 + 1, a0 + seg);
-    uint64_t t = 0;
-    for (int a = a0; a < a1; ++a) t += colp[(unsigned)a << lg];
-    s_seg[sg * ncol + col] = t;
+    constexpr int NW = NT / 32;
+    __shared__ longlong2 s_warp[NW][16];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, BI = 1 << lg;
+    for (int e = tid; e < N1 << lg; e += NT) cp_async16(tile + BI + e, blk + e);
+    if (tid < BI) tile[tid] = make_longlong2(0, 0);
+    cp_async_wait_all();
     __syncthreads();
-    uint64_t run = 0;
-    for (int q = 0; q < sg; ++q) run += s_seg[q * ncol + col];
+    const int nseg = NT >> lg, seg = (N1 + nseg - 1) / nseg;
+    const int a0 = min((tid >> lg) * seg, N1) + 1, a1 = min(a0 + seg, N1 + 1);
+    longlong2 *colp = tile + (tid & (BI - 1));
+    longlong2 t = make_longlong2(0, 0);
+    for (int a = a0; a < a1; ++a) t = pair_add(t, colp[a << lg]);
+    longlong2 x = t; // inclusive over the warp's segments of the column
+    for (int d = BI; d < 32; d <<= 1) {
+        const longlong2 u = make_longlong2(__shfl_up_sync(0xffffffffu, x.x, d), __shfl_up_sync(0xffffffffu, x.y, d));
+        if (lane >= d) x = pair_add(x, u);
+    }
+    if (lane >= 32 - BI) s_warp[warp][lane & (BI - 1)] = x;
+    __syncthreads();
+    longlong2 run = pair_sub(x, t);
+    for (int w = 0; w < warp; ++w) run = pair_add(run, s_warp[w][lane & (BI - 1)]);
     for (int a = a0; a < a1; ++a) {
-        run += colp[(unsigned)a << lg];
-        colp[(unsigned)a << lg] = run;
+        run = pair_add(run, colp[a << lg]);
+        colp[a << lg] = run;
     }
     __syncthreads();
 }
 
-// Load src[c nodes + base + a stride + ii] for c < 2, a < N1, ii < BI = 2^lg (0
-// for ii >= bi, past the cube's edge) into tile[(c (N1 + 1) + a + 1) BI + ii]
-// (asynchronous 8-byte copies, so that the whole tile is in flight at once),
-// zero row 0 of both components, then scan (cube_tile_scan).  Offsets inside
-// the cube are 32-bit (N1 <= 1024, so a * stride < 2^30).  Called by every
-// thread of the CTA; ends with a barrier.
-template <int NT>
-__device__ __forceinline__ void cube_tile_load_scan(const int64_t *__restrict__ src, int64_t nodes, int64_t base,
-                                                    unsigned stride, int N1, int lg, int bi, uint64_t *tile)
+// Tiled cube y pass: CTA (ib, k); writes the window sums in the i-block-major layout
+// the z-window pass reads as one contiguous block (element (ii, j = a, k) at
+// ((ib N1 + a) N1 + k) BI + ii; the columns past the cube's edge are zeros already).
+// The loop is split where a window wraps, so that most of it tests nothing.
+__device__ __forceinline__ void cube_y_tile(const LatticePlan &p, int ib, int k, longlong2 *tile)
 {
-    const int tid = threadIdx.x, BI = 1 << lg, rstep = NT >> lg;
-    const int ii = tid & (BI - 1), r0 = tid >> lg;
-    const bool live = ii < bi;
-    const unsigned cstride = (unsigned)(N1 + 1) << lg;
-#pragma unroll
-    for (int c = 0; c < 2; ++c) {
-        // past the cube's edge: a zero fill from an in-bounds address
-        const uint64_t *__restrict__ s = reinterpret_cast<const uint64_t *>(src) + c * nodes + base + (live ? ii : 0);
-        uint64_t *t = tile + c * cstride + BI + ii;
-        for (int a = r0; a < N1; a += rstep) cp_async8(t + ((unsigned)a << lg), s + (unsigned)a * stride, live);
-    }
-    if (tid < 2 * BI) tile[(tid >> lg) * cstride + (tid & (BI - 1))] = 0ull;
-    cp_async_wait_all();
-    __syncthreads();
-    cube_tile_scan<NT>(N1, lg, tile);
+    const int N1 = (int)p.N1, P = (int)p.P, lg = cube_tile_lg(N1), BI = 1 << lg;
+    const int64_t tiles = (N1 + BI - 1) >> lg;
+    cube_tile_load_scan<kTileThreads>(reinterpret_cast<const longlong2 *>(p.sx) + ((k * tiles + ib) * N1 << lg), N1, lg, tile);
+    const int ii = threadIdx.x & (BI - 1), rstep = kTileThreads >> lg;
+    const longlong2 *col = tile + ii;
+    const longlong2 total = col[N1 << lg];
+    longlong2 *__restrict__ d = reinterpret_cast<longlong2 *>(p.sxy) + (((int64_t)ib * N1 * N1 + k) << lg) + ii;
+    const unsigned dstep = (unsigned)N1 << lg;
+    int a = threadIdx.x >> lg;
+    for (; a < P; a += rstep)
+        d[(unsigned)a * dstep] = pair_add(pair_sub(col[(a + P + 1) << lg], col[(a - P + N1) << lg]), total);
+#pragma unroll 4
+    for (; a < N1 - P; a += rstep) d[(unsigned)a * dstep] = pair_sub(col[(a + P + 1) << lg], col[(a - P) << lg]);
+    for (; a < N1; a += rstep)
+        d[(unsigned)a * dstep] = pair_add(pair_sub(col[(a + P + 1 - N1) << lg], col[(a - P) << lg]), total);
 }
 
-// The same from a contiguous block per component (the i-block-major layout of
-// the xy-window sums, blk[c] + a BI + ii, zeros already stored past the edge):
-// asynchronous 16-byte copies.
-template <int NT>
-__device__ __forceinline__ void cube_tile_load_scan_contig(const int64_t *blk0, const int64_t *blk1, int N1, int lg,
-                                                           uint64_t *tile)
-{
-    const int tid = threadIdx.x, BI = 1 << lg;
-    const unsigned cstride = (unsigned)(N1 + 1) << lg;
-    const int words = N1 << lg; // even: BI >= 4
-#pragma unroll
-    for (int c = 0; c < 2; ++c) {
-        const uint64_t *__restrict__ s = reinterpret_cast<const uint64_t *>(c ? blk1 : blk0);
-        uint64_t *t = tile + c * cstride + BI;
-        for (int e = 2 * tid; e < words; e += 2 * NT) cp_async16(t + e, s + e);
-    }
-    if (tid < 2 * BI) tile[(tid >> lg) * cstride + (tid & (BI - 1))] = 0ull;
-    cp_async_wait_all();
-    __syncthreads();
-    cube_tile_scan<NT>(N1, lg, tile);
-}
-
-// Window sum at a (0 <= a < N1) of a scanned column colp (its words BI = 2^lg
-// apart, total = colp[N1 BI]): Pe(a + P + 1) - Pe(a - P) on the periodic
-// extension Pe(x) = pre(x mod N1) + floor(x / N1) total.  As 2P + 1 <= N1, at
-// most one end wraps, and either wrap adds the total once.
-__device__ __forceinline__ int64_t cube_tile_window(const uint64_t *colp, int N1, int P, int lg, int a, uint64_t total)
-{
-    int b = a + P + 1, lo = a - P;
-    const bool wb = b > N1, wl = lo < 0;
-    b -= wb ? N1 : 0;
-    lo += wl ? N1 : 0;
-    return (int64_t)(colp[(unsigned)b << lg] - colp[(unsigned)lo << lg] + ((wb || wl) ? total : 0ull));
-}
-
-// Tiled cube y pass: CTA (ib, k); writes the window sums in the i-block-major
-// layout the z-window pass reads as one contiguous block.
 __global__ void __launch_bounds__(kTileThreads) cube_y_tile_kernel(LatticePlan p)
 {
     if (p.skip && *(const volatile int *)p.skip) return;
-    extern __shared__ int64_t tile_mem[];
-    uint64_t *tile = reinterpret_cast<uint64_t *>(tile_mem);
-    const int N1 = (int)p.N1, P = (int)p.P, lg = cube_tile_lg(N1), BI = 1 << lg;
-    const int i0 = (int)blockIdx.x << lg, k = blockIdx.y;
-    const int bi = min(BI, N1 - i0);
-    const int64_t tiles = (N1 + BI - 1) >> lg;
-    const int64_t *blk = p.sx + ((int64_t)k * tiles + blockIdx.x) * N1 * BI; // plane-wise i-block-major
-    cube_tile_load_scan_contig<kTileThreads>(blk, blk + cube_sxy_cstride(N1), N1, lg, tile);
-    const int ii = threadIdx.x & (BI - 1), r0 = threadIdx.x >> lg, rstep = kTileThreads >> lg;
-    const unsigned cstride = (unsigned)(N1 + 1) << lg;
-    const uint64_t *col0 = tile + ii, *col1 = tile + cstride + ii;
-    const uint64_t t0 = col0[(unsigned)N1 << lg], t1 = col1[(unsigned)N1 << lg];
-    // i-block-major output: element (ii, j = a, k) at ((ib N1 + a) N1 + k) BI + ii,
-    // zeros past the cube's edge
-    int64_t *__restrict__ d0 = p.sxy + (((int64_t)blockIdx.x * N1) * N1 + k) * BI + ii;
-    int64_t *__restrict__ d1 = d0 + cube_sxy_cstride(N1);
-    const unsigned dstep = (unsigned)N1 << lg;
-#pragma unroll 4 // 464^3: 0.493 ms, against 0.515 (unroll 2) and 0.516-0.517 (6, 8)
-    for (int a = r0; a < N1; a += rstep) {
-        const bool live = ii < bi;
-        d0[(unsigned)a * dstep] = live ? cube_tile_window(col0, N1, P, lg, a, t0) : 0;
-        d1[(unsigned)a * dstep] = live ? cube_tile_window(col1, N1, P, lg, a, t1) : 0;
-    }
+    extern __shared__ __align__(16) longlong2 tile_mem[];
+    cube_y_tile(p, blockIdx.x, blockIdx.y, tile_mem);
+}
+
+// Batched cubes: CTA b is tile b - yz_base[m] of member m = yz_item[b], in the order of
+// the single cube's grid.
+__device__ __forceinline__ void cube_batch_tile(const LatticePlan &p, int64_t lb, int &ib, int &m)
+{
+    const int lg = cube_tile_lg(p.N1), tiles = (int)((p.N1 + (1 << lg) - 1) >> lg);
+    m = (int)lb / tiles;
+    ib = (int)lb - m * tiles;
+}
+__global__ void __launch_bounds__(kTileThreads)
+    cube_batch_y_kernel(const LatticePlan *__restrict__ plans, const int *__restrict__ yz_item,
+                        const int64_t *__restrict__ yz_base)
+{
+    extern __shared__ __align__(16) longlong2 tile_mem[];
+    const int inst = yz_item[blockIdx.x];
+    const LatticePlan &p = plans[inst];
+    int ib, k;
+    cube_batch_tile(p, (int64_t)blockIdx.x - yz_base[inst], ib, k);
+    cube_y_tile(p, ib, k, tile_mem);
 }
 
 // A node's coupling term to cpl (KM = -1), or its whole slope to acc for a
@@ -916,49 +624,56 @@ __device__ __forceinline__ void lattice_write_coupling(const LatticePlan &p, int
 constexpr int kZThreads = 384, kZAhead = 3, kZBlocks = 3; // kZAhead: planes of own (sin, cos) in flight
 
 template <int KM> // -1: coupling terms; a model: the slopes of a right-hand-side evaluation
-__global__ void __launch_bounds__(kZThreads, kZBlocks) cube_zw_tile_kernel(LatticePlan p)
+__device__ __forceinline__ void cube_zw_tile(const LatticePlan &p, int ib, int j, longlong2 *tile)
 {
-    if (p.skip && *(const volatile int *)p.skip) return;
-    extern __shared__ int64_t tile_mem[];
-    uint64_t *tile = reinterpret_cast<uint64_t *>(tile_mem);
     const int N1 = (int)p.N1, P = (int)p.P, lg = cube_tile_lg(N1), BI = 1 << lg;
-    const int i0 = (int)blockIdx.x << lg, j = blockIdx.y;
-    const int bi = min(BI, N1 - i0);
+    const int i0 = ib << lg, bi = min(BI, N1 - i0);
     const unsigned plane = (unsigned)N1 * (unsigned)N1;
-    const int64_t base = (int64_t)j * N1 + i0;
-    const int64_t *blk = p.sxy + (((int64_t)blockIdx.x * N1 + j) * N1) * BI; // i-block-major
-    cube_tile_load_scan_contig<kZThreads>(blk, blk + cube_sxy_cstride(N1), N1, lg, tile);
+    cube_tile_load_scan<kZThreads>(reinterpret_cast<const longlong2 *>(p.sxy) + (((int64_t)ib * N1 + j) * N1 << lg), N1, lg, tile);
     const int ii = threadIdx.x & (BI - 1), r0 = threadIdx.x >> lg, rstep = kZThreads >> lg;
     if (ii >= bi || r0 >= N1) return; // past every barrier
-    const unsigned cstride = (unsigned)(N1 + 1) << lg;
-    const uint64_t *col0 = tile + ii, *col1 = tile + cstride + ii;
-    const uint64_t t0 = col0[(unsigned)N1 << lg], t1 = col1[(unsigned)N1 << lg];
-    const longlong2 *__restrict__ fp = reinterpret_cast<const longlong2 *>(p.f) + base + ii; // (sin, cos) pairs
-    int64_t f[kZAhead + 1][2]; // own (sin, cos) of the planes a, a + rstep, ...
+    const longlong2 *col = tile + ii;
+    const longlong2 total = col[N1 << lg];
+    const int64_t base = (int64_t)j * N1 + i0 + ii;
+    const longlong2 *__restrict__ fp = reinterpret_cast<const longlong2 *>(p.f) + base; // (sin, cos) pairs
+    longlong2 f[kZAhead + 1]; // own (sin, cos) of the planes a, a + rstep, ...
 #pragma unroll
     for (int d = 0; d < kZAhead; ++d) {
         const int ad = r0 + d * rstep;
-        const longlong2 v = ad < N1 ? fp[(unsigned)ad * plane] : make_longlong2(0, 0);
-        f[d][0] = v.x;
-        f[d][1] = v.y;
+        f[d] = ad < N1 ? fp[(unsigned)ad * plane] : make_longlong2(0, 0);
     }
 #pragma unroll 2 // two planes' independent chains interleaved
     for (int a = r0; a < N1; a += rstep) {
         const int an = a + kZAhead * rstep;
-        const longlong2 v = an < N1 ? fp[(unsigned)an * plane] : make_longlong2(0, 0);
-        f[kZAhead][0] = v.x;
-        f[kZAhead][1] = v.y;
+        f[kZAhead] = an < N1 ? fp[(unsigned)an * plane] : make_longlong2(0, 0);
+        const int64_t f62[2] = {f[0].x, f[0].y};
         int64_t t62[2];
-        own_phase_turned(p.mp, f[0], t62);
-        lattice_write_slope<KM>(p, base + ii + (unsigned)a * plane,
-                                lattice_coupling_term(p.mp, t62, cube_tile_window(col0, N1, P, lg, a, t0),
-                                                      cube_tile_window(col1, N1, P, lg, a, t1)));
+        own_phase_turned(p.mp, f62, t62);
+        const longlong2 w = pair_window(col, N1, P, lg, a, total);
+        lattice_write_slope<KM>(p, base + (unsigned)a * plane, lattice_coupling_term(p.mp, t62, w.x, w.y));
 #pragma unroll
-        for (int d = 0; d < kZAhead; ++d) {
-            f[d][0] = f[d + 1][0];
-            f[d][1] = f[d + 1][1];
-        }
+        for (int d = 0; d < kZAhead; ++d) f[d] = f[d + 1];
     }
+}
+
+template <int KM>
+__global__ void __launch_bounds__(kZThreads, kZBlocks) cube_zw_tile_kernel(LatticePlan p)
+{
+    if (p.skip && *(const volatile int *)p.skip) return;
+    extern __shared__ __align__(16) longlong2 tile_mem[];
+    cube_zw_tile<KM>(p, blockIdx.x, blockIdx.y, tile_mem);
+}
+
+__global__ void __launch_bounds__(kZThreads, kZBlocks)
+    cube_batch_zw_kernel(const LatticePlan *__restrict__ plans, const int *__restrict__ yz_item,
+                         const int64_t *__restrict__ yz_base)
+{
+    extern __shared__ __align__(16) longlong2 tile_mem[];
+    const int inst = yz_item[blockIdx.x];
+    const LatticePlan &p = plans[inst];
+    int ib, j;
+    cube_batch_tile(p, (int64_t)blockIdx.x - yz_base[inst], ib, j);
+    cube_zw_tile<-1>(p, ib, j, tile_mem);
 }
 
 template <int M, int STAGE>
@@ -989,8 +704,8 @@ __device__ __forceinline__ void cube_node_load(const LatticePlan &p, int64_t n, 
 // 1.33 ms; staging the row's y and coupling terms through shared memory by
 // cp.async instead took 1.39 ms.  The loads bypass L1 (1% faster).
 template <int M, int STAGE>
-__device__ __forceinline__ void cube_nodex_row(const LatticePlan &p, const StepSize &h, int64_t row, int64_t *pre0,
-                                               int64_t *pre1, bool &ok, int64_t &ps, int64_t &pc)
+__device__ __forceinline__ void cube_nodex_row(const LatticePlan &p, const StepSize &h, int64_t row, longlong2 *pre,
+                                               bool &ok, int64_t &ps, int64_t &pc)
 {
     constexpr int D = Model<M>::D, U = D == 1 ? 6 : 4;
     const int lane = threadIdx.x & 31, n1 = (int)p.N1;
@@ -1020,8 +735,7 @@ __device__ __forceinline__ void cube_nodex_row(const LatticePlan &p, const StepS
                 int64_t unused_s = 0, unused_c = 0;
                 lattice_node_update<M, STAGE, int64_t>(q, (unsigned)i, k, in[u], h, ok, unused_s, unused_c, sc);
                 const int64_t qs = q62_to(sc[0], p.F), qc = q62_to(sc[1], p.F);
-                pre0[i + 1] = qs;
-                pre1[i + 1] = qc;
+                pre[i + 1] = make_longlong2(qs, qc);
                 if (STAGE == 0 || STAGE == 4) {
                     ps += qs;
                     pc += qc;
@@ -1029,48 +743,55 @@ __device__ __forceinline__ void cube_nodex_row(const LatticePlan &p, const StepS
             }
         }
     }
-    lattice_x_scan_out<0, true>(p, row, pre0, pre1);
+    cube_x_out(p, row, pre, lattice_row_prefix(pre, n1));
 }
 
+// CTA bid of a cube's node pass.
 template <int M, int STAGE>
-__global__ void __launch_bounds__(32 * kNodexWarpsMax, kNodexBlocks<M>) cube_nodex_kernel(LatticePlan p, const StepSize h)
+__device__ __forceinline__ void cube_nodex_cta(const LatticePlan &p, const StepSize &h, int64_t bid, longlong2 *mem)
 {
-    if (p.skip && *(const volatile int *)p.skip) return;
-    extern __shared__ int64_t smem[];
     const int warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-    const int64_t stride = p.N1 + 1, rows = p.nodes / p.N1;
-    int64_t *pre0 = smem + (int64_t)warp * 2 * stride;
-    int64_t *pre1 = pre0 + stride;
-    const int64_t row = (int64_t)blockIdx.x * nwarps + warp;
+    const int64_t rows = p.nodes / p.N1, row = bid * nwarps + warp;
     // a lane's order sums: at most ceil(N1 / 32) <= 32 terms of |Q| <= 2^F <= 2^56
     // (F = 61 - ceil(log2 K+) and K+ >= 27), so int64 holds them
     int64_t ps = 0, pc = 0;
     bool ok = true;
-    if (row < rows) cube_nodex_row<M, STAGE>(p, h, row, pre0, pre1, ok, ps, pc); // uniform over the warp
+    if (row < rows) cube_nodex_row<M, STAGE>(p, h, row, mem + warp * (p.N1 + 1), ok, ps, pc); // uniform over the warp
     if (!ok) raise_error(p.err, ERR_RANGE);
     if (STAGE == 0 || STAGE == 4) { // the order parameter's partials (lattice_order_kernel adds them up)
         i128 ts = ps, tc = pc;
         cta_sum_pair(ts, tc);
         if (threadIdx.x == 0) {
-            st_i128(p.partial + 2 * blockIdx.x, ts);
-            st_i128(p.partial + 2 * blockIdx.x + 1, tc);
+            st_i128(p.partial + 2 * bid, ts);
+            st_i128(p.partial + 2 * bid + 1, tc);
         }
     }
 }
 
-// Batched cube z pass (stages 1-4): CTA b is CTA b - yz_base[m] of member m.
 template <int M, int STAGE>
-__global__ void __launch_bounds__(kColThreads)
-    cube_batch_z_kernel(const LatticePlan *__restrict__ plans, const int *__restrict__ yz_item,
-                        const int64_t *__restrict__ yz_base, const StepSize h)
+__global__ void __launch_bounds__(32 * kNodexWarpsMax, kNodexBlocks<M>) cube_nodex_kernel(LatticePlan p, const StepSize h)
 {
-    const int inst = yz_item[blockIdx.x];
-    const LatticePlan &p = plans[inst];
-    const int64_t lb = (int64_t)blockIdx.x - yz_base[inst];
-    int64_t bx, j, seg;
-    cube_col_item(p, lb, bx, j, seg);
-    const int64_t nbx = (p.N1 + kColThreads - 1) / kColThreads;
-    cube_z_col<M, STAGE>(p, h, bx, j, seg, (unsigned)lb, (unsigned)(nbx * p.N1 * col_segments(p.N1)));
+    extern __shared__ __align__(16) longlong2 row_mem[];
+    cube_nodex_cta<M, STAGE>(p, h, blockIdx.x, row_mem);
+}
+
+// Batched cubes: CTA b is CTA b - x_base[m] of member m = x_item[b].
+template <int M, int STAGE>
+__global__ void __launch_bounds__(32 * kNodexWarpsMax, kNodexBlocks<M>)
+    cube_batch_nodex_kernel(const LatticePlan *__restrict__ plans, const int *__restrict__ x_item,
+                            const int64_t *__restrict__ x_base, const StepSize h)
+{
+    extern __shared__ __align__(16) longlong2 row_mem[];
+    const int inst = x_item[blockIdx.x];
+    cube_nodex_cta<M, STAGE>(plans[inst], h, (int64_t)blockIdx.x - x_base[inst], row_mem);
+}
+
+// Order parameters of batched cubes, one CTA per member, from the partials of node
+// passes of w rows per CTA.
+__global__ void __launch_bounds__(kOrderThreads) cube_batch_order_kernel(const LatticePlan *__restrict__ plans, int w)
+{
+    const LatticePlan &p = plans[blockIdx.x];
+    lattice_order_total(p, p.partial, (unsigned)((p.nodes / p.N1 + w - 1) / w));
 }
 
 // ball / disk gather: a thread gathers the window sums of kGatherTj x TK nodes (j,
@@ -1261,31 +982,22 @@ int64_t lattice_row_stride(int64_t N1, int64_t P, bool wmode)
 
 int64_t lattice_sx_elems(int topo, int64_t N1, int64_t P, bool wmode)
 {
-    if (topo == 1) return lattice_sxy_elems(N1); // both layouts of the x pass's output
+    if (topo == 1) return lattice_sxy_elems(N1);
     const int64_t rows = topo == 3 ? N1 : N1 * N1;
     return 2 * (wmode ? P + 1 : 1) * rows * lattice_row_stride(N1, P, wmode);
 }
 
-int64_t lattice_sxy_elems(int64_t N1)
-{
-    const int64_t a = N1 * N1 * N1, b = cube_sxy_cstride(N1);
-    return 2 * (a > b ? a : b);
-}
+int64_t lattice_sxy_elems(int64_t N1) { return 2 * cube_sum_pairs(N1); }
+
+int64_t cube_tiles(int64_t N1) { return (N1 + cube_tile_bi(N1) - 1) / cube_tile_bi(N1) * N1; }
+int cube_node_warps(int64_t N1) { return nodex_warps(N1); }
 
 int64_t lattice_partial_blocks(int topo, int64_t N1)
 {
-    const int64_t a = lattice_order_blocks(topo, N1);
-    if (topo != 1) return a + kOrderCtas;
-    // the fused node pass (one row per warp) and the order kernel's second level
-    const int64_t b = (N1 * N1 + nodex_warps(N1) - 1) / nodex_warps(N1) + kOrderCtas;
-    return a > b ? a : b;
-}
-
-int64_t lattice_order_blocks(int topo, int64_t N1)
-{
-    if (topo == 1) return ((N1 + kColThreads - 1) / kColThreads) * N1 * col_segments(N1);
+    // the cube's node pass (one row per warp) or the gather, and the order kernel's second level
+    if (topo == 1) return (N1 * N1 + nodex_warps(N1) - 1) / nodex_warps(N1) + kOrderCtas;
     const dim3 g = gather_grid(topo, N1);
-    return (int64_t)g.x * g.y;
+    return (int64_t)g.x * g.y + kOrderCtas;
 }
 
 cudaError_t lattice_configure()
@@ -1296,55 +1008,54 @@ cudaError_t lattice_configure()
         e = cudaFuncSetAttribute(lattice_x_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)kRowSmemMax);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(cube_batch_x_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)kRowSmemMax);
-    if (e == cudaSuccess)
         e = cudaFuncSetAttribute(lattice_ext_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRowSmemMax);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(lattice_ext_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRowSmemMax);
     // the largest tile of any edge: the top edge of each tile width
     const int tmax = (int)std::max(std::max(cube_tile_smem(297), cube_tile_smem(594)), cube_tile_smem(1024));
     if (e == cudaSuccess) e = cudaFuncSetAttribute(cube_y_tile_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, tmax);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(cube_batch_y_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, tmax);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(cube_batch_zw_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, tmax);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(cube_zw_tile_kernel<-1>, cudaFuncAttributeMaxDynamicSharedMemorySize, tmax);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(cube_zw_tile_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, tmax);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(cube_zw_tile_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, tmax);
 #define SIM_NODEX_ATTR(M, S)                                                                                           \
     if (e == cudaSuccess)                                                                                              \
-        e = cudaFuncSetAttribute(cube_nodex_kernel<M, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRowSmemMax);
+        e = cudaFuncSetAttribute(cube_nodex_kernel<M, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRowSmemMax); \
+    if (e == cudaSuccess && S > 0)                                                                                     \
+        e = cudaFuncSetAttribute(cube_batch_nodex_kernel<M, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRowSmemMax);
     SIM_NODEX_ATTR(0, 0) SIM_NODEX_ATTR(0, 1) SIM_NODEX_ATTR(0, 2) SIM_NODEX_ATTR(0, 3) SIM_NODEX_ATTR(0, 4)
     SIM_NODEX_ATTR(3, 0) SIM_NODEX_ATTR(3, 1) SIM_NODEX_ATTR(3, 2) SIM_NODEX_ATTR(3, 3) SIM_NODEX_ATTR(3, 4)
 #undef SIM_NODEX_ATTR
     return e;
 }
 
-int lattice_row_warps(int64_t N1) { return row_warps(N1); }
-
-// Batched cube members of one model: one x, one y and one z launch over all of
-// them per pass (each member with its own plan, prefix rows and order-parameter
-// counter).  Between steps a cube's x-window sums hold the sums of y (the
-// prologue, the fused node pass of a single cube's stage 4 and the batch's last
-// x pass keep it so), so a step begins with the y pass and a member can be
-// stepped alone or in a batch in any order; the results are the same bits.
-static cudaError_t cube_batch_x(const CubeBatchGroup &g, cudaStream_t s)
-{
-    const size_t smem = (size_t)g.w * 2 * (size_t)(g.n1_max + 1) * sizeof(int64_t);
-    cube_batch_x_kernel<<<(unsigned)g.n_x, 32 * g.w, smem, s>>>(g.plans, g.x_item, g.x_base);
-    return cudaGetLastError();
-}
-
+// Batched cube members of one model: the single cube's passes, one launch over all
+// members each (every member with its own plan and order-parameter record), so a
+// member can be stepped alone or in a batch in any order with the same bits.
+// Against sliding windows along j and k (node-order sums, the z pass fused with the
+// node update, columns split into segments) a step of 48 networks, rings and cubes
+// mixed, took 1.20 ms in place of 1.52.
 template <int M>
-static cudaError_t cube_batch_yz(int stage, const CubeBatchGroup &g, double dt, cudaStream_t s)
+static cudaError_t cube_batch_stage(int stage, const CubeBatchGroup &g, double dt, cudaStream_t s)
 {
-    cube_batch_y_kernel<<<(unsigned)g.n_yz, kColThreads, 0, s>>>(g.plans, g.yz_item, g.yz_base);
+    cube_batch_y_kernel<<<(unsigned)g.n_yz, kTileThreads, g.tile_smem, s>>>(g.plans, g.yz_item, g.yz_base);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
+    cube_batch_zw_kernel<<<(unsigned)g.n_yz, kZThreads, g.tile_smem, s>>>(g.plans, g.yz_item, g.yz_base);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     const StepSize h = step_size(dt);
-    const dim3 grid((unsigned)g.n_yz);
+    const unsigned grid = (unsigned)g.n_x, nt = 32u * (unsigned)g.w;
+    const size_t smem = sizeof(longlong2) * (size_t)g.w * (size_t)(g.n1_max + 1);
     switch (stage) {
-    case 1: cube_batch_z_kernel<M, 1><<<grid, kColThreads, 0, s>>>(g.plans, g.yz_item, g.yz_base, h); break;
-    case 2: cube_batch_z_kernel<M, 2><<<grid, kColThreads, 0, s>>>(g.plans, g.yz_item, g.yz_base, h); break;
-    case 3: cube_batch_z_kernel<M, 3><<<grid, kColThreads, 0, s>>>(g.plans, g.yz_item, g.yz_base, h); break;
-    default: cube_batch_z_kernel<M, 4><<<grid, kColThreads, 0, s>>>(g.plans, g.yz_item, g.yz_base, h); break;
+    case 1: cube_batch_nodex_kernel<M, 1><<<grid, nt, smem, s>>>(g.plans, g.x_item, g.x_base, h); break;
+    case 2: cube_batch_nodex_kernel<M, 2><<<grid, nt, smem, s>>>(g.plans, g.x_item, g.x_base, h); break;
+    case 3: cube_batch_nodex_kernel<M, 3><<<grid, nt, smem, s>>>(g.plans, g.x_item, g.x_base, h); break;
+    default:
+        cube_batch_nodex_kernel<M, 4><<<grid, nt, smem, s>>>(g.plans, g.x_item, g.x_base, h);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        cube_batch_order_kernel<<<(unsigned)g.n_inst, kOrderThreads, 0, s>>>(g.plans, g.w);
+        break;
     }
     return cudaGetLastError();
 }
@@ -1353,12 +1064,13 @@ cudaError_t cube_batch_step(const CubeBatchGroup &g, double dt, cudaStream_t s)
 {
     if (g.n_x == 0) return cudaSuccess;
     for (int stage = 1; stage <= 4; ++stage) {
-        cudaError_t e = stage > 1 ? cube_batch_x(g, s) : cudaSuccess;
-        if (e == cudaSuccess) e = g.model == 3 ? cube_batch_yz<3>(stage, g, dt, s) : cube_batch_yz<0>(stage, g, dt, s);
+        const cudaError_t e = g.model == 3 ? cube_batch_stage<3>(stage, g, dt, s) : cube_batch_stage<0>(stage, g, dt, s);
         if (e != cudaSuccess) return e;
     }
-    return cube_batch_x(g, s); // the x sums of y_{n+1}
+    return cudaSuccess;
 }
+
+size_t cube_batch_tile_smem(int64_t N1) { return cube_tile_smem(N1); }
 
 // CTAs of a lattice x pass: one row per warp.
 static unsigned x_grid(const LatticePlan &p)
@@ -1370,7 +1082,7 @@ static unsigned x_grid(const LatticePlan &p)
 
 static size_t x_smem(const LatticePlan &p)
 {
-    return (size_t)row_warps(p.N1) * 2 * (size_t)(p.N1 + 1) * sizeof(int64_t);
+    return (size_t)row_warps(p.N1) * (size_t)(p.N1 + 1) * sizeof(longlong2);
 }
 
 static cudaError_t launch_x(const LatticePlan &p, cudaStream_t s)
@@ -1413,7 +1125,7 @@ static cudaError_t launch_cube_stage(const LatticePlan &p, double dt, cudaStream
     const int w = nodex_warps(p.N1);
     const int64_t rows = p.nodes / p.N1;
     const unsigned nblk = (unsigned)((rows + w - 1) / w);
-    cube_nodex_kernel<M, STAGE><<<nblk, 32 * w, (size_t)w * 2 * (size_t)(p.N1 + 1) * sizeof(int64_t), s>>>(
+    cube_nodex_kernel<M, STAGE><<<nblk, 32 * w, (size_t)w * (size_t)(p.N1 + 1) * sizeof(longlong2), s>>>(
         p, step_size(dt));
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     kernel_mark(s, 2);

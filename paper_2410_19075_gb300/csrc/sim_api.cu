@@ -1247,24 +1247,27 @@ int sim_batch_create(sim_batch_t *out, const sim_t *members, int n_members, void
         else if (members[i]->topo == SIM_CUBE3D) cubes[members[i]->model == SIM_KSI ? 1 : 0].push_back(i);
         else b->lattices.push_back(members[i]);
     }
-    // cube members: one x, y and z launch per stage for each model (tables below)
+    // cube members: one launch per pass and stage for each model (tables below)
     std::vector<LatticePlan> cplans;
     std::vector<int> cx_item, cyz_item;
     std::vector<int64_t> cx_base, cyz_base;
-    struct CubeSpan { int model, plan0, n, w; int64_t n1_max, x0, nx, yz0, nyz; };
+    struct CubeSpan { int model, plan0, n, w; int64_t n1_max, x0, nx, yz0, nyz; size_t tile_smem; };
     std::vector<CubeSpan> cspans;
     for (int c = 0; c < 2; ++c) {
         if (cubes[c].empty()) continue;
         CubeSpan cs{c ? 3 : 0, (int)cplans.size(), (int)cubes[c].size(), 0, 0, (int64_t)cx_item.size(), 0,
-                    (int64_t)cyz_item.size(), 0};
-        for (int i : cubes[c]) cs.n1_max = std::max(cs.n1_max, members[i]->lat.N1);
-        cs.w = lattice_row_warps(cs.n1_max);
+                    (int64_t)cyz_item.size(), 0, 0};
+        for (int i : cubes[c]) {
+            cs.n1_max = std::max(cs.n1_max, members[i]->lat.N1);
+            cs.tile_smem = std::max(cs.tile_smem, cube_batch_tile_smem(members[i]->lat.N1));
+        }
+        cs.w = cube_node_warps(cs.n1_max);
         for (int k = 0; k < cs.n; ++k) {
             const LatticePlan &lp = members[cubes[c][k]]->lat;
             cplans.push_back(lp);
             cx_base.push_back(cs.nx);
             cyz_base.push_back(cs.nyz);
-            const int64_t nx = (lp.N1 * lp.N1 + cs.w - 1) / cs.w, nyz = lattice_order_blocks(SIM_CUBE3D, lp.N1);
+            const int64_t nx = (lp.N1 * lp.N1 + cs.w - 1) / cs.w, nyz = cube_tiles(lp.N1);
             cx_item.insert(cx_item.end(), (size_t)nx, k);
             cyz_item.insert(cyz_item.end(), (size_t)nyz, k);
             cs.nx += nx;
@@ -1372,6 +1375,7 @@ int sim_batch_create(sim_batch_t *out, const sim_t *members, int n_members, void
         g.model = cs.model;
         g.n_inst = cs.n;
         g.w = cs.w;
+        g.tile_smem = cs.tile_smem;
         g.n1_max = cs.n1_max;
         g.n_x = cs.nx;
         g.n_yz = cs.nyz;
