@@ -8,21 +8,22 @@
 // Methods (textbook; constants derived for this code from pi and ln 2 in
 // high-precision arithmetic):
 //   sin/cos  fixed_sincos, in integer arithmetic only: additive range
-//            reduction by pi/512 (Cody & Waite 1980), t = |x| * 512/pi from one
+//            reduction by pi/2048 (Cody & Waite 1980), t = |x| * 2048/pi from one
 //            unsigned 64 x 64 high product of |x| 2^55 and 512/pi 2^56 (grid
-//            2^-47); k = nearest integer to t, r = (t - k) pi/512 with
-//            |r| <= pi/1024; Taylor polynomials sin r = r - r^3 (1/6 - r^2/120)
-//            and cos r - 1 = -r^2/2 + r^4/24 (first omitted terms below 2^-73
-//            and 2^-59), whose small terms take 32 x 32 products; the
-//            angle-addition formula around the table point j pi/512,
-//            j = k mod 1024 (the "accurate table" approach of Tang and Gal):
-//            sin x = S_j + C_j sin r + S_j (cos r - 1) and
-//            cos x = C_j - S_j sin r + C_j (cos r - 1), (S_j, C_j) rounded to
-//            2^-62.  The result is sin and cos on the grid 2^-62 within 2^-53.4
-//            of the true values for |x| < 256 (a host model of the same integer
-//            steps was checked against long double sinl/cosl over 2 * 10^7
-//            arguments and every reduction edge: worst error 7.7e-17, set by the
-//            grid 2^-47 of t); that grid is what the exact window sums consume.
+//            2^-45); k = floor t, r = (t - k) pi/2048 >= 0; Taylor polynomials
+//            sin r = r - r^3 (1/6 - r^2/120) and cos r - 1 = -r^2/2 + r^4/24
+//            (first omitted terms below 2^-65), whose small terms take 32 x 32
+//            products; the angle-addition formula around the table point
+//            j pi/2048 of the first quadrant, j = k mod 1024 (the "accurate table"
+//            approach of Tang and Gal): S_j + C_j sin r + S_j (cos r - 1) and
+//            C_j - S_j sin r + C_j (cos r - 1), (S_j, C_j) on the grid 2^-62, then
+//            k / 1024 quarter turns.  Every factor is non-negative, so that no
+//            product needs a sign correction.  The result is sin and cos on the
+//            grid 2^-62, of magnitude at most 2^62, within 2^-53.6 of the true
+//            values for |x| < 256 (a host model of the same integer steps was
+//            checked against long double sinl/cosl over 2 * 10^7 arguments and the
+//            reduction edges: worst error 7.2e-17, set by the grid of t); that
+//            grid is what the exact window sums consume.
 //            |x| >= 256, Inf and NaN use the library routine.
 //   exp      Tang (1989) table-driven method: x = (64 m + j) ln2/64 + r,
 //            exp(x) = 2^m 2^(j/64) exp(r), degree-5 Taylor polynomial for
@@ -39,27 +40,25 @@
 namespace simk {
 
 // Tables (host-filled at handle creation; see sim_api.cu).
-constexpr int kSinTab = 1024;  // sin/cos(j pi/512), j in [0, 1024)
+constexpr int kSinTab = 1024;  // sin/cos(j pi/2048), j in [0, 1024)
 constexpr int kExpTab = 64;    // 2^(j/64), j in [0, 64)
 constexpr int kExp2Tab = 256;  // 2^(j/256), j in [0, 256)
 
 struct MathTables {
-    const double2 *sincos;     // (sin, cos) of j*pi/512
+    const ulonglong2 *sincos_q; // (sin, cos) of j*pi/2048 on the grid 2^-62 (fill_math_tables)
     const double *exp2j;       // 2^(j/64)
-    const longlong2 *sincos_q; // (sin, cos) of j*pi/512 rounded onto the grid 2^-62
     const unsigned long long *exp2q; // 2^(j/256) rounded onto the grid 2^-63
 };
 
 // The tables as one block of 64-bit words (host-filled in long double, uploaded
-// once per network or device): sincos (2 kSinTab doubles), exp2j (kExpTab
-// doubles), sincos_q (2 kSinTab int64), exp2q (kExp2Tab uint64).
-constexpr int kMathTableWords = 2 * kSinTab + kExpTab + 2 * kSinTab + kExp2Tab;
+// once per network or device): sincos_q (2 kSinTab uint64), exp2j (kExpTab
+// doubles), exp2q (kExp2Tab uint64).
+constexpr int kMathTableWords = 2 * kSinTab + kExpTab + kExp2Tab;
 __host__ __device__ inline MathTables math_tables_at(const void *block)
 {
     const double *d = static_cast<const double *>(block);
-    return MathTables{reinterpret_cast<const double2 *>(d), d + 2 * kSinTab,
-                      reinterpret_cast<const longlong2 *>(d + 2 * kSinTab + kExpTab),
-                      reinterpret_cast<const unsigned long long *>(d + 4 * kSinTab + kExpTab)};
+    return MathTables{reinterpret_cast<const ulonglong2 *>(d), d + 2 * kSinTab,
+                      reinterpret_cast<const unsigned long long *>(d + 2 * kSinTab + kExpTab)};
 }
 
 // |x| as a float by truncating the mantissa (integer instructions; |x| must be
@@ -96,10 +95,29 @@ __device__ __forceinline__ int round_scaled(float xf, float scale)
 
 // Constants of fixed_sincos (derived from pi in 60-digit arithmetic).
 constexpr uint64_t kPio512Inv56 = 0xa2f9836e4e44152aull; // round(512/pi * 2^56)
-constexpr uint64_t kPio512Q71 = 0xc90fdaa22168c235ull;   // round(pi/512 * 2^71)
+constexpr uint64_t kPio2048Q73 = 0xc90fdaa22168c235ull;  // round(pi/2048 * 2^73)
 constexpr uint32_t kSixthQ34 = 2863311531u;               // round(2^34 / 6)
-constexpr uint32_t kInv120Q32 = 35791394u;                // round(2^32 / 120)
-constexpr uint32_t kInv24Q36 = 2863311531u;               // round(2^36 / 24)
+constexpr uint32_t kInv120Q16 = 546u;                     // round(2^16 / 120)
+constexpr uint32_t kInv24Q28 = 11184811u;                 // round(2^28 / 24)
+
+// a b / 2^64 from three 32 x 32 products, the low words' product left out: the
+// exact floor or one less.  a <= 2^63 and b <= 2^63, so that the sum of the middle
+// products stays below 2^64.  (On GB300 a 32 x 32 + 64 multiply-add retires at half
+// rate, and the exact high product takes four and their carries.)
+__device__ __forceinline__ uint64_t umulhi_near(uint64_t a, uint64_t b)
+{
+    const uint32_t ah = (uint32_t)(a >> 32), al = (uint32_t)a, bh = (uint32_t)(b >> 32), bl = (uint32_t)b;
+    return (uint64_t)ah * bh + (((uint64_t)ah * bl + (uint64_t)al * bh) >> 32);
+}
+
+// A signed factor v in [-2^62, 2^62] moved to [0, 2^63] for an unsigned product:
+// with a constant b that is a multiple of 4, floor(v b / 2^64) is the high product
+// of biased62(v) and b less b / 4 (one addition in the high word, against a compare,
+// two selects and a 64-bit subtraction in mulhi_su).
+__device__ __forceinline__ uint64_t biased62(int64_t v)
+{
+    return (uint64_t)v + (1ull << 62);
+}
 
 // floor(a b / 2^64) for signed a and unsigned b: the unsigned high product of
 // a's two's-complement bits, less b when a is negative.
@@ -118,16 +136,18 @@ __device__ __forceinline__ int64_t mulhi_ss(int64_t a, int64_t b)
 }
 
 // sin x and cos x on the grid 2^-62 (s62, c62 in [-2^62, 2^62]), absolute
-// error below 2^-53.4.  Integer instructions only on the fast path |x| < 256;
+// error below 2^-53.6.  Integer instructions only on the fast path |x| < 256;
 // beyond it, and for Inf and NaN, the library routine (ok = false for a
-// non-finite x).  Every 64 x 64 product is unsigned (on GB300 the signed
-// high product costs about 1.7 unsigned ones):
-//   X = |x| 2^55 (truncated), t = X (512/pi) 2^-64 on the grid 2^-47,
-//   k = nearest integer to t, f = t - k in [-1/2, 1/2), r = f pi/512;
-//   sin|r| = |r| - |r|^3 (1/6 - r^2/120) and 1 - cos r = r^2/2 - r^4/24, the
-//   small terms from 32 x 32 products of the top words;
-//   the angle-addition formula around the table point j pi/512, j = k mod 1024:
-//   sin = S_j - S_j (1 - cos r) + C_j sin r, cos = C_j - C_j (1 - cos r) - S_j sin r.
+// non-finite x).
+//   X = |x| 2^55 (truncated), t = X (512/pi) 2^-64: |x| 2048/pi on the grid 2^-45,
+//   k = floor t, r = (t - k) pi/2048 in [0, pi/2048);
+//   sin r = r - r^3 (1/6 - r^2/120) and 1 - cos r = r^2/2 - r^4/24, the small
+//   terms from 32 x 32 products of the top words;
+//   the angle-addition formula around the table point j pi/2048, j = k mod 1024;
+//   quarter turns by k / 1024.
+// Against a table over the half turn, r rounded to nearest and signed factors (33
+// wide multiplies and four sign corrections; here 26 and none) a Kuramoto ring of
+// 10^6 nodes takes 98 us per RK4 step in place of 104, a 101^3 cube 151 of 160.
 __device__ __forceinline__ void fixed_sincos(double x, const MathTables &T, int64_t &s62, int64_t &c62, bool &ok)
 {
     const uint64_t b = (uint64_t)__double_as_longlong(x);
@@ -139,26 +159,28 @@ __device__ __forceinline__ void fixed_sincos(double x, const MathTables &T, int6
         c62 = to_fixed(c, 62, 1, ok);
         return;
     }
-    const uint64_t m = (b & 0xFFFFFFFFFFFFFull) | (1ull << 52);
-    const uint64_t X = e >= 1020 ? m << (e - 1020) : m >> min(1020 - e, 63); // |x| 2^55 < 2^63
-    const uint64_t t = __umul64hi(X, kPio512Inv56);                          // |x| 512/pi 2^47
-    const uint64_t k = (t + (1ull << 46)) >> 47;
-    const int64_t f47 = (int64_t)(t - (k << 47)); // f 2^47, |f| <= 1/2
-    const bool rneg = f47 < 0;
-    const uint64_t R = __umul64hi((uint64_t)(rneg ? -f47 : f47) << 17, kPio512Q71); // |r| 2^71
-    const uint64_t z = __umul64hi(R, R);                                             // r^2 2^78
-    const uint32_t zh = (uint32_t)(z >> 32);                                         // r^2 2^46
-    const uint32_t v57 = (uint32_t)(((uint64_t)(uint32_t)(R >> 32) * zh) >> 28);    // |r|^3 2^57
-    const uint32_t u34 = kSixthQ34 - __umulhi((uint32_t)(z >> 44), kInv120Q32);     // (1/6 - r^2/120) 2^34
-    const uint64_t sr = (R >> 7) - (((uint64_t)v57 * u34) >> 27);                   // sin|r| 2^64
-    const uint32_t w = (uint32_t)(((uint64_t)zh * zh) >> 32);                       // r^4 2^60
-    const uint64_t cm = (z >> 15) - (((uint64_t)w * kInv24Q36) >> 32);              // (1 - cos r) 2^64
-    const longlong2 tq = __ldg(T.sincos_q + (k & (kSinTab - 1)));                   // (S_j, C_j) 2^62
-    const int64_t p1 = mulhi_su(tq.y, sr), p3 = mulhi_su(tq.x, sr);
-    const int64_t s = tq.x - mulhi_su(tq.x, cm) + (rneg ? -p1 : p1);
-    const int64_t c = tq.y - mulhi_su(tq.y, cm) - (rneg ? -p3 : p3);
-    s62 = (b >> 63) ? -s : s;
-    c62 = c;
+    const uint64_t m = ((b << 10) & ((1ull << 62) - 1)) | (1ull << 62); // significand 2^62
+    const uint64_t t = __umul64hi(m >> min(1030 - e, 63), kPio512Inv56); // |x| 2048/pi 2^45
+    const uint32_t k = (uint32_t)(t >> 45);
+    const uint64_t g = t << 19; // t - k on the grid 2^-64
+    const uint32_t gh = (uint32_t)(g >> 32), gl = (uint32_t)g;
+    constexpr uint32_t ph = (uint32_t)(kPio2048Q73 >> 32), pl = (uint32_t)kPio2048Q73;
+    const uint64_t u = (uint64_t)gh * pl; // r 2^73, the product of the low words left out
+    const uint64_t R = (uint64_t)gh * ph + (u >> 32) + (((uint64_t)gl * ph + (uint32_t)u) >> 32);
+    const uint32_t rh = (uint32_t)(R >> 32);
+    const uint64_t z = (uint64_t)rh * rh + (((uint64_t)rh * (uint32_t)R) >> 31); // r^2 2^82
+    const uint32_t zh = (uint32_t)(z >> 32);                                     // r^2 2^50
+    const uint32_t v59 = __umulhi(rh, zh);                                       // r^3 2^59
+    const uint32_t u34 = kSixthQ34 - __umulhi(zh, kInv120Q16);                   // (1/6 - r^2/120) 2^34
+    const uint64_t sr = (R >> 9) - (((uint64_t)v59 * u34) >> 29);                // sin r 2^64
+    const uint64_t cm = (z >> 19) - __umulhi(__umulhi(zh, zh), kInv24Q28);       // (1 - cos r) 2^64
+    const ulonglong2 tq = __ldg(T.sincos_q + (k & (kSinTab - 1)));               // (S_j, C_j) 2^62
+    const int64_t s1 = (int64_t)(tq.x - umulhi_near(tq.x, cm) + umulhi_near(tq.y, sr));
+    const int64_t c1 = (int64_t)(tq.y - umulhi_near(tq.y, cm) - umulhi_near(tq.x, sr));
+    const bool odd = k & kSinTab;
+    const int64_t s = odd ? c1 : s1, c = odd ? s1 : c1;
+    s62 = ((k << 20) ^ (uint32_t)(b >> 32)) >> 31 ? -s : s; // k's half-turn bit and the sign of x
+    c62 = (k ^ (k << 1)) & (2 * kSinTab) ? -c : c;          // quarter turns 1 and 2
 }
 
 // v 2^-62 rounded onto the coarser grid 2^-F (F <= 61), half up.

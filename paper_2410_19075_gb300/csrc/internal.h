@@ -181,7 +181,7 @@ struct LatticePlan {
     int F;            // fixed-point grid of the window sums
     // ball, disk: the x pass rotates every node's (sin, cos) by -alpha =
     // -(rot_q pi/2 + alpha0), alpha0 in [0, pi/2): rot_c, rot_s = cos alpha0,
-    // sin alpha0 on the grid 2^-63 (lattice_rotated_q)
+    // sin alpha0 on the grid 2^-63, multiples of 4 (lattice_rotated_q)
     uint64_t rot_c, rot_s;
     int rot_q;
     ModelParams mp;

@@ -66,6 +66,12 @@ static int row_warps(int64_t N1)
 // prefix rows of a CTA round up to less of the SM (seven CTAs of four 464-node
 // rows, against three of eight).
 constexpr int kNodexWarpsMax = 4;
+// Shared memory's share of the L1 of the node pass, in percent of its maximum.  Left
+// to the driver, rows of 464 nodes take nearly all of it for seven CTAs per SM and
+// the sin/cos table misses: 9.93 ms per step, 9.52 with five CTAs and 92 KB of L1
+// (72%); edges 320, 200 and 101 lose 0.5% against the driver's choice, and 58% or 86%
+// are worse at 464.
+constexpr int kNodexCarveout = 72;
 // CTAs per SM the fused node pass is compiled for: six for Kuramoto (at most 80
 // registers, so stage 4 fits six too), five for the model with inertia.
 template <int M> constexpr int kNodexBlocks = M == 0 ? 6 : 5;
@@ -88,8 +94,10 @@ __device__ __forceinline__ void lattice_rotated_q(const LatticePlan &p, int64_t 
 {
     const int sh = 61 - p.F;
     const int64_t h = int64_t(1) << (sh - 1);
-    const int64_t c1 = (mulhi_su(c62, p.rot_c) + mulhi_su(s62, p.rot_s) + h) >> sh;
-    const int64_t s1 = (mulhi_su(s62, p.rot_c) - mulhi_su(c62, p.rot_s) + h) >> sh;
+    const uint64_t bs = biased62(s62), bc = biased62(c62);
+    const int64_t qc4 = (int64_t)(p.rot_c >> 2), qs4 = (int64_t)(p.rot_s >> 2);
+    const int64_t c1 = ((int64_t)(__umul64hi(bc, p.rot_c) + __umul64hi(bs, p.rot_s)) + (h - qc4 - qs4)) >> sh;
+    const int64_t s1 = ((int64_t)(__umul64hi(bs, p.rot_c) - __umul64hi(bc, p.rot_s)) + (h - qc4 + qs4)) >> sh;
     switch (p.rot_q) { // e^{-i q pi/2}: 1, -i, -1, i
     case 0: qc = c1; qs = s1; break;
     case 1: qc = s1; qs = -c1; break;
@@ -1022,6 +1030,8 @@ cudaError_t lattice_configure()
 #define SIM_NODEX_ATTR(M, S)                                                                                           \
     if (e == cudaSuccess)                                                                                              \
         e = cudaFuncSetAttribute(cube_nodex_kernel<M, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRowSmemMax); \
+    if (e == cudaSuccess)                                                                                              \
+        e = cudaFuncSetAttribute(cube_nodex_kernel<M, S>, cudaFuncAttributePreferredSharedMemoryCarveout, kNodexCarveout); \
     if (e == cudaSuccess && S > 0)                                                                                     \
         e = cudaFuncSetAttribute(cube_batch_nodex_kernel<M, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRowSmemMax);
     SIM_NODEX_ATTR(0, 0) SIM_NODEX_ATTR(0, 1) SIM_NODEX_ATTR(0, 2) SIM_NODEX_ATTR(0, 3) SIM_NODEX_ATTR(0, 4)

@@ -12,17 +12,17 @@ namespace simk {
 void fill_math_tables(double *block)
 {
     const long double pi = 3.141592653589793238462643383279502884L;
-    double *sincos = block, *exp2j = block + 2 * kSinTab;
-    int64_t *sincos_q = reinterpret_cast<int64_t *>(block + 2 * kSinTab + kExpTab);
+    double *exp2j = block + 2 * kSinTab;
+    uint64_t *sincos_q = reinterpret_cast<uint64_t *>(block);
     for (int j = 0; j < kSinTab; ++j) {
-        const long double a = pi * (long double)j / 512.0L;
-        sincos[2 * j] = (double)sinl(a);
-        sincos[2 * j + 1] = (double)cosl(a);
-        sincos_q[2 * j] = (int64_t)llroundl(sinl(a) * 4611686018427387904.0L); // 2^62
-        sincos_q[2 * j + 1] = (int64_t)llroundl(cosl(a) * 4611686018427387904.0L);
+        // the sines one unit low: fixed_sincos truncates what it subtracts, and near
+        // pi/2 its sum must not exceed 2^62
+        const long double a = pi * (long double)j / 2048.0L;
+        sincos_q[2 * j] = (uint64_t)llroundl(sinl(a) * 4611686018427387904.0L) - (j > 0 ? 1u : 0u); // 2^62
+        sincos_q[2 * j + 1] = (uint64_t)llroundl(cosl(a) * 4611686018427387904.0L);
     }
     for (int j = 0; j < kExpTab; ++j) exp2j[j] = (double)exp2l((long double)j / 64.0L);
-    uint64_t *exp2q = reinterpret_cast<uint64_t *>(block + 4 * kSinTab + kExpTab);
+    uint64_t *exp2q = reinterpret_cast<uint64_t *>(block + 2 * kSinTab + kExpTab);
     for (int j = 0; j < kExp2Tab; ++j) exp2q[j] = (uint64_t)rintl(exp2l((long double)j / 256.0L) * 9223372036854775808.0L); // 2^63
 }
 

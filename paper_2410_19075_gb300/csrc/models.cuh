@@ -26,7 +26,9 @@ struct ModelParams {
     double c[8];
     int64_t q[2];     // Kuramoto models: cos alpha and sin alpha on the grid 2^-62
     uint64_t a0[2];   // Kuramoto models: alpha = aq pi/2 + alpha0, alpha0 in [0, pi/2):
-    int aq;           //   cos alpha0, sin alpha0 on the grid 2^-63 (non-negative), aq in 0..3
+                      //   cos alpha0, sin alpha0 on the grid 2^-63 (non-negative multiples of 4)
+    int64_t at[2];    //   (a0[0] - a0[1]) / 4 and (a0[0] + a0[1]) / 4 (turned_by_alpha0)
+    int aq;           //   in 0..3
     int ksh;          // rings: right shift taking the exact window sums into int64
     uint64_t wsm;     // FHN and HH rings: wsize 2^(56 - ksh), for own_multiple
     int fx;           // FHN rings: 1 = the slope's bracket in integer arithmetic (kq, a54 in range)
@@ -58,6 +60,16 @@ __device__ __forceinline__ double lattice_coupling(const int64_t (&f62)[2], int6
     return __ll2double_rn(mulhi_ss(f62[1], W0) - mulhi_ss(f62[0], W1));
 }
 
+// e^{i alpha0} (c + i s) from the grid 2^-62 onto 2^-61: four high products of the
+// biased (s, c) with the non-negative cos alpha0, sin alpha0.  Each is short of its
+// floor by at most one (2^-61 of the node's phase, whose own error is 2^-53.6).
+__device__ __forceinline__ void turned_by_alpha0(const ModelParams &P, int64_t s, int64_t c, int64_t &s1, int64_t &c1)
+{
+    const uint64_t bs = biased62(s), bc = biased62(c);
+    c1 = (int64_t)(umulhi_near(bc, P.a0[0]) - umulhi_near(bs, P.a0[1])) - P.at[0];
+    s1 = (int64_t)(umulhi_near(bs, P.a0[0]) + umulhi_near(bc, P.a0[1])) - P.at[1];
+}
+
 // The node's own (sin, cos) on the grid 2^-62 turned by +alpha = aq pi/2 +
 // alpha0: e^{i alpha0} (c + i s) by four high products with the non-negative cos
 // alpha0, sin alpha0 (grid 2^-63, landing on 2^-61), back onto 2^-62 by one bit
@@ -67,10 +79,8 @@ __device__ __forceinline__ double lattice_coupling(const int64_t (&f62)[2], int6
 // cube; the ball and disk rotate their sums instead).
 __device__ __forceinline__ void own_phase_turned(const ModelParams &P, const int64_t (&f62)[2], int64_t (&t62)[2])
 {
-    const int64_t s = f62[0], c = f62[1];
-    const int64_t c1 = mulhi_su(c, P.a0[0]) - mulhi_su(s, P.a0[1]);
-    const int64_t s1 = mulhi_su(s, P.a0[0]) + mulhi_su(c, P.a0[1]);
-    int64_t ca, sa;
+    int64_t s1, c1, ca, sa;
+    turned_by_alpha0(P, f62[0], f62[1], s1, c1);
     switch (P.aq) { // times i^aq
     case 0: ca = c1; sa = s1; break;
     case 1: ca = -s1; sa = c1; break;
@@ -101,9 +111,8 @@ __device__ __forceinline__ int64_t ring_coupling(const ModelParams &P, const int
                                                  int64_t S_c)
 {
     const int64_t s = qo[0] * (int64_t(1) << (62 - F)), c = qo[1] * (int64_t(1) << (62 - F));
-    const int64_t c1 = mulhi_su(c, P.a0[0]) - mulhi_su(s, P.a0[1]); // e^{i alpha0} (c + i s), grid 2^-61
-    const int64_t s1 = mulhi_su(s, P.a0[0]) + mulhi_su(c, P.a0[1]);
-    int64_t ca, sa;
+    int64_t s1, c1, ca, sa;
+    turned_by_alpha0(P, s, c, s1, c1);
     switch (P.aq) { // times i^aq
     case 0: ca = c1; sa = s1; break;
     case 1: ca = -s1; sa = c1; break;

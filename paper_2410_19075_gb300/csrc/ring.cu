@@ -78,9 +78,11 @@ __device__ __forceinline__ void ring_stage_body(const RingPlan &P, const RingSta
 // independent right-hand sides per thread and one warp scan per node pair.  The
 // same integers and FP64 expressions as ring_stage_body, so the same bits.
 constexpr int kRing2Threads = kSubTile / 2;
-#ifndef SIM_RING2_MIN_BLOCKS
-#define SIM_RING2_MIN_BLOCKS 8
-#endif
+// Resident CTAs per SM the registers are sized for.  Kuramoto with inertia: 6 (80
+// registers) 27.1 us per RK4 step at 10^5 nodes, 8 (64, spilling) 29.3; the other
+// models lose 2% with 7.
+template <int M> struct Ring2MinBlocks { static constexpr int value = 8; };
+template <> struct Ring2MinBlocks<3> { static constexpr int value = 6; };
 
 template <int M, int STAGE>
 __device__ __forceinline__ void ring_stage_body2(const RingPlan &P, const RingStageIO &a, const StepSize &h,
@@ -180,7 +182,7 @@ __device__ __forceinline__ void ring_stage_body2(const RingPlan &P, const RingSt
 }
 
 template <int M, int STAGE>
-__global__ void __launch_bounds__(kRing2Threads, SIM_RING2_MIN_BLOCKS)
+__global__ void __launch_bounds__(kRing2Threads, Ring2MinBlocks<M>::value)
     ring_stage_kernel2(const RingPlan p, const StepSize h)
 {
     if (p.skip && *(const volatile int *)p.skip) return; // uniform over the launch
@@ -212,7 +214,7 @@ __global__ void __launch_bounds__(kRingThreads, MinBlocks<M>::value)
 
 // The same with two adjacent nodes per thread (ring_stage_body2).
 template <int M, int STAGE>
-__global__ void __launch_bounds__(kRing2Threads, SIM_RING2_MIN_BLOCKS)
+__global__ void __launch_bounds__(kRing2Threads, Ring2MinBlocks<M>::value)
     ring_batch_stage_kernel2(const RingPlan *__restrict__ plans, const int *__restrict__ inst_of_item,
                              const int64_t *__restrict__ item_base, const StepSize h)
 {

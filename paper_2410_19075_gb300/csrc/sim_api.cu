@@ -431,8 +431,10 @@ void simk::model_constants(int model, const double *params, double K, ModelParam
             const long double half_pi = 1.570796326794896619231321691639751442L;
             const long double a = (long double)alpha, q = floorl(a / half_pi), a0 = a - q * half_pi;
             const long double two63 = 9223372036854775808.0L;
-            mp.a0[0] = (uint64_t)roundl(fminl(fmaxl(cosl(a0), 0.0L), 1.0L) * two63);
-            mp.a0[1] = (uint64_t)roundl(fminl(fmaxl(sinl(a0), 0.0L), 1.0L) * two63);
+            mp.a0[0] = (uint64_t)roundl(fminl(fmaxl(cosl(a0), 0.0L), 1.0L) * two63 / 4) * 4;
+            mp.a0[1] = (uint64_t)roundl(fminl(fmaxl(sinl(a0), 0.0L), 1.0L) * two63 / 4) * 4;
+            mp.at[0] = (int64_t)(mp.a0[0] / 4) - (int64_t)(mp.a0[1] / 4);
+            mp.at[1] = (int64_t)(mp.a0[0] / 4) + (int64_t)(mp.a0[1] / 4);
             const long long qi = (long long)q % 4;
             mp.aq = (int)(qi < 0 ? qi + 4 : qi);
         }
@@ -500,8 +502,8 @@ void simk::lattice_rotation(LatticePlan &p, double alpha)
     const long double a0 = a - q * half_pi; // in [0, pi/2) up to rounding
     const long double c0 = cosl(a0), s0 = sinl(a0);
     const long double two63 = 9223372036854775808.0L;
-    p.rot_c = (uint64_t)roundl(fminl(fmaxl(c0, 0.0L), 1.0L) * two63); // <= 2^63
-    p.rot_s = (uint64_t)roundl(fminl(fmaxl(s0, 0.0L), 1.0L) * two63);
+    p.rot_c = (uint64_t)roundl(fminl(fmaxl(c0, 0.0L), 1.0L) * two63 / 4) * 4; // <= 2^63
+    p.rot_s = (uint64_t)roundl(fminl(fmaxl(s0, 0.0L), 1.0L) * two63 / 4) * 4;
     long long qi = (long long)q % 4;
     p.rot_q = (int)(qi < 0 ? qi + 4 : qi);
     // the cross product T lands on the grid 2^-(F-2): fold that scale into the coefficient
