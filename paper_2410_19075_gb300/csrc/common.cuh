@@ -266,6 +266,18 @@ __device__ i128 block_exclusive_scan(const T *in, i128 *out, int64_t n)
     return total;
 }
 
+// A batch member's plan (device memory) copied into shared memory by the whole CTA,
+// so that its fields cost one round trip to memory together and not one each where
+// they are first used; ends with a barrier.
+template <typename Plan> __device__ __forceinline__ void stage_plan(Plan &dst, const Plan *src)
+{
+    static_assert(sizeof(Plan) % 8 == 0, "copied in 8-byte words");
+    const unsigned long long *s = reinterpret_cast<const unsigned long long *>(src);
+    unsigned long long *d = reinterpret_cast<unsigned long long *>(&dst);
+    for (unsigned i = threadIdx.x; i < sizeof(Plan) / 8; i += blockDim.x) d[i] = __ldg(s + i);
+    __syncthreads();
+}
+
 // Called by one thread after it made its global writes visible (__threadfence).
 // Returns true for the last of `count` arrivals on a monotonically increasing
 // counter; the counter never needs resetting because every launch adds exactly

@@ -77,6 +77,7 @@ struct RingBatchGroup {
     const RingPlan *plans;  // n_inst plans (device)
     const int *inst_of_item; // n_items (device)
     const int64_t *item_base; // n_inst: first item of each member (device)
+    const long long *steps_left; // n_inst: the members' step budgets (device; plans[k].steps_left points at entry k)
     int npt;                  // nodes per thread of the batched stage kernels (1, or 2 if not HH)
 };
 

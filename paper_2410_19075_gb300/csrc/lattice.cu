@@ -578,8 +578,10 @@ __global__ void __launch_bounds__(kTileThreads)
                         const int64_t *__restrict__ yz_base)
 {
     extern __shared__ __align__(16) longlong2 tile_mem[];
+    __shared__ __align__(16) unsigned char plan_mem[sizeof(LatticePlan)];
+    LatticePlan &p = *reinterpret_cast<LatticePlan *>(plan_mem);
     const int inst = yz_item[blockIdx.x];
-    const LatticePlan &p = plans[inst];
+    stage_plan(p, plans + inst);
     int ib, k;
     cube_batch_tile(p, (int64_t)blockIdx.x - yz_base[inst], ib, k);
     cube_y_tile(p, ib, k, tile_mem);
@@ -677,8 +679,10 @@ __global__ void __launch_bounds__(kZThreads, kZBlocks)
                          const int64_t *__restrict__ yz_base)
 {
     extern __shared__ __align__(16) longlong2 tile_mem[];
+    __shared__ __align__(16) unsigned char plan_mem[sizeof(LatticePlan)];
+    LatticePlan &p = *reinterpret_cast<LatticePlan *>(plan_mem);
     const int inst = yz_item[blockIdx.x];
-    const LatticePlan &p = plans[inst];
+    stage_plan(p, plans + inst);
     int ib, j;
     cube_batch_tile(p, (int64_t)blockIdx.x - yz_base[inst], ib, j);
     cube_zw_tile<-1>(p, ib, j, tile_mem);
@@ -790,8 +794,11 @@ __global__ void __launch_bounds__(32 * kNodexWarpsMax, kNodexBlocks<M>)
                             const int64_t *__restrict__ x_base, const StepSize h)
 {
     extern __shared__ __align__(16) longlong2 row_mem[];
+    __shared__ __align__(16) unsigned char plan_mem[sizeof(LatticePlan)];
+    LatticePlan &p = *reinterpret_cast<LatticePlan *>(plan_mem);
     const int inst = x_item[blockIdx.x];
-    cube_nodex_cta<M, STAGE>(plans[inst], h, (int64_t)blockIdx.x - x_base[inst], row_mem);
+    stage_plan(p, plans + inst);
+    cube_nodex_cta<M, STAGE>(p, h, (int64_t)blockIdx.x - x_base[inst], row_mem);
 }
 
 // Order parameters of batched cubes, one CTA per member, from the partials of node

@@ -1367,6 +1367,7 @@ int sim_batch_create(sim_batch_t *out, const sim_t *members, int n_members, void
         g.plans = reinterpret_cast<const RingPlan *>(blk + o_plans) + gs.plan0;
         g.inst_of_item = reinterpret_cast<const int *>(blk + o_items) + gs.item0;
         g.item_base = reinterpret_cast<const int64_t *>(blk + o_base) + gs.plan0;
+        g.steps_left = b->budgets + gs.plan0;
         g.npt = gs.model == SIM_HH ? 1 : 2;
         TuneVal tv;
         if (gs.model != SIM_HH && tune_lookup(batch_tune_key(b, nitem), &tv)) g.npt = tv.npt == 1 ? 1 : 2;
