@@ -88,7 +88,8 @@ typedef enum {
 /* Creation flags. */
 #define SIM_FLAG_INCLUDE_SELF 1u /* count the node itself as one of its links */
 #define SIM_FLAG_STREAMING 2u    /* rings of <= 8192 nodes (HH 5120): use the multi-launch streaming
-                                    kernels instead of the thread-block-cluster kernel (same results) */
+                                    kernels instead of the thread-block-cluster kernels, for RK4 and for
+                                    Dormand-Prince runs (same results) */
 #define SIM_FLAG_LOW_MEMORY 4u   /* ball lattices: keep one periodically extended row prefix (about
                                     16 B per node, what disks always keep) instead of one x-window
                                     array per chord half-width ((P+1) * 16 B per node, the default
@@ -160,7 +161,8 @@ int sim_set_state_device(sim_t h, const double *dev_soa, int64_t n_values);
 int sim_set_node_param(sim_t h, int which, const double *host, int64_t n);
 
 /* Advance the network by n_steps classic RK4 steps of size dt (asynchronous on
- * the handle's stream; launched as a captured CUDA graph).  dt > 0.
+ * the handle's stream; launched as captured CUDA graphs, or for rings in a
+ * thread-block cluster as one kernel per 4096 steps).  dt > 0.
  * Errors from the device (SIM_ETIMEOUT, SIM_ENONFINITE) surface at the next
  * synchronising call. */
 int sim_step(sim_t h, int64_t n_steps, double dt);
@@ -248,7 +250,8 @@ typedef struct {
 /* One network.  Returns SIM_OK, the run's SIM_ESTEPS / SIM_ESMALL (the state is
  * then that of the last accepted step, stats->t), SIM_EINVAL (invalid options),
  * SIM_ENOMEM, or a device error.  stats may be NULL.  Synchronises the handle's
- * stream.  A ring run uses fused Dormand-Prince stage kernels; a lattice or
+ * stream.  A ring run uses fused Dormand-Prince stage kernels (small rings: one
+ * kernel per 256 attempts, inside a thread-block cluster); a lattice or
  * link-matrix run evaluates each stage with the network's own right-hand-side
  * kernels from a stage-input buffer. */
 int sim_dp5(sim_t h, const sim_dp5_opts *opts, sim_dp5_stats *stats);
@@ -444,9 +447,10 @@ int sim_ring_step_noalloc(int model, int64_t N, int64_t radius, const double *pa
 
 /* Evaluate the library's device elementary functions on n arguments (host
  * buffers; synchronous), for accuracy checks: fn 0 = sin, 1 = cos, 2 = exp,
- * 3 = reciprocal 1/x, 4 = x / (1 - exp(-x)).  These are the table-driven FP64
- * routines the node right-hand sides use (Kuramoto phases, Hodgkin-Huxley
- * rates of Eq. (1)).  Allocates and frees its own device buffers. */
+ * 3 = reciprocal 1/x, 4 = x / (1 - exp(-x)).  sin and cos are the integer
+ * routine that the Kuramoto right-hand sides use, the others table-driven FP64
+ * (the Hodgkin-Huxley rates of Eq. (1) use integer forms of them).  Allocates and
+ * frees its own device buffers. */
 int sim_math_eval(int fn, const double *host_x, double *host_out, int64_t n);
 
 /* Measured peak rate of one arithmetic pipe of the current device, for roofline

@@ -3,7 +3,9 @@
 // GB300 retires about 2 FP64 lanes per clock per SM, against 64 lanes of 32-bit
 // integer arithmetic and 128 of FP32.  The routines below keep every FP64
 // instruction that the result's accuracy needs and move the rest to the
-// integer and FP32 pipes; sin and cos need none at all.
+// integer and FP32 pipes; sin and cos need none at all.  The Hodgkin-Huxley rates
+// take the integer forms of exp and the quotients in hh_rates.cuh; exp and 1/d here
+// serve sim_math_eval.
 //
 // Methods (textbook; constants derived for this code from pi and ln 2 in
 // high-precision arithmetic):

@@ -1,6 +1,7 @@
 """Edges of the ball's and disk's gather: blocks of one, two and four nodes per
 thread (lattice edges 48 and 72 for balls, 400 for disks), ragged blocks, windows as
-wide as the lattice, more reads than one table chunk, window arrays and row prefixes."""
+wide as the lattice, more reads than one table chunk, window arrays and row prefixes.
+Edges of the cube's tiles, alone and in a batch."""
 import numpy as np
 import pytest
 
@@ -54,3 +55,42 @@ def test_gather_blocks(topo, N, P, model):
             k.append(net.rhs())
     y = y0 + 0.01 / 6.0 * (k[0] + 2.0 * k[1] + 2.0 * k[2] + k[3])
     assert np.abs(y1 - y).max() < 1e-14
+
+
+@pytest.mark.parametrize("model", [0, 3])
+def test_cube_tiles(model):
+    """Cubes around the edges of their tiles (16 columns up to edge 297, 8 above), windows
+    from the smallest to the whole edge: slopes at sampled nodes against the oracle, and
+    all of them in one batch, small and large tiles in the same launches, against the
+    same steps alone, bit for bit."""
+    from paper_2410_19075_gb300 import Batch, Network
+    params = I.ks_params(alpha=1.3) if model == 0 else I.ksi_params(mu=1.0)
+    cubes = [(3, 1), (16, 7), (17, 8), (31, 15), (33, 2), (113, 1), (297, 2), (298, 3), (305, 1)]
+    rng = np.random.default_rng(5 + model)
+    ys, alone, nets = [], [], []
+    for N, P in cubes:
+        n = N ** 3
+        y0 = np.concatenate([rng.uniform(-3.1, 3.1, n)] + ([rng.uniform(-0.1, 0.1, n)] if model == 3 else []))
+        ys.append(y0)
+        with Network(model, 1, N, P, params) as net:
+            net.set_state(y0)
+            k1 = net.rhs()
+            net.step(2, 0.01)
+            alone.append((net.get_state(), net.observables()))
+        edge = [0, 1, N - 2, N - 1]
+        q = np.unique([(z * N + j) * N + i for z in edge for j in edge for i in edge])
+        # window sums: exact but for the rounding onto 2^-F, 1e-13 as for the other lattices
+        assert np.abs(k1.reshape(-1, n)[:, q] - oracle.rhs_sampled(model, 1, N, P, params, y0, q)).max() < 1e-13
+    try:
+        for (N, P), y0 in zip(cubes, ys):
+            nets.append(Network(model, 1, N, P, params))
+            nets[-1].set_state(y0)
+        with Batch(nets) as batch:
+            batch.step(2, 0.01)
+            batch.sync()
+        for net, (y, order) in zip(nets, alone):
+            assert np.array_equal(net.get_state(), y)
+            assert np.array_equal(net.observables(), order)
+    finally:
+        for net in nets:
+            net.close()

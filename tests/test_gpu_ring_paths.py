@@ -1,5 +1,6 @@
 """Edges of the ring kernels' dispatch rules: the cluster-resident kernel's slice
-sizes, and the FitzHugh-Nagumo slope in integer or FP64 arithmetic."""
+sizes, and the FitzHugh-Nagumo slope in integer or FP64 arithmetic; the sine's
+reduction edges."""
 import numpy as np
 import pytest
 
@@ -98,3 +99,23 @@ def test_link_matrix_prefix_forms(model, N):
         net.close()
     for a, b in zip(*outs):
         assert np.abs(np.asarray(a) - np.asarray(b)).max(initial=0.0) < 1e-12 * max(1.0, np.abs(outs[0][0]).max())
+
+
+@pytest.mark.parametrize("sign", [-1.0, 1.0])
+def test_sincos_reduction_edges(sign):
+    """sin and cos next to every point where the reduction changes its table entry or
+    quadrant.  The routine's error is below 2^-53.6 and its conversion rounds by 2^-54,
+    numpy's rounds by 2^-54: 2e-16 in all."""
+    from paper_2410_19075_gb300.sim import math_eval
+    j = np.concatenate([np.arange(0, 4 * 1024 + 2), np.arange(0, 166800, 1024), [166885, 166886]])
+    x = [j * (np.pi / 2048)]
+    for d in (np.inf, -np.inf):
+        e = x[0]
+        for _ in range(3):
+            e = np.nextafter(e, d)
+            x.append(e)
+    x = sign * np.concatenate(x)
+    x = x[np.abs(x) < 256]
+    s, c = math_eval(0, x), math_eval(1, x)
+    assert np.abs(s - np.sin(x)).max() < 2e-16 and np.abs(c - np.cos(x)).max() < 2e-16
+    assert np.abs(s).max() <= 1.0 and np.abs(c).max() <= 1.0
