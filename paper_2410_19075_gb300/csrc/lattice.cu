@@ -42,8 +42,10 @@ constexpr int kGatherThreads = 128;   // ball/disk gather: a block of rows x pla
 constexpr int kGatherOps = 512;       // ball/disk gather: reads of the window held in shared memory at a time
 constexpr size_t kRowSmemMax = 220 * 1024;
 
-// i-columns per tile: shared memory (N1 + 1) BI 16 bytes stays below ~76 KB
-// (two or three CTAs per SM) and every row segment of a load is BI * 8 bytes.
+// i-columns per tile: shared memory (N1 + 1) BI 16 bytes stays below ~76 KB, so that
+// three CTAs fit on an SM; the widest such tile pads least and keeps a window pass's
+// own (sin, cos) in segments of BI 16 bytes (8 columns where 16 fit: 165 us per step
+// against 151 at 101^3, 907 against 867 at 200^3).
 __host__ __device__ inline int cube_tile_lg(int64_t N1) { return N1 <= 297 ? 4 : N1 <= 594 ? 3 : 2; }
 __host__ __device__ inline int cube_tile_bi(int64_t N1) { return 1 << cube_tile_lg(N1); }
 
@@ -630,7 +632,10 @@ __device__ __forceinline__ void lattice_write_coupling(const LatticePlan &p, int
 // consecutive nodes.  Three window CTAs per SM at the tile sizes of N1 <= 594.
 // At 464^3 (interleaved (sin, cos) pairs): two planes per unrolled iteration
 // with three planes of prefetch 0.826 ms, two planes of prefetch 0.831 ms, one
-// plane per iteration 0.860 ms; 512 threads (at most 42 registers) 0.884 ms.
+// plane per iteration 0.860 ms; 512 threads (at most 42 registers) 0.884 ms.  With
+// pairs in the tile too: 0.766 ms.  256 threads and four CTAs per SM take 9.72 ms per
+// step against 9.51 at 464^3 (only three fit), 2.70 against 2.77 at 300^3 and 0.859
+// against 0.867 at 200^3.
 constexpr int kZThreads = 384, kZAhead = 3, kZBlocks = 3; // kZAhead: planes of own (sin, cos) in flight
 
 template <int KM> // -1: coupling terms; a model: the slopes of a right-hand-side evaluation
