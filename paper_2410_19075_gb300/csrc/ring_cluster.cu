@@ -50,6 +50,7 @@ __global__ void __launch_bounds__(kClusterThreadsMax, 1)
     constexpr int D = Mo::D, NQ = Mo::NQ, NX = Mo::NX, XOFF = D - NX;
     constexpr bool KURAMOTO = M == 0 || M == 3;
     cg::cluster_group cluster = cg::this_cluster();
+    cluster.barrier_arrive(); // the CTA runs: the others may store into its shared memory (publish)
     const int rank = (int)cluster.block_rank(), CL = (int)cluster.num_blocks();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = (int)(blockDim.x >> 5) - 1; // node warps
     const int N = (int)P.N, R = (int)P.R, sh = P.mp.ksh;
@@ -133,6 +134,7 @@ __global__ void __launch_bounds__(kClusterThreadsMax, 1)
         }
     };
 
+    cluster.barrier_wait(); // every CTA has started (a store into one that has not is undefined)
     // f(y) into buffer 0 (the observable of y was recorded when the state was set)
     publish(0);
     int cur = 0; // buffer holding f of the current stage input

@@ -73,6 +73,7 @@ __global__ void __launch_bounds__(DpShape<M>::NT, 2)
     if (tid == 0) s_ctl = *Q.ctl;
     __syncthreads();
     if (s_ctl.done && !first) return; // the whole cluster: every CTA reads the same word
+    if constexpr (!ONE) cluster.barrier_arrive(); // the CTA runs: the others may store into its shared memory (publish)
     if (tid == 0) s_bad = 0;
     for (int q = tid; q < kDpMaxOut * 4; q += nt) (&s_out[0][0][0])[q] = 0ull;
 
@@ -217,6 +218,7 @@ __global__ void __launch_bounds__(DpShape<M>::NT, 2)
         publish(cur);
     };
 
+    if constexpr (!ONE) cluster.barrier_wait(); // every CTA has started (a store into one that has not is undefined)
     if (first) { // R(t0), k1 = f(y_n)
         publish_y();
         SliceOffsets<NQ> o;
