@@ -127,11 +127,11 @@ __global__ void __launch_bounds__(kClusterThreadsMax, 1)
             v[1] = w.y;
         } else v[0] = *p;
     };
-    auto record_order = [&](const SliceOffsets<NQ> &o) { // the recording warp of CTA 0
-        if (KURAMOTO && rank == 0 && lane == 0) {
-            ring_record_order(P, ((i128)o.tot_hi[0] << sh) + o.tot_lo[0],
-                              ((i128)o.tot_hi[NQ - 1] << sh) + o.tot_lo[NQ - 1]);
-        }
+    auto record_order = [&](int b) { // R from buffer b's totals, by the recording warp of CTA 0
+        if (!KURAMOTO || rank != 0) return;
+        i128 t[NQ];
+        ring_total<NQ>(s_tot[b], CL, t);
+        if (lane == 0) ring_record_order(P, t[0], t[NQ - 1]);
     };
 
     cluster.barrier_wait(); // every CTA has started (a store into one that has not is undefined)
@@ -172,9 +172,7 @@ __global__ void __launch_bounds__(kClusterThreadsMax, 1)
                     Mo::coupled_q(P.mp, xn, P.F, P.lim, ok, qn);
                 }
             } else if (KURAMOTO && stage == 1 && step > 0) { // R of y after the previous step
-                SliceOffsets<NQ> o;
-                slice_offsets<NQ>(s_tot[cur], CL, sh, o);
-                record_order(o);
+                record_order(cur);
             }
             cur ^= 1;
             publish(cur);
@@ -182,37 +180,14 @@ __global__ void __launch_bounds__(kClusterThreadsMax, 1)
     }
     if (!ok) raise_error(P.err, ERR_RANGE);
 
-    // results: y, the last order parameter, and the streaming path's two-level
-    // prefix of f(y) (buffer 0): lam256(i) = P(i + 1) - P(start of i's 256-node
-    // sub-tile), the start's prefix read like a window end at e = start - 1
-    SliceOffsets<NQ> o;
-    slice_offsets<NQ>(s_tot[cur], CL, sh, o);
-    if (recorder && n_steps > 0) record_order(o);
-    if (!recorder) {
-        const int e = (i & ~(kSubTile - 1)) - 1, re = live && e >= 0 ? e / per : 0; // e < 0: prefix 0
-        int64_t hs[NQ], hi[NQ];
-        int los[NQ], lo[NQ];
-        slice_base<NQ>(o, re, 0, hs, los);
-        slice_base<NQ>(o, rank, 0, hi, lo);
-        if (live) {
-            const int64_t *ps = cluster.map_shared_rank(lam, re) + (cur * per + (e >= 0 ? e - re * per : 0)) * NQ;
-            const int64_t *pi = lam + (cur * per + tid) * NQ;
-            const int sub = i >> kSubLog2;
+    // results: y, the last order parameter, and the streaming path's two-level prefix of f(y)
+    if (recorder && n_steps > 0) record_order(cur);
+    if (live) {
+        const int e = (i & ~(kSubTile - 1)) - 1, re = e >= 0 ? e / per : 0;
+        const int64_t *ps = e >= 0 ? cluster.map_shared_rank(lam, re) + (cur * per + e - re * per) * NQ : nullptr;
 #pragma unroll
-            for (int v = 0; v < D; ++v) P.y[(int64_t)v * N + i] = y[v];
-#pragma unroll
-            for (int c = 0; c < NQ; ++c) {
-                const i128 start = e >= 0 ? ((i128)hs[c] << sh) + los[c] + ps[c] : (i128)0;
-                const i128 here = ((i128)hi[c] << sh) + lo[c] + pi[c];
-                P.lam[0][(int64_t)i * NQ + c] = (int64_t)(here - start);
-                // one prefix group (at most 32 sub-tiles): in-group offsets are the sub-tile starts
-                if (!(i & (kSubTile - 1))) st_i128(P.ingrp[0] + c * P.nsub + sub, start);
-                if (i == 0) {
-                    st_i128(P.grpofs[0] + c * (P.ngroups + 1), 0);
-                    st_i128(P.grpofs[0] + c * (P.ngroups + 1) + 1, ((i128)o.tot_hi[c] << sh) + o.tot_lo[c]);
-                }
-            }
-        }
+        for (int v = 0; v < D; ++v) P.y[(int64_t)v * N + i] = y[v];
+        slice_store_prefix<NQ>(P, s_tot[cur], CL, i, rank, lam + (cur * per + tid) * NQ, re, ps);
     }
     cluster.sync(); // no CTA exits while others may still read its shared memory
 }

@@ -223,9 +223,10 @@ __global__ void __launch_bounds__(DpShape<M>::NT, 2)
         publish_y();
         SliceOffsets<NQ> o;
         offsets(o);
-        if (KURAMOTO && rank == 0 && tid == 0 && P.obs) {
-            ring_record_order(P, ((i128)o.tot_hi[0] << sh) + o.tot_lo[0],
-                              ((i128)o.tot_hi[NQ - 1] << sh) + o.tot_lo[NQ - 1]);
+        if (KURAMOTO && rank == 0 && warp == 0 && P.obs) {
+            i128 t[NQ];
+            ring_total<NQ>(s_tot[cur], CL, t);
+            if (lane == 0) ring_record_order(P, t[0], t[NQ - 1]);
         }
         if (!s_ctl.done) {
 #pragma unroll
@@ -391,36 +392,18 @@ __global__ void __launch_bounds__(DpShape<M>::NT, 2)
     // results: y, k1 and the controls for a next launch, and the two-level prefix of
     // f(y) the other kernels read (buffer 0), as in ring_cluster.cu
     publish_y();
-    SliceOffsets<NQ> o;
-    offsets(o);
 #pragma unroll
     for (int m = 0; m < MPT; ++m) {
         int l;
-        const bool live = local(m, l);
-        const int i = i0 + l, e = (i & ~(kSubTile - 1)) - 1, re = live && e >= 0 ? e / per : 0; // e < 0: prefix 0
-        int64_t hs[NQ], hi[NQ];
-        int los[NQ], lo[NQ];
-        base(o, re, 0, hs, los);
-        base(o, rank, 0, hi, lo);
-        if (!live) continue;
-        const int64_t *ps = at(lam, re) + (cur * per + (e >= 0 ? e - re * per : 0)) * NQ;
-        const int64_t *pi = lam + (cur * per + l) * NQ;
+        if (!local(m, l)) continue;
+        const int i = i0 + l, e = (i & ~(kSubTile - 1)) - 1, re = e >= 0 ? e / per : 0;
+        const int64_t *ps = e >= 0 ? at(lam, re) + (cur * per + e - re * per) * NQ : nullptr;
 #pragma unroll
         for (int v = 0; v < D; ++v) {
             Q.ybuf[0][(int64_t)v * N + i] = ys[v * per + l];
             Q.k[0][(int64_t)v * N + i] = ks[v * per + l];
         }
-#pragma unroll
-        for (int c = 0; c < NQ; ++c) {
-            const i128 start = e >= 0 ? ((i128)hs[c] << sh) + los[c] + ps[c] : (i128)0;
-            const i128 here = ((i128)hi[c] << sh) + lo[c] + pi[c];
-            P.lam[0][(int64_t)i * NQ + c] = (int64_t)(here - start);
-            if (!(i & (kSubTile - 1))) st_i128(P.ingrp[0] + c * P.nsub + (i >> kSubLog2), start);
-            if (i == 0) {
-                st_i128(P.grpofs[0] + c * (P.ngroups + 1), 0);
-                st_i128(P.grpofs[0] + c * (P.ngroups + 1) + 1, ((i128)o.tot_hi[c] << sh) + o.tot_lo[c]);
-            }
-        }
+        slice_store_prefix<NQ>(P, s_tot[cur], CL, i, rank, lam + (cur * per + l) * NQ, re, ps);
     }
     if (rank == 0 && tid == 0) {
         s_ctl.cur = 0; // y_n and k1 are in the first buffers
