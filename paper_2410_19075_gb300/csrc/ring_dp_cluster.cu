@@ -30,6 +30,11 @@ template <int M> struct DpShape { static constexpr int NT = 512, MPT = M == 0 ? 
 template <> struct DpShape<2> { static constexpr int NT = 256, MPT = 1; };
 static int dp_slice(int model) { return model == 0 ? 1024 : model == 2 ? 256 : 512; } // NT * MPT
 
+// Nodes of a CTA at most: a slice's prefix stays below 2^63 in magnitude.  The Kuramoto
+// models' |q| reaches 2^53 (a sine or cosine of exactly 1), so 1024 coherent nodes would
+// wrap; the others' |q| stays below 2^54 and their slices hold 512.
+static int dp_slice_nodes(int model) { return model == 0 ? 1023 : dp_slice(model); }
+
 constexpr int kDpClusterNodes = 8192; // 32 sub-tiles: one lane each in the error sum
 
 template <int M> static size_t dp_cluster_smem(int per)
@@ -418,8 +423,12 @@ int dp_cluster_size(int model, int64_t N, int n_rings)
 {
     const int maxc = cluster_max_ctas(), slice = dp_slice(model);
     if (N > kDpClusterNodes) return 0;
+    auto fits = [&](int cl) {
+        const int64_t per = ((N + cl - 1) / cl + 31) / 32 * 32; // the kernel's slices, all but the last one full
+        return per <= slice && std::min(per, N) <= dp_slice_nodes(model);
+    };
     int cl = 1;
-    while ((int64_t)cl * slice < N) cl *= 2;
+    while (cl <= maxc && !fits(cl)) cl *= 2;
     if (cl > maxc) return 0;
     while (cl * 2 <= maxc && (int64_t)n_rings * cl * 2 <= 304 && N / (2 * cl) >= 96) cl *= 2;
     return cl;

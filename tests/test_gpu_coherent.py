@@ -55,3 +55,26 @@ def test_order_parameter_of_coherent_rings(N, R, phase, spread, model, dp5):
     assert abs(order[1] - R0) < 1e-2  # 0.01 time units on (Dormand-Prince: the run's own R(t0))
     if spread == 0.0:  # identical nodes stay identical
         assert np.abs(order - 1.0).max() < 1e-12
+
+
+@pytest.mark.parametrize("n_rings,N,R", [(200, 1024, 350), (200, 1023, 350), (200, 1000, 7), (160, 2048, 128), (24, 8192, 700),
+                                         (24, 7937, 700)])
+@pytest.mark.parametrize("model,phase", [(0, 0.0), (0, np.pi / 2), (3, 0.0)])
+def test_batched_dormand_prince_of_rings_in_phase(model, phase, n_rings, N, R):
+    """Batches large enough that a CTA takes as many nodes as it can, every node's sine or
+    cosine exactly 2^53 on its grid: the streaming kernels' bits."""
+    from paper_2410_19075_gb300 import Batch
+    y0 = _state(model, N, phase, 0.0)
+    opts = dict(t_end=0.3, rtol=1e-7, atol=1e-8, h0=0.1, out_dt=0.1)
+    outs = []
+    for n, streaming in ((n_rings, False), (1, True)):
+        nets = [_net(model, N, R, y0, streaming) for _ in range(n)]
+        with Batch(nets) as batch:
+            stats = batch.dp5([opts] * n)
+        outs.append([(st, net.get_state(), net.observables()) for st, net in zip(stats, nets)])
+        for net in nets:
+            net.close()
+    st, y, order = outs[1][0]
+    assert np.abs(order - 1.0).max() < 1e-12
+    for got in outs[0]:
+        assert got[0] == st and np.array_equal(got[1], y) and np.array_equal(got[2], order)
