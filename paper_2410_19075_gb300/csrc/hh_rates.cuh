@@ -92,10 +92,12 @@ __device__ __forceinline__ UFloat uf_rcp(const UFloat &a)
     return UFloat{y << 1, -a.e - 1};
 }
 
-// Nearest double (the values here lie far inside its exponent range).
+// Nearest double (the values here lie far inside its exponent range).  The rounding bit is
+// added after the shift: m + 1024 wraps for m within 1024 of 2^64, where the carry has to
+// reach the exponent.
 __device__ __forceinline__ double uf_double(const UFloat &a)
 {
-    return __longlong_as_double((long long)(((uint64_t)(int64_t)(a.e + 1022) << 52) + ((a.m + 1024) >> 11)));
+    return __longlong_as_double((long long)(((uint64_t)(int64_t)(a.e + 1022) << 52) + (a.m >> 11) + ((a.m >> 10) & 1)));
 }
 
 struct HHRates {
