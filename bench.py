@@ -54,7 +54,7 @@ RING_BYTES = {0: 344, 1: 432, 2: 704, 3: 480}
 # and the RK4 updates (13 per state variable: FMA, 2 FMA, 2 FMA, ADD + FMA).
 # Sine and cosine, the FitzHugh-Nagumo bracket and the Hodgkin-Huxley rates run in
 # integer arithmetic (no FP64).
-RING_FLOPS = {0: 4 * 5 + 13, 1: 4 * 3 + 2 * 13, 2: 4 * 28 + 3 * 16 + 12, 3: 4 * 6 + 2 * 13}
+RING_FLOPS = {0: 4 * 5 + 13, 1: 4 * 3 + 2 * 13, 2: 4 * 31 + 3 * 16 + 12, 3: 4 * 6 + 2 * 13}
 # Cube (Kuramoto), bytes per node of each pass (launch): y pass reads the x
 # sums and writes the xy sums (16 + 16); z-window pass reads the xy sums (16) and
 # the node's own (sin, cos) (16) and writes the coupling term (8); the node pass,

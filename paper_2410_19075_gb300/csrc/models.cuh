@@ -267,7 +267,7 @@ template <> struct Model<1> {
 //   dx/dt    = alpha_x(V) (1-x) - beta_x(V) x,   x in {m, h, n}
 // with CV = sum_{j in W(i)} (V_j - V_i) = W_V - wsize * Q(V_i), exact in fixed point.
 // c = {1/Cm, gNa, gK, gL, ENa, EK, EL, g/K}.  Coupled quantity V; the gates are
-// local variables.  The rates come from integer arithmetic (hh_rates.cuh); 31
+// local variables.  The rates come from integer arithmetic (hh_rates.cuh); 34
 // FP64 instructions per node are left.
 template <> struct Model<2> {
     static constexpr int D = 4, NQ = 1, NX = 3, F = 46;
@@ -299,9 +299,14 @@ template <> struct Model<2> {
         const double I = Iext - P.c[1] * m3h * (V - P.c[4]) - P.c[2] * n4 * (V - P.c[5]) -
                          P.c[3] * (V - P.c[6]) + P.c[7] * CV;
         k[0] = I * P.c[0];
-        k[1] = fma(-(r.am + r.bm), m, r.am); // alpha (1 - x) - beta x
-        k[2] = fma(-(r.ah + r.bh), h, r.ah);
-        k[3] = fma(-(r.an + r.bn), n, r.an);
+        // alpha (1 - x) - beta x, as it stands: from x = 1/2 on 1 - x is exact, and a gate near 1
+        // keeps the relative accuracy of its slope.  alpha - (alpha + beta) x, one FP64
+        // instruction less per gate, had 3.5 times the rms error at x in (0.95, 1) and took
+        // 282 us per RK4 step at 10^6 neurons, this takes 305 (48.6 and 51.4 at 10^5); the sum
+        // in integer arithmetic with the smaller of x and 1 - x: 306 and 51.1.
+        k[1] = fma(r.am, 1.0 - m, -(r.bm * m));
+        k[2] = fma(r.ah, 1.0 - h, -(r.bh * h));
+        k[3] = fma(r.an, 1.0 - n, -(r.bn * n));
     }
 };
 
