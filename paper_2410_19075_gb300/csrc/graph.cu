@@ -18,8 +18,6 @@
 // the pieces the CTA's run ends fall in is computed once per CTA, so a run costs
 // a node one load per end and component.  The degree of the node (its link
 // count, which normalises the coupling) comes with its entry.
-#include <mutex>
-
 #include "ring_parts.cuh"
 
 namespace simk {
@@ -238,16 +236,16 @@ __global__ void __launch_bounds__(kRingThreads, GraphMinBlocks<M>::value)
 // static bases and dynamic table together pass 48 KB
 template <int M> static cudaError_t configure()
 {
-    static std::once_flag once;
-    static cudaError_t err = cudaSuccess;
-    std::call_once(once, [] {
+    static PerDevice<cudaError_t> done;
+    return done.get(current_device(), [] {
+        cudaError_t err = cudaSuccess;
         const int bytes = (int)(sizeof(i128) * Model<M>::NQ * kGraphTab);
         const void *k[] = {(const void *)graph_stage_kernel<M, 1, true>, (const void *)graph_stage_kernel<M, 2, true>,
                            (const void *)graph_stage_kernel<M, 3, true>, (const void *)graph_stage_kernel<M, 4, true>};
         for (const void *f : k)
             if (err == cudaSuccess) err = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+        return err;
     });
-    return err;
 }
 
 template <int M, bool FLAT>

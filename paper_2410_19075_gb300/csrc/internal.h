@@ -6,8 +6,16 @@
 
 #include "common.cuh"
 #include "models.cuh"
+#include "per_device.h"
 
 namespace simk {
+
+inline int current_device()
+{
+    int d = 0;
+    cudaGetDevice(&d);
+    return d;
+}
 
 constexpr int kRingThreads = 256;       // threads per CTA, one node each
 constexpr int kSubTile = 256;           // nodes per CTA = exact-prefix sub-tile
@@ -248,7 +256,7 @@ cudaError_t lat_dp_attempt(const LatDpPlan &d, cudaStream_t s);   // one attempt
 cudaError_t graph_dp_start(const GraphDpPlan &d, cudaStream_t s);
 cudaError_t graph_dp_attempt(const GraphDpPlan &d, cudaStream_t s);
 
-cudaError_t lattice_configure(); // once per process, before the first launch
+cudaError_t lattice_configure(); // once per device, before the first launch
 int64_t cube_tiles(int64_t N1);     // CTAs of a cube's y and z-window passes
 int cube_node_warps(int64_t N1);    // rows per CTA of a cube's node pass
 size_t cube_batch_tile_smem(int64_t N1); // shared bytes of its y and z-window CTAs

@@ -14,7 +14,6 @@
 // then the ring) and the controller are those of dp5.cu: the same bits, whatever
 // the cluster's size.
 #include <algorithm>
-#include <mutex>
 
 #include <cooperative_groups.h>
 
@@ -438,13 +437,13 @@ template <int M, bool ONE>
 static cudaError_t launch_shape(const DpPlan *plans, int n, int cl, int64_t n_max, int max_attempts, int first, cudaStream_t s)
 {
     const int per = (int)(((n_max + cl - 1) / cl + 31) / 32 * 32); // of the largest ring of the launch
-    static std::once_flag once;
-    static cudaError_t err = cudaSuccess;
-    std::call_once(once, [] {
-        err = cudaFuncSetAttribute(ring_dp_cluster_kernel<M, ONE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    static PerDevice<cudaError_t> done;
+    const cudaError_t err = done.get(current_device(), [] {
+        cudaError_t err = cudaFuncSetAttribute(ring_dp_cluster_kernel<M, ONE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                    (int)dp_cluster_smem<M>(dp_slice(M)));
         if (err == cudaSuccess)
             err = cudaFuncSetAttribute(ring_dp_cluster_kernel<M, ONE>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        return err;
     });
     if (err != cudaSuccess) return err;
     cudaLaunchConfig_t cfg = {};

@@ -512,10 +512,8 @@ void simk::lattice_rotation(LatticePlan &p, double alpha)
 
 static cudaError_t ensure_cluster_configured()
 {
-    static std::once_flag once;
-    static cudaError_t err = cudaSuccess;
-    std::call_once(once, [] { err = ring_cluster_configure(); });
-    return err;
+    static PerDevice<cudaError_t> done;
+    return done.get(current_device(), ring_cluster_configure);
 }
 
 extern "C" {
@@ -683,10 +681,8 @@ static int create_impl(sim_t *out, int model, int topology, int64_t N, int64_t r
             e = cudaMemcpyAsync(b + L.chords, h->gather_ops.data(), sizeof(int4) * h->gather_ops.size(),
                                 cudaMemcpyHostToDevice, h->stream);
         }
-        static std::once_flag lat_once;
-        static cudaError_t lat_err = cudaSuccess;
-        std::call_once(lat_once, [] { lat_err = lattice_configure(); });
-        if (e == cudaSuccess) e = lat_err;
+        static PerDevice<cudaError_t> lat_done;
+        if (e == cudaSuccess) e = lat_done.get(current_device(), lattice_configure);
         if (e != cudaSuccess) {
             sim_destroy(h);
             return cuda_fail(e, "lattice set-up");
