@@ -4,6 +4,7 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "cluster_size.h"
 #include "common.cuh"
 #include "models.cuh"
 #include "per_device.h"
@@ -159,20 +160,16 @@ cudaError_t dp_launch(int ds, const DpGroup &g, cudaStream_t s);
 // Small rings: attempts of each ring's run inside one cluster (ring_dp_cluster.cu), at
 // most max_attempts per launch; first = 1 also records R(t0) and computes k1.  Every
 // launch leaves y in ybuf[0], k1 in k[0] and the two-level prefix of f(y).
-int dp_cluster_size(int model, int64_t N, int n_rings); // CTAs per ring (0: dp_launch's kernels)
+int dp_largest_cluster(int model); // sets its kernels' attributes; by cluster_limits
 cudaError_t dp_cluster_launch(int model, const DpPlan *plans, int n, int cl, int64_t n_max, int max_attempts, int first,
                               cudaStream_t s);
 
 // Ring: f(y) -> lam[0], ofs[0] and the order parameter of y (Kuramoto).
 cudaError_t ring_prologue(const RingPlan &p, cudaStream_t s);
-// Small rings (N <= kClusterMaxNodes, HH kClusterMaxNodesHH): all stages of n_steps
-// RK4 steps in one thread-block-cluster launch (ring_cluster.cu).  Same results
-// as ring_step.  Per RK4 step, cluster against streaming kernels: KS 10.2 / 21.8 us
-// at N = 5000 and 12.0 / 21.3 us at 8192 (512 nodes per CTA, the most a CTA takes);
-// HH 20.7 / 23.6 us at 5000, 30.5 / 23.1 us at 8192.
-constexpr int64_t kClusterMaxNodes = 8192, kClusterMaxNodesHH = 5120;
-cudaError_t ring_cluster_configure(); // per device, before the first cluster launch
-int cluster_max_ctas();               // 8 or 16
+// What the current device can do (asked once per device; sets the cluster kernels' attributes).
+ClusterLimits cluster_limits();
+// Small rings (cluster_size.h): all stages of n_steps RK4 steps in one thread-block-cluster
+// launch (ring_cluster.cu).  Same results as ring_step.
 int cluster_size_for(int model, int64_t N); // CTAs of the cluster for a ring of N nodes (0: not eligible)
 cudaError_t ring_cluster_steps(const RingPlan &p, double dt, int64_t n_steps, cudaStream_t s);
 

@@ -30,7 +30,6 @@ namespace cg = cooperative_groups;
 
 namespace simk {
 
-constexpr int kClusterSlice = 512; // nodes of a CTA at most (two warps' worth of int64 headroom: 512 2^54 = 2^63)
 constexpr int kClusterThreadsMax = kClusterSlice + 32;
 
 // Threads of a CTA that owns `per` nodes: one per node and the recording warp.
@@ -192,24 +191,6 @@ __global__ void __launch_bounds__(kClusterThreadsMax, 1)
     cluster.sync(); // no CTA exits while others may still read its shared memory
 }
 
-static int g_max_cluster = 8; // 16 when the device can co-schedule it (set by configure)
-int cluster_max_ctas() { return g_max_cluster; }
-
-int cluster_size_for(int model, int64_t N)
-{
-    if (N > (model == 2 ? kClusterMaxNodesHH : kClusterMaxNodes)) return 0;
-    int cl = (int)((N + 127) / 128);
-    if (cl < 2) cl = 2;
-    if (cl > g_max_cluster) cl = g_max_cluster;
-    return (N + cl - 1) / cl <= (int64_t)kClusterSlice ? cl : 0;
-}
-
-template <int M>
-static cudaError_t configure_one()
-{
-    return cudaFuncSetAttribute(ring_cluster_kernel<M>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-}
-
 static cudaLaunchConfig_t cluster_config(int cl, int per, size_t smem, cudaStream_t s, cudaLaunchAttribute *attr)
 {
     cudaLaunchConfig_t cfg = {};
@@ -226,24 +207,38 @@ static cudaLaunchConfig_t cluster_config(int cl, int per, size_t smem, cudaStrea
     return cfg;
 }
 
-cudaError_t ring_cluster_configure()
+// Largest cluster of model M's kernel at its largest slice (16, or 8, the portable size)
+// that the device can co-schedule, 0 if none.
+template <int M> static int largest_cluster()
 {
-    cudaError_t e = configure_one<0>();
-    if (e == cudaSuccess) e = configure_one<1>();
-    if (e == cudaSuccess) e = configure_one<2>();
-    if (e == cudaSuccess) e = configure_one<3>();
-    if (e != cudaSuccess) return e;
-    // largest cluster the device can co-schedule
-    cudaLaunchAttribute attr;
-    cudaLaunchConfig_t cfg = cluster_config(kClusterMaxCtas, (int)kClusterMaxNodes / kClusterMaxCtas,
-                                            cluster_smem_bytes<2>((int)kClusterMaxNodes / kClusterMaxCtas), nullptr, &attr);
-    int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, ring_cluster_kernel<0>, &cfg) == cudaSuccess && n >= 1)
-        g_max_cluster = kClusterMaxCtas;
-    else g_max_cluster = 8;
-    cudaGetLastError();
-    return cudaSuccess;
+    if (cudaFuncSetAttribute(ring_cluster_kernel<M>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return 0;
+    for (int cl = kClusterMaxCtas; cl >= 8; cl /= 2) {
+        cudaLaunchAttribute attr;
+        const cudaLaunchConfig_t cfg = cluster_config(cl, kClusterSlice, cluster_smem_bytes<Model<M>::NQ>(kClusterSlice), nullptr, &attr);
+        int n = 0;
+        if (cudaOccupancyMaxActiveClusters(&n, ring_cluster_kernel<M>, &cfg) == cudaSuccess && n >= 1) return cl;
+    }
+    return 0;
 }
+
+ClusterLimits cluster_limits()
+{
+    static PerDevice<ClusterLimits> known;
+    const int dev = current_device();
+    return known.get(dev, [dev] {
+        ClusterLimits l;
+        if (cudaDeviceGetAttribute(&l.sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) l.sms = 0;
+        const int rk4[4] = {largest_cluster<0>(), largest_cluster<1>(), largest_cluster<2>(), largest_cluster<3>()};
+        for (int m = 0; m < 4; ++m) {
+            l.rk4[m] = rk4[m];
+            l.dp[m] = dp_largest_cluster(m);
+        }
+        cudaGetLastError(); // a query that failed answers "none"
+        return l;
+    });
+}
+
+int cluster_size_for(int model, int64_t N) { return rk4_cluster_size(cluster_limits(), model, N); }
 
 template <int M>
 static cudaError_t launch_cluster(const RingPlan &p, double dt, int64_t n_steps, int cl, cudaStream_t s)

@@ -27,14 +27,9 @@ namespace simk {
 // Threads of a CTA and nodes per thread; two CTAs per SM by registers and shared memory.
 template <int M> struct DpShape { static constexpr int NT = 512, MPT = M == 0 ? 2 : 1; };
 template <> struct DpShape<2> { static constexpr int NT = 256, MPT = 1; };
-static int dp_slice(int model) { return model == 0 ? 1024 : model == 2 ? 256 : 512; } // NT * MPT
-
-// Nodes of a CTA at most: a slice's prefix stays below 2^63 in magnitude.  The Kuramoto
-// models' |q| reaches 2^53 (a sine or cosine of exactly 1), so 1024 coherent nodes would
-// wrap; the others' |q| stays below 2^54 and their slices hold 512.
-static int dp_slice_nodes(int model) { return model == 0 ? 1023 : dp_slice(model); }
-
-constexpr int kDpClusterNodes = 8192; // 32 sub-tiles: one lane each in the error sum
+template <int M> constexpr bool dp_shape_fits_rule() { return DpShape<M>::NT * DpShape<M>::MPT == dp_slice(M); }
+static_assert(dp_shape_fits_rule<0>() && dp_shape_fits_rule<1>() && dp_shape_fits_rule<2>() && dp_shape_fits_rule<3>(),
+              "dp_slice: the kernel's slots");
 
 template <int M> static size_t dp_cluster_smem(int per)
 {
@@ -416,48 +411,63 @@ __global__ void __launch_bounds__(DpShape<M>::NT, 2)
     sync_cluster(); // no CTA exits while others may still read its shared memory
 }
 
-// CTAs per ring for a run of n_rings rings: as few as hold the ring when the rings
-// alone fill the chip, more while they do not and a CTA keeps at least 96 nodes.
-int dp_cluster_size(int model, int64_t N, int n_rings)
+template <int M, bool ONE> static cudaError_t configure_shape()
 {
-    const int maxc = cluster_max_ctas(), slice = dp_slice(model);
-    if (N > kDpClusterNodes) return 0;
-    auto fits = [&](int cl) {
-        const int64_t per = ((N + cl - 1) / cl + 31) / 32 * 32; // the kernel's slices, all but the last one full
-        return per <= slice && std::min(per, N) <= dp_slice_nodes(model);
-    };
-    int cl = 1;
-    while (cl <= maxc && !fits(cl)) cl *= 2;
-    if (cl > maxc) return 0;
-    while (cl * 2 <= maxc && (int64_t)n_rings * cl * 2 <= 304 && N / (2 * cl) >= 96) cl *= 2;
-    return cl;
+    cudaError_t e = cudaFuncSetAttribute(ring_dp_cluster_kernel<M, ONE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)dp_cluster_smem<M>(dp_slice(M)));
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(ring_dp_cluster_kernel<M, ONE>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    return e;
+}
+
+template <int M>
+static cudaLaunchConfig_t shape_config(int n, int cl, int per, cudaStream_t s, cudaLaunchAttribute *attr)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(cl * n));
+    cfg.blockDim = dim3((unsigned)std::min(DpShape<M>::NT, per));
+    cfg.dynamicSmemBytes = dp_cluster_smem<M>(per);
+    cfg.stream = s;
+    attr->id = cudaLaunchAttributeClusterDimension;
+    attr->val.clusterDim.x = (unsigned)cl;
+    attr->val.clusterDim.y = 1;
+    attr->val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cfg;
+}
+
+// Attributes of model M's kernels on the current device, and the largest cluster at a
+// full slice it can co-schedule (0: none).
+template <int M> static int largest_cluster()
+{
+    if (configure_shape<M, true>() != cudaSuccess || configure_shape<M, false>() != cudaSuccess) return 0;
+    for (int cl = kClusterMaxCtas; cl >= 1; cl /= 2) {
+        cudaLaunchAttribute attr;
+        const cudaLaunchConfig_t cfg = shape_config<M>(1, cl, dp_slice(M), nullptr, &attr);
+        int n = 0;
+        const cudaError_t e = cl > 1 ? cudaOccupancyMaxActiveClusters(&n, ring_dp_cluster_kernel<M, false>, &cfg)
+                                     : cudaOccupancyMaxActiveClusters(&n, ring_dp_cluster_kernel<M, true>, &cfg);
+        if (e == cudaSuccess && n >= 1) return cl;
+    }
+    return 0;
+}
+int dp_largest_cluster(int model)
+{
+    switch (model) {
+    case 0: return largest_cluster<0>();
+    case 1: return largest_cluster<1>();
+    case 2: return largest_cluster<2>();
+    default: return largest_cluster<3>();
+    }
 }
 
 template <int M, bool ONE>
 static cudaError_t launch_shape(const DpPlan *plans, int n, int cl, int64_t n_max, int max_attempts, int first, cudaStream_t s)
 {
     const int per = (int)(((n_max + cl - 1) / cl + 31) / 32 * 32); // of the largest ring of the launch
-    static PerDevice<cudaError_t> done;
-    const cudaError_t err = done.get(current_device(), [] {
-        cudaError_t err = cudaFuncSetAttribute(ring_dp_cluster_kernel<M, ONE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)dp_cluster_smem<M>(dp_slice(M)));
-        if (err == cudaSuccess)
-            err = cudaFuncSetAttribute(ring_dp_cluster_kernel<M, ONE>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-        return err;
-    });
-    if (err != cudaSuccess) return err;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(cl * n));
-    cfg.blockDim = dim3((unsigned)std::min(DpShape<M>::NT, per));
-    cfg.dynamicSmemBytes = dp_cluster_smem<M>(per);
-    cfg.stream = s;
     cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim.x = (unsigned)cl;
-    attr.val.clusterDim.y = 1;
-    attr.val.clusterDim.z = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
+    const cudaLaunchConfig_t cfg = shape_config<M>(n, cl, per, s, &attr);
     return cudaLaunchKernelEx(&cfg, ring_dp_cluster_kernel<M, ONE>, plans, max_attempts, first);
 }
 

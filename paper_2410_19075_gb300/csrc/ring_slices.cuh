@@ -6,8 +6,6 @@
 
 namespace simk {
 
-constexpr int kClusterMaxCtas = 16;
-
 // Offsets of the cluster's slices from their totals, by one warp: lane r holds the
 // prefix in front of slice r as hi 2^sh + lo (ex_*), every lane the ring's total
 // (tot_*).  hi is exact modulo 2^64 only (sh goes with the window, so from 1024 nodes

@@ -510,12 +510,6 @@ void simk::lattice_rotation(LatticePlan &p, double alpha)
     p.mp.c[5] = std::ldexp(p.model == SIM_KS ? p.mp.c[1] : p.mp.c[0], -(p.F - 2));
 }
 
-static cudaError_t ensure_cluster_configured()
-{
-    static PerDevice<cudaError_t> done;
-    return done.get(current_device(), ring_cluster_configure);
-}
-
 extern "C" {
 
 size_t sim_workspace_bytes(int model, int topology, int64_t N, int64_t radius)
@@ -644,9 +638,7 @@ static int create_impl(sim_t *out, int model, int topology, int64_t N, int64_t r
             for (int k = 0; k < 4; ++k) p.facc[k] = reinterpret_cast<unsigned *>(b + L.facc) + k * slot;
             p.flat_ctr = ctrs + 3;
         }
-        if (N <= kClusterMaxNodes && !(flags & SIM_FLAG_STREAMING)) {
-            if (ensure_cluster_configured() != cudaSuccess) h->flags |= SIM_FLAG_STREAMING; // fall back to the streaming kernels
-        }
+        if (N <= kClusterMaxNodes && !(flags & SIM_FLAG_STREAMING)) cluster_limits(); // asked here, not by the first step
     } else {
         LatticePlan &p = h->lat;
         p.model = model;
@@ -1675,14 +1667,14 @@ int dp_run(const std::vector<sim_t> &mem, const sim_dp5_opts *opts, sim_dp5_stat
     std::vector<int> lat_members;
     int n_rings = 0;
     for (int i = 0; i < n; ++i) n_rings += mem[i]->topo == SIM_RING;
-    if (n_rings && ensure_cluster_configured() != cudaSuccess) n_rings = 0; // streaming kernels only
+    const ClusterLimits limits = n_rings ? cluster_limits() : ClusterLimits{};
     for (int i = 0; i < n; ++i) {
         const sim_t h = mem[i];
         if (h->topo != SIM_RING) {
             lat_members.push_back(i);
             continue;
         }
-        const int cl = n_rings && !(h->flags & SIM_FLAG_STREAMING) ? dp_cluster_size(h->model, h->N, n_rings) : 0;
+        const int cl = h->flags & SIM_FLAG_STREAMING ? 0 : dp_cluster_size(limits, h->model, h->N, n_rings);
         if (cl) resident[{h->model, cl}].push_back(i);
         else by_model[h->model].push_back(i);
     }
