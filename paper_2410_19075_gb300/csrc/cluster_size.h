@@ -39,22 +39,44 @@ inline int rk4_cluster_size(const ClusterLimits &d, int model, int64_t N)
 constexpr int dp_slice(int model) { return model == 0 ? 1024 : model == 2 ? 256 : 512; }
 constexpr int dp_slice_nodes(int model) { return model == 0 ? 1023 : dp_slice(model); }
 
-// CTAs per ring of a run of n_rings rings: as few as hold the ring when the rings alone
-// fill the chip (two CTAs per SM), more while they do not and a CTA keeps at least 96
-// nodes.  0: dp_launch's kernels.
-inline int dp_cluster_size(const ClusterLimits &d, int model, int64_t N, int n_rings)
+// The fewest CTAs that hold a ring (0: none do, or the device cannot co-schedule them).
+inline int dp_cluster_fewest(const ClusterLimits &d, int model, int64_t N)
 {
-    const int maxc = d.dp[model];
     if (N > kDpClusterNodes) return 0;
-    auto fits = [&](int cl) {
+    for (int cl = 1; cl <= d.dp[model]; ++cl) {
         const int64_t per = ((N + cl - 1) / cl + 31) / 32 * 32; // the kernel's slices, all but the last one full
-        return per <= dp_slice(model) && std::min(per, N) <= dp_slice_nodes(model);
-    };
-    int cl = 1;
-    while (cl <= maxc && !fits(cl)) cl *= 2;
-    if (cl > maxc) return 0;
-    while (cl * 2 <= maxc && (int64_t)n_rings * cl * 2 <= 2 * d.sms && N / (2 * cl) >= 96) cl *= 2;
+        if (per <= dp_slice(model) && std::min(per, N) <= dp_slice_nodes(model)) return cl;
+    }
+    return 0;
+}
+
+// A run whose rings at their fewest CTAs fill the chip (two CTAs per SM) more than twice
+// over is bound by throughput, not by its longest chain.  There the streaming kernels are
+// the faster ones for Hodgkin-Huxley rings of more than 1024 nodes and FitzHugh-Nagumo
+// rings of more than 2560 (256 rings, streaming against cluster: HH 38.3 / 38.3 ms at 1100
+// nodes, 45.4 / 48.7 at 1500, 82.6 / 97.0 at 3000; FHN 31.5 / 30.0 at 2100, 42.4 / 43.8 at
+// 3000, 58.2 / 61.3 at 4100); the Kuramoto models gain at every size (4.07 / 3.30 at 4100).
+inline bool dp_run_is_full(const ClusterLimits &d, int64_t fewest_ctas) { return fewest_ctas > 4 * (int64_t)d.sms; }
+constexpr int64_t dp_full_run_nodes(int model) { return model == 2 ? 1024 : model == 1 ? 2560 : kDpClusterNodes; }
+
+// CTAs per ring of a run of n_rings rings (full: dp_run_is_full): the fewest that hold the
+// ring, or more, a power of two, while the rings still fit on the chip together and a CTA
+// keeps at least 96 nodes.  0: dp_launch's kernels.
+inline int dp_cluster_size(const ClusterLimits &d, int model, int64_t N, int n_rings, bool full = false)
+{
+    int cl = dp_cluster_fewest(d, model, N);
+    if (cl == 0 || (full && N > dp_full_run_nodes(model))) return 0;
+    for (int c = 2; c <= d.dp[model]; c *= 2)
+        if (c > cl && (int64_t)n_rings * c <= 2 * d.sms && N / c >= 96) cl = c;
     return cl;
+}
+
+// One of few cluster sizes for a ring of cl CTAs: the next power of two, if the device takes it.
+inline int dp_cluster_class(const ClusterLimits &d, int model, int cl)
+{
+    int c = 1;
+    while (c < cl) c *= 2;
+    return c <= d.dp[model] ? c : cl;
 }
 
 } // namespace simk

@@ -20,9 +20,11 @@ int main(int, char **v)
     for (int m = 0; m < 4; ++m) d.rk4[m] = std::atoi(v[2]), d.dp[m] = std::atoi(v[3]);
     int model, rings;
     long long n;
-    while (std::scanf("%d %lld %d", &model, &n, &rings) == 3)
-        std::printf("%d %d %d %d\n", simk::rk4_cluster_size(d, model, n), simk::dp_cluster_size(d, model, n, rings),
-                    simk::dp_slice(model), simk::dp_slice_nodes(model));
+    while (std::scanf("%d %lld %d", &model, &n, &rings) == 3) {
+        const int cl = simk::dp_cluster_size(d, model, n, rings), full = simk::dp_cluster_size(d, model, n, rings, true);
+        std::printf("%d %d %d %d %d %d\n", simk::rk4_cluster_size(d, model, n), cl, simk::dp_slice(model),
+                    simk::dp_slice_nodes(model), full, cl ? simk::dp_cluster_class(d, model, cl) : 0);
+    }
 }
 """
 
@@ -51,18 +53,23 @@ NODES = sorted({*range(2, 70), 255, 256, 257, *range(990, 1060), 2047, 2048, 204
 @pytest.mark.parametrize("sms", [1, 132, 148, 152])
 def test_slices_fit_and_do_not_wrap(sizes, sms, largest):
     rings = [(m, n, k) for m in range(4) for n in NODES for k in (1, 24, 200, 1000)]
-    for (m, n, k), (rk4, dp, slots, filled) in zip(rings, sizes(sms, largest, largest, rings)):
+    for (m, n, k), (rk4, dp, slots, filled, full, cls) in zip(rings, sizes(sms, largest, largest, rings)):
         # no kernel whose own shape the device cannot co-schedule: 0 is the streaming kernels
-        assert 0 <= rk4 <= largest and 0 <= dp <= largest
+        assert 0 <= rk4 <= largest and 0 <= dp <= cls <= largest
         assert filled * MAX_Q[m] < 2 ** 63 and 512 * MAX_Q[m] < 2 ** 63
         if rk4:
             assert n <= (5120 if m == 2 else 8192) and -(-n // rk4) <= 512
+
+        def per(c):  # nodes of a slice, and slots
+            slice_slots = -(-(-(-n // c)) // 32) * 32
+            return slice_slots <= slots and min(slice_slots, n) <= filled
+        fewest = next((c for c in range(1, largest + 1) if n <= 8192 and per(c)), 0)
+        assert (dp > 0) == (fewest > 0) and full in (0, dp)
         if dp:
-            per = -(-(-(-n // dp)) // 32) * 32
-            assert per <= slots and min(per, n) <= filled and n <= 8192
-            smallest = next(c for c in (1, 2, 4, 8, 16) if -(-(-(-n // c)) // 32) * 32 <= slots
-                            and min(-(-(-(-n // c)) // 32) * 32, n) <= filled)
-            assert dp == smallest or (k * dp <= 2 * sms and n // dp >= 96)  # more only while the chip is not full
+            assert per(dp) and per(cls)
+            # more than the fewest only while the chip is not full
+            assert dp == fewest or (dp > fewest and k * dp <= 2 * sms and n // dp >= 96)
+            assert (full == 0) == (n > {0: 8192, 1: 2560, 2: 1024, 3: 8192}[m])
 
 
 def test_the_two_kernels_are_asked_separately(sizes):
