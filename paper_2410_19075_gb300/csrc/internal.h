@@ -209,11 +209,11 @@ struct LatticePlan {
     double *obs;
     int64_t obs_cap;
     unsigned long long *obs_ctr;
-    // ball/disk: the reads (row shift, plane shift, half-width, 0) of the windows of a
+    // ball/disk: the reads (row shift | plane shift << 16, half-width) of the windows of a
     // thread's block of lattice_gather_nodes nodes together (lattice_gather_kernel), by the set of nodes
     // that add them: the reads of set m (bit jj + 2 kk = node (j + jj, k + kk)) end at
     // op_end[m] and start at op_end[m - 1]
-    const int4 *ops;
+    const int2 *ops;
     int nops, op_end[16];
     const int *skip;    // if set and nonzero, the x, y and gather passes of stage 1 return at once
                         // (a finished Dormand-Prince run); nullptr for every other use

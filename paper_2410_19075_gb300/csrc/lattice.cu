@@ -927,10 +927,10 @@ __global__ void __launch_bounds__(kGatherThreads, 7) lattice_gather_kernel(Latti
             const int n = min(kGatherOps, nops - c0);
             if (c0) __syncthreads();
             for (int q = tid; q < n; q += kGatherThreads) {
-                const int4 op = __ldg(p.ops + c0 + q); // (a, z, w, 0)
-                const int kk = k0 + op.y;
+                const int2 op = __ldg(p.ops + c0 + q); // (a | z << 16, w)
+                const int kk = k0 + (op.x >> 16);
                 const unsigned kw = ball ? (unsigned)(kk >= n1 ? kk - n1 : kk) : 0u;
-                s_op[q] = make_uint2((unsigned)op.x | (unsigned)op.z << 16, kw * (unsigned)n1 * rowlen + (unsigned)op.z * warray);
+                s_op[q] = make_uint2((unsigned)(op.x & 0xffff) | (unsigned)op.y << 16, kw * (unsigned)n1 * rowlen + (unsigned)op.y * warray);
             }
             __syncthreads();
             if (live) gather_classes<1, NB, WMODE>(s_start, c0, n, s_op, base, j0, n1, rowlen, W);

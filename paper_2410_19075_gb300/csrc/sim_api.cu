@@ -92,16 +92,17 @@ std::vector<int4> chords_of(int topo, int64_t P, int64_t *count)
 }
 
 // The reads of the windows of a block of nb nodes (4: rows j, j + 1 of planes k, k + 1;
-// 2: rows j, j + 1; 1) of a ball or disk together, as (row shift from row j - P, plane
-// shift from plane k - P, half-width, 0): see LatticePlan::ops.
-std::vector<int4> gather_ops(int topo, int64_t P, int nb, LatticePlan &p)
+// 2: rows j, j + 1; 1) of a ball or disk together, as (row shift from row j - P | plane
+// shift from plane k - P << 16, half-width), and the ends of each set's reads: see
+// LatticePlan::ops.
+std::vector<int2> gather_ops(int topo, int64_t P, int nb, int *op_end)
 {
     int64_t count = 0;
     const int tk = nb > 2 ? 2 : 1, tj = nb > 1 ? 2 : 1, rows = 2 * (int)P + 1, np = topo == SIM_BALL3D ? rows : 1;
     std::vector<int> w((size_t)np * rows, -1); // half-width at (plane shift, dy + P)
     for (const int4 &c : chords_of(topo, P, &count))
         w[(size_t)(np > 1 ? c.y + (int)P : 0) * rows + c.x + (int)P] = c.z;
-    std::vector<std::vector<int4>> by_set(16);
+    std::vector<std::vector<int2>> by_set(16);
     for (int z = 0; z < np + tk - 1; ++z)
         for (int a = 0; a < rows + tj - 1; ++a) {
             int wb[4] = {-1, -1, -1, -1}; // the half-width node b of the block reads there
@@ -118,15 +119,14 @@ std::vector<int4> gather_ops(int topo, int64_t P, int nb, LatticePlan &p)
                         set |= 1 << c;
                         first = first && c >= b;
                     }
-                if (first) by_set[set].push_back(make_int4(a, z, wb[b], 0));
+                if (first) by_set[set].push_back(make_int2(a | z << 16, wb[b])); // a, z <= 2 P + 1 < 2^14
             }
         }
-    std::vector<int4> out;
+    std::vector<int2> out;
     for (int m = 0; m < 16; ++m) {
         out.insert(out.end(), by_set[m].begin(), by_set[m].end());
-        p.op_end[m] = (int)out.size();
+        op_end[m] = (int)out.size();
     }
-    p.nops = (int)out.size();
     return out;
 }
 
@@ -193,7 +193,7 @@ struct Layout {
     size_t total = 0;
     size_t y, acc, xg0, xg1, npar, lam0, lam1, ingrp0, ingrp1, grpofs0, grpofs1, subtot, grptot, grpctr;
     size_t fsub0, fsub1, facc; // one-pass prefix (rings of at most kFlatMaxGroups groups)
-    size_t f, xs, sx, sxy, cpl, partial, chords, ctrs, obs, tabs;
+    size_t f, xs, sx, sxy, cpl, partial, ops, ctrs, obs, tabs;
 };
 
 // Ball: one x-window array per chord half-width (one load per read instead of two)
@@ -252,7 +252,8 @@ Layout layout_of(int model, int topo, int64_t N, int64_t R, unsigned flags = 0)
         L.sxy = take(topo == SIM_CUBE3D ? sizeof(int64_t) * lattice_sxy_elems(N) : 0);
         L.cpl = take(topo == SIM_CUBE3D ? sizeof(double) * n : 0);
         L.partial = take(sizeof(i128) * 2 * nblk);
-        L.chords = take(topo == SIM_CUBE3D ? 0 : sizeof(int4) * 4 * (2 * R + 2) * (topo == SIM_DISK2D ? 1 : 2 * R + 2));
+        int op_end[16];
+        L.ops = take(topo == SIM_CUBE3D ? 0 : sizeof(int2) * gather_ops(topo, R, lattice_gather_nodes(topo, N), op_end).size());
     }
     L.ctrs = take(64);
     L.obs = take(sizeof(double) * kObsCap);
@@ -296,7 +297,7 @@ struct sim_handle {
     Layout L;
     RingPlan ring{};
     LatticePlan lat{};
-    std::vector<int4> gather_ops; // host copy (the upload reads it asynchronously)
+    std::vector<int2> gather_ops; // host copy (the upload reads it asynchronously)
     unsigned *err = nullptr;
     unsigned long long *obs_ctr = nullptr;
     double *obs = nullptr;
@@ -669,9 +670,10 @@ static int create_impl(sim_t *out, int model, int topology, int64_t N, int64_t r
         p.obs_ctr = h->obs_ctr;
         p.ops = nullptr;
         if (topology != SIM_CUBE3D) {
-            h->gather_ops = gather_ops(topology, radius, lattice_gather_nodes(topology, N), p);
-            p.ops = reinterpret_cast<const int4 *>(b + L.chords);
-            e = cudaMemcpyAsync(b + L.chords, h->gather_ops.data(), sizeof(int4) * h->gather_ops.size(),
+            h->gather_ops = gather_ops(topology, radius, lattice_gather_nodes(topology, N), p.op_end);
+            p.nops = (int)h->gather_ops.size();
+            p.ops = reinterpret_cast<const int2 *>(b + L.ops);
+            e = cudaMemcpyAsync(b + L.ops, h->gather_ops.data(), sizeof(int2) * h->gather_ops.size(),
                                 cudaMemcpyHostToDevice, h->stream);
         }
         static PerDevice<cudaError_t> lat_done;
