@@ -1792,6 +1792,9 @@ int dp_run(const std::vector<sim_t> &mem, const sim_dp5_opts *opts, sim_dp5_stat
             GraphDpPlan q{e, mem[i]->graph};
             q.rhs.r.y = e.xbuf;
             q.rhs.r.obs = nullptr;
+            // each evaluation is a prologue and a stage 1: with the one-pass prefix both would clear
+            // accumulators by a memset between the launches (376 us per attempt at 20000 nodes, 283 here)
+            q.rhs.r.flat = 0;
             q.rhs.r.skip = &(d_ctl + i)->done;
             q.rhs.r.err = reinterpret_cast<unsigned *>(&(d_ctl + i)->bad); // out of range: reject
             gplans.push_back(q);
