@@ -78,11 +78,13 @@ __device__ __forceinline__ void ring_stage_body(const RingPlan &P, const RingSta
 // independent right-hand sides per thread and one warp scan per node pair.  The
 // same integers and FP64 expressions as ring_stage_body, so the same bits.
 constexpr int kRing2Threads = kSubTile / 2;
-// Resident CTAs per SM the registers are sized for.  Kuramoto with inertia: 6 (80
-// registers) 27.1 us per RK4 step at 10^5 nodes, 8 (64, spilling) 29.3; the other
-// models lose 2% with 7.
+// Resident CTAs per SM the registers are sized for: 8 (64 registers), for Kuramoto with
+// inertia 7 (72), which spills less.  Its RK4 steps with 8 / 7 / 6 per SM, in us: 26.2 / 24.2 /
+// 24.2 at 50000 nodes, 64.5 / 63.4 / 71.9 at 5 10^5, 539 / 533 / 570 at 5 10^6, 512 rings of
+// 1000 80.7 / 80.3 / 87.6; but 42.7 / 51.9 / 52.1 at 3 10^5, where 8 make one wave of what takes
+// two with 7 (ring2_in_one_wave).  The other models lose 2% with 7.
 template <int M> struct Ring2MinBlocks { static constexpr int value = 8; };
-template <> struct Ring2MinBlocks<3> { static constexpr int value = 6; };
+template <> struct Ring2MinBlocks<3> { static constexpr int value = 7; };
 
 template <int M, int STAGE>
 __device__ __forceinline__ void ring_stage_body2(const RingPlan &P, const RingStageIO &a, const StepSize &h,
@@ -181,9 +183,8 @@ __device__ __forceinline__ void ring_stage_body2(const RingPlan &P, const RingSt
         a.facc_zero);
 }
 
-template <int M, int STAGE>
-__global__ void __launch_bounds__(kRing2Threads, Ring2MinBlocks<M>::value)
-    ring_stage_kernel2(const RingPlan p, const StepSize h)
+template <int M, int STAGE, int CTAS = Ring2MinBlocks<M>::value>
+__global__ void __launch_bounds__(kRing2Threads, CTAS) ring_stage_kernel2(const RingPlan p, const StepSize h)
 {
     if (p.skip && *(const volatile int *)p.skip) return; // uniform over the launch
     ring_stage_body2<M, STAGE>(p, stage_io<M, STAGE>(p), h, blockIdx.x);
@@ -237,6 +238,31 @@ __global__ void __launch_bounds__(kRing2Threads, Ring2MinBlocks<M>::value)
     ring_stage_body2<M, STAGE>(p, stage_io<M, STAGE>(p), h, sub);
 }
 
+// Whether all sub-tiles of a ring are resident at once with 8 CTAs per SM and not with
+// the fewer its model is compiled for.
+template <int M> static bool ring2_in_one_wave(const RingPlan &p)
+{
+    if (Ring2MinBlocks<M>::value >= 8) return false;
+    static PerDevice<int> sms;
+    const int dev = current_device(), n = sms.get(dev, [dev] {
+        int v = 0;
+        return cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess ? v : 0;
+    });
+    return p.nsub > Ring2MinBlocks<M>::value * n && p.nsub <= 8 * n;
+}
+
+template <int M, int CTAS> static void launch_stage2(int stage, const RingPlan &p, const StepSize &h, cudaStream_t s)
+{
+    const dim3 grid((unsigned)p.nsub), block(kRing2Threads);
+    switch (stage) {
+    case 0: ring_stage_kernel2<M, 0><<<grid, block, 0, s>>>(p, h); break;
+    case 1: ring_stage_kernel2<M, 1, CTAS><<<grid, block, 0, s>>>(p, h); break;
+    case 2: ring_stage_kernel2<M, 2, CTAS><<<grid, block, 0, s>>>(p, h); break;
+    case 3: ring_stage_kernel2<M, 3, CTAS><<<grid, block, 0, s>>>(p, h); break;
+    default: ring_stage_kernel2<M, 4, CTAS><<<grid, block, 0, s>>>(p, h); break;
+    }
+}
+
 // The kernel variant is the plan's (p.npt, from sim_create or the autotuner):
 // two nodes per thread (128 threads per sub-tile) or one (256).
 template <int M>
@@ -245,14 +271,8 @@ static cudaError_t launch_stage(int stage, const RingPlan &p, double dt, cudaStr
     const dim3 grid((unsigned)p.nsub), block(kRingThreads);
     if constexpr (M != 2) {
         if (p.npt == 2) {
-            const dim3 block2(kRing2Threads);
-            switch (stage) {
-            case 0: ring_stage_kernel2<M, 0><<<grid, block2, 0, s>>>(p, step_size(dt)); break;
-            case 1: ring_stage_kernel2<M, 1><<<grid, block2, 0, s>>>(p, step_size(dt)); break;
-            case 2: ring_stage_kernel2<M, 2><<<grid, block2, 0, s>>>(p, step_size(dt)); break;
-            case 3: ring_stage_kernel2<M, 3><<<grid, block2, 0, s>>>(p, step_size(dt)); break;
-            default: ring_stage_kernel2<M, 4><<<grid, block2, 0, s>>>(p, step_size(dt)); break;
-            }
+            if (ring2_in_one_wave<M>(p)) launch_stage2<M, 8>(stage, p, step_size(dt), s);
+            else launch_stage2<M, Ring2MinBlocks<M>::value>(stage, p, step_size(dt), s);
             return cudaGetLastError();
         }
     }
