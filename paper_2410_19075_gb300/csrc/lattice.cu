@@ -43,9 +43,12 @@ constexpr int kGatherOps = 512;       // ball/disk gather: reads of the window h
 constexpr size_t kRowSmemMax = 220 * 1024;
 
 // i-columns per tile: shared memory (N1 + 1) BI 16 bytes stays below ~76 KB, so that
-// three CTAs fit on an SM; the widest such tile pads least and keeps a window pass's
+// three y CTAs fit on an SM; the widest such tile pads least and keeps a window pass's
 // own (sin, cos) in segments of BI 16 bytes (8 columns where 16 fit: 165 us per step
-// against 151 at 101^3, 907 against 867 at 200^3).
+// against 151 at 101^3, 907 against 867 at 200^3).  At the top of a range, edges 288 to
+// 297 and 576 to 594, only two z-window CTAs fit, and the wider tile is still no worse:
+// per step 2.33 ms with 16 columns and 2.37 with 8 at 288^3, 2.57 both at 290^3, 2.66 and 2.64
+// at 293^3; with 8 and 4 columns 18.7 and 20.1 at 576^3, 21.6 and 23.1 at 594^3.
 __host__ __device__ inline int cube_tile_lg(int64_t N1) { return N1 <= 297 ? 4 : N1 <= 594 ? 3 : 2; }
 __host__ __device__ inline int cube_tile_bi(int64_t N1) { return 1 << cube_tile_lg(N1); }
 
@@ -68,12 +71,14 @@ static int row_warps(int64_t N1)
 // prefix rows of a CTA round up to less of the SM (seven CTAs of four 464-node
 // rows, against three of eight).
 constexpr int kNodexWarpsMax = 4;
-// Shared memory's share of the L1 of the node pass, in percent of its maximum.  Left
-// to the driver, rows of 464 nodes take nearly all of it for seven CTAs per SM and
-// the sin/cos table misses: 9.93 ms per step, 9.52 with five CTAs and 92 KB of L1
-// (72%); edges 320, 200 and 101 lose 0.5% against the driver's choice, and 58% or 86%
-// are worse at 464.
+// Shared memory's share of the L1 of the node pass, in percent of its maximum, for rows
+// longer than kNodexCarveoutRow<M> nodes.  Left to the driver, long rows take nearly all
+// of it for six or seven CTAs per SM and the sin/cos table misses.  Per step in ms, the
+// driver's choice and 72%: Kuramoto 3.17 / 3.20 at 320^3, 4.54 / 4.54 at 358^3, 4.73 / 4.72 at
+// 362^3, 6.14 / 6.07 at 400^3, 9.99 / 9.48 at 464^3; with inertia 7.37 / 7.52 at 400^3, 9.51 / 9.71
+// at 430^3, 11.55 / 11.46 at 464^3, 15.3 / 15.15 at 500^3.  58% and 86% are worse at 464^3.
 constexpr int kNodexCarveout = 72;
+template <int M> constexpr int64_t kNodexCarveoutRow = M == 0 ? 360 : 448;
 // CTAs per SM the fused node pass is compiled for: six for Kuramoto (at most 80
 // registers, so stage 4 fits six too), five for the model with inertia.
 template <int M> constexpr int kNodexBlocks = M == 0 ? 6 : 5;
@@ -629,7 +634,7 @@ __device__ __forceinline__ void lattice_write_coupling(const LatticePlan &p, int
 //                of y, its x sums and its order parameter.
 // The window pass keeps the tile's 64-byte row segments (the z columns are
 // N1^2 elements apart), the node pass reads and writes whole warps of
-// consecutive nodes.  Three window CTAs per SM at the tile sizes of N1 <= 594.
+// consecutive nodes.  Three window CTAs per SM up to N1 = 287 and from 298 to 575.
 // At 464^3 (interleaved (sin, cos) pairs): two planes per unrolled iteration
 // with three planes of prefetch 0.826 ms, two planes of prefetch 0.831 ms, one
 // plane per iteration 0.860 ms; 512 threads (at most 42 registers) 0.884 ms.  With
@@ -1042,8 +1047,6 @@ cudaError_t lattice_configure()
 #define SIM_NODEX_ATTR(M, S)                                                                                           \
     if (e == cudaSuccess)                                                                                              \
         e = cudaFuncSetAttribute(cube_nodex_kernel<M, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRowSmemMax); \
-    if (e == cudaSuccess)                                                                                              \
-        e = cudaFuncSetAttribute(cube_nodex_kernel<M, S>, cudaFuncAttributePreferredSharedMemoryCarveout, kNodexCarveout); \
     if (e == cudaSuccess && S > 0)                                                                                     \
         e = cudaFuncSetAttribute(cube_batch_nodex_kernel<M, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRowSmemMax);
     SIM_NODEX_ATTR(0, 0) SIM_NODEX_ATTR(0, 1) SIM_NODEX_ATTR(0, 2) SIM_NODEX_ATTR(0, 3) SIM_NODEX_ATTR(0, 4)
@@ -1147,9 +1150,17 @@ static cudaError_t launch_cube_stage(const LatticePlan &p, double dt, cudaStream
     const int w = nodex_warps(p.N1);
     const int64_t rows = p.nodes / p.N1;
     const unsigned nblk = (unsigned)((rows + w - 1) / w);
-    cube_nodex_kernel<M, STAGE><<<nblk, 32 * w, (size_t)w * (size_t)(p.N1 + 1) * sizeof(longlong2), s>>>(
-        p, step_size(dt));
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+    attr.val.sharedMemCarveout = kNodexCarveout;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(nblk);
+    cfg.blockDim = dim3(32 * w);
+    cfg.dynamicSmemBytes = (size_t)w * (size_t)(p.N1 + 1) * sizeof(longlong2);
+    cfg.stream = s;
+    cfg.attrs = &attr;
+    cfg.numAttrs = p.N1 > kNodexCarveoutRow<M> ? 1 : 0;
+    if ((e = cudaLaunchKernelEx(&cfg, cube_nodex_kernel<M, STAGE>, p, step_size(dt))) != cudaSuccess) return e;
     kernel_mark(s, 2);
     if (STAGE == 0 || STAGE == 4) {
         lattice_order_kernel<<<order_grid(nblk), kOrderThreads, 0, s>>>(p, nblk);
