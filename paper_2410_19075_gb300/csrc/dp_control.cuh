@@ -21,8 +21,10 @@ __constant__ double c_dp_a[7][6] = {
 __constant__ double c_dp_e[7] = {71.0 / 57600.0, 0.0, -71.0 / 16695.0, 71.0 / 1920.0, -17253.0 / 339200.0,
                                  22.0 / 525.0, -1.0 / 40.0};
 
-// The roundings of the tableau sums, fixed so that every kernel gives the same
-// bits: the first two products in one FMA, every further one in an FMA of its own.
+// The roundings of the tableau sums of the ring kernels, fixed so that those of dp5.cu and
+// of the cluster give the same bits (lattice_dp.cu, which has no second kernel to agree
+// with, leaves its sums to the compiler): the first two products in one FMA, every further
+// one in an FMA of its own.
 __device__ __forceinline__ double dp_sum2(double a, double x, double b, double y) { return fma(a, x, __dmul_rn(b, y)); }
 
 // Hermite interpolant of the phase at t + th h from the step's ends (a0, a1) and slopes (f0, f1).

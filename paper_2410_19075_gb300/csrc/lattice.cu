@@ -819,7 +819,7 @@ __global__ void __launch_bounds__(kOrderThreads) cube_batch_order_kernel(const L
     lattice_order_total(p, p.partial, (unsigned)((p.nodes / p.N1 + w - 1) / w));
 }
 
-// ball / disk gather: a thread gathers the window sums of kGatherTj x TK nodes (j,
+// ball / disk gather: a thread gathers the window sums of TJ x TK nodes (j,
 // j + 1; k, k + 1; disks one plane) at column i.  The plan's table lists the reads
 // of all its windows together, (row shift a from row j - P, plane shift z from plane
 // k - P, half-width w) in the order of the set of nodes that add them: a row segment
@@ -906,7 +906,7 @@ __device__ __forceinline__ void gather_classes(const int *start, int c0, int n, 
 }
 
 // STAGE 1-4: the RK4 stage; 0: the prologue (no gather); 5: the slopes into acc (a
-// right-hand-side evaluation).  NB nodes per thread (LatticePlan::nb).
+// right-hand-side evaluation).  NB nodes per thread (lattice_gather_nodes).
 template <int M, int STAGE, bool WMODE, int NB>
 __global__ void __launch_bounds__(kGatherThreads, 7) lattice_gather_kernel(LatticePlan p, const StepSize h)
 {

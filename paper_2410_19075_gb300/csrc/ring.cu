@@ -13,7 +13,7 @@
 //       sub-tile (one CTA), and, without any CTA waiting for another, the exact
 //       prefix at every sub-tile start: the last CTA to finish in each group of
 //       64 sub-tiles scans that group, and the last group scans the groups; or,
-//       for rings of at most 64 groups (one-pass prefix, ring_parts.cuh), the
+//       for rings of at most 128 groups (one-pass prefix, ring_parts.cuh), the
 //       sub-tile totals and group accumulators the next kernel sums itself;
 //   a6  (stage 4) the Kuramoto order parameter of y_{n+1} from the global totals.
 // The prologue kernel does a1/a2/a6 for the initial state.  The Kuramoto and

@@ -425,8 +425,6 @@ void simk::model_constants(int model, const double *params, double K, ModelParam
         }
         mp.c[2] = std::sin(alpha);
         mp.c[3] = std::cos(alpha);
-        mp.q[0] = (int64_t)std::llround(std::ldexp(mp.c[3], 62)); // exact: |cos| <= 1, 53-bit significand
-        mp.q[1] = (int64_t)std::llround(std::ldexp(mp.c[2], 62));
         // alpha = aq pi/2 + alpha0 with alpha0 in [0, pi/2): the angle addition of
         // the ring and link-matrix right-hand side (ring_coupling)
         {
