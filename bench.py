@@ -12,7 +12,8 @@ handle's stream), so the same events give the whole-step time (value) and each
 kernel's average launch time (roofline); 512 MiB are written between iterations
 to flush L2 (the lattice's 4 GB of state exceed L2 anyway).
 
-Beside the headline the JSON line carries the FitzHugh-Nagumo ring of 10^6 nodes
+The one JSON line on stdout holds the headline.  The full record goes to stderr as a
+line "bench detail: {...}", with the FitzHugh-Nagumo ring of 10^6 nodes
 (the plain one-network path at its config), the 1000-node Kuramoto ring, rings of
 10^7 and 10^8 nodes, Hodgkin-Huxley rings, the paper's 3D inertia network, link
 matrices, the 4096-ring batched sweep, Dormand-Prince sweeps and the served mix
@@ -973,6 +974,33 @@ def bench_served_sweep(args, stream, rates=(10.0, 50.0, 200.0, 800.0, 3200.0)):
     return out
 
 
+# ----------------------------------------------------------------------------- output
+HEADLINE_KEYS = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+                 "vs_baseline", "dtype", "data", "config", "e2e", "gpu_launches", "clocks", "roofline", "cpu_baseline")
+HEADLINE_INNER = {"e2e": ("value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step"),
+                  "roofline": ("kernel", "bound", "achieved", "peak", "unit", "frac", "share_of_timed_region", "traffic"),
+                  "cpu_baseline": ("value", "unit", "cores", "kind", "sample")}
+HEADLINE_MAX = 2000  # characters: a record that keeps only the end of the output keeps this line whole
+
+
+def headline(line):
+    """The measured line's headline: what identifies and explains the main workload, in at most
+    HEADLINE_MAX characters.  Everything else goes out in the detail line."""
+    out = {k: line[k] for k in HEADLINE_KEYS if k in line}
+    for k, inner in HEADLINE_INNER.items():
+        if isinstance(out.get(k), dict):
+            out[k] = {i: out[k][i] for i in inner if i in out[k]}
+    return out
+
+
+def print_line(line):
+    """One JSON line on stdout; the full record, with the other workloads, on stderr before it."""
+    print("bench detail: " + json.dumps(line), file=sys.stderr, flush=True)
+    text = json.dumps(headline(line))
+    assert len(text) <= HEADLINE_MAX, len(text)
+    print(text, flush=True)
+
+
 # ----------------------------------------------------------------------------- native
 def run_native(args):
     import torch
@@ -1070,7 +1098,7 @@ def run_native(args):
         line["served"] = bench_served(args, stream)
         line["served_rate_sweep"] = bench_served_sweep(args, stream)
     if rank == 0:
-        print(json.dumps(line), flush=True)
+        print_line(line)
     if world > 1:
         import torch.distributed as dist
         dist.destroy_process_group()
