@@ -171,7 +171,7 @@ ClusterLimits cluster_limits();
 // Small rings (cluster_size.h): all stages of n_steps RK4 steps in one thread-block-cluster
 // launch (ring_cluster.cu).  Same results as ring_step.
 int cluster_size_for(int model, int64_t N); // CTAs of the cluster for a ring of N nodes (0: not eligible)
-cudaError_t ring_cluster_steps(const RingPlan &p, double dt, int64_t n_steps, cudaStream_t s);
+cudaError_t ring_cluster_steps(const RingPlan &p, int cl, double dt, int64_t n_steps, cudaStream_t s);
 
 cudaError_t ring_clear_slot(const RingPlan &p, int slot, cudaStream_t s); // zero a one-pass accumulator slot
 // Ring: stage 1 only with dt = 0, so acc receives f(y) and y is untouched.

@@ -238,7 +238,10 @@ ClusterLimits cluster_limits()
     });
 }
 
-int cluster_size_for(int model, int64_t N) { return rk4_cluster_size(cluster_limits(), model, N); }
+int cluster_size_for(int model, int64_t N)
+{
+    return N <= kClusterMaxNodes ? rk4_cluster_size(cluster_limits(), model, N) : 0;
+}
 
 template <int M>
 static cudaError_t launch_cluster(const RingPlan &p, double dt, int64_t n_steps, int cl, cudaStream_t s)
@@ -249,10 +252,8 @@ static cudaError_t launch_cluster(const RingPlan &p, double dt, int64_t n_steps,
     return cudaLaunchKernelEx(&cfg, ring_cluster_kernel<M>, p, step_size(dt), per, n_steps);
 }
 
-cudaError_t ring_cluster_steps(const RingPlan &p, double dt, int64_t n_steps, cudaStream_t s)
+cudaError_t ring_cluster_steps(const RingPlan &p, int cl, double dt, int64_t n_steps, cudaStream_t s)
 {
-    const int cl = cluster_size_for(p.model, p.N);
-    if (cl == 0) return cudaErrorInvalidValue;
     cudaError_t e;
     switch (p.model) {
     case 0: e = launch_cluster<0>(p, dt, n_steps, cl, s); break;

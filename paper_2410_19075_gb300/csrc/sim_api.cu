@@ -296,6 +296,7 @@ struct sim_handle {
     size_t bytes = 0;
     Layout L;
     RingPlan ring{};
+    int cluster = 0; // CTAs of the cluster-resident RK4 kernel (0: the streaming kernels)
     LatticePlan lat{};
     std::vector<int2> gather_ops; // host copy (the upload reads it asynchronously)
     unsigned *err = nullptr;
@@ -339,12 +340,12 @@ int check_device_error(sim_t h)
 
 bool use_cluster(sim_t h)
 {
-    return h->topo == SIM_RING && !(h->flags & SIM_FLAG_STREAMING) && cluster_size_for(h->model, h->N) > 0;
+    return h->cluster > 0;
 }
 
 cudaError_t launch_steps(sim_t h, int64_t n, double dt, cudaStream_t s)
 {
-    if (use_cluster(h)) return n > 0 ? ring_cluster_steps(h->ring, dt, n, s) : cudaSuccess;
+    if (use_cluster(h)) return n > 0 ? ring_cluster_steps(h->ring, h->cluster, dt, n, s) : cudaSuccess;
     for (int64_t t = 0; t < n; ++t) {
         const cudaError_t e = h->topo == SIM_RING    ? ring_step(h->ring, dt, s)
                               : h->topo == SIM_GRAPH ? graph_step(h->graph, dt, s)
@@ -638,7 +639,7 @@ static int create_impl(sim_t *out, int model, int topology, int64_t N, int64_t r
             for (int k = 0; k < 4; ++k) p.facc[k] = reinterpret_cast<unsigned *>(b + L.facc) + k * slot;
             p.flat_ctr = ctrs + 3;
         }
-        if (N <= kClusterMaxNodes && !(flags & SIM_FLAG_STREAMING)) cluster_limits(); // asked here, not by the first step
+        if (topology == SIM_RING && !(flags & SIM_FLAG_STREAMING)) h->cluster = cluster_size_for(model, N);
     } else {
         LatticePlan &p = h->lat;
         p.model = model;
@@ -926,7 +927,7 @@ int sim_step(sim_t h, int64_t n_steps, double dt)
     int64_t left = n_steps;
     while (left > 0 && use_cluster(h)) { // one launch runs all the steps
         const int64_t n = left < kClusterSteps ? left : kClusterSteps;
-        const cudaError_t e = ring_cluster_steps(h->ring, dt, n, h->stream);
+        const cudaError_t e = ring_cluster_steps(h->ring, h->cluster, dt, n, h->stream);
         if (e != cudaSuccess) return cuda_fail(e, "cluster launch");
         left -= n;
         h->steps_done += n;
