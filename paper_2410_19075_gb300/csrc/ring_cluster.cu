@@ -13,8 +13,8 @@
 //     of the CTA that owns that end of the window (its address is fixed for the
 //     call), plus the difference of the two slices' offsets, which every warp
 //     scans from the totals itself while those reads are in flight;
-//   * the order parameter of every step is recorded by one more warp of CTA 0,
-//     beside the stage that follows.
+//   * the order parameter of every step is recorded by one more warp of CTA 0, from
+//     the exact sum of the slice totals, beside the stage that follows.
 // What bounds a stage is one dependent chain: barrier, remote reads, right-hand
 // side, sin/cos, scan.
 // The arithmetic (grid, exact sums, right-hand sides, RK4) is the streaming

@@ -1,10 +1,10 @@
 // Adaptive Dormand-Prince 5(4) on small rings, a whole run inside one thread-block
-// cluster per ring (dp5.cu runs larger rings with seven launches per attempt).
+// cluster per ring (cluster_size.h; dp5.cu runs the others with seven launches per attempt).
 //
 // A batch of 1000-node rings spent seven launches per attempt on it, each reading
 // every earlier slope from global memory and rebuilding the prefix hierarchy, and
 // finished rings kept their share of the launches.  Here a ring's state, slopes and
-// prefix stay in the shared memory of its cluster (one CTA for up to kDpSlice nodes),
+// prefix stay in the shared memory of its cluster (one CTA for up to dp_slice_nodes),
 // every CTA a slice of consecutive nodes as in ring_cluster.cu; the cluster takes its
 // own step decisions and loops until its run is done, so rings of a batch neither
 // wait for one another nor share launches.  What bounds it: the FP64 pipe (about 70
