@@ -194,6 +194,8 @@ struct Layout {
     size_t y, acc, xg0, xg1, npar, lam0, lam1, ingrp0, ingrp1, grpofs0, grpofs1, subtot, grptot, grpctr;
     size_t fsub0, fsub1, facc; // one-pass prefix (rings of at most kFlatMaxGroups groups)
     size_t f, xs, sx, sxy, cpl, partial, ops, ctrs, obs, tabs;
+    std::vector<int2> gather; // ball, disk: the reads (LatticePlan::ops)
+    int op_end[16];
 };
 
 // Ball: one x-window array per chord half-width (one load per read instead of two)
@@ -252,8 +254,8 @@ Layout layout_of(int model, int topo, int64_t N, int64_t R, unsigned flags = 0)
         L.sxy = take(topo == SIM_CUBE3D ? sizeof(int64_t) * lattice_sxy_elems(N) : 0);
         L.cpl = take(topo == SIM_CUBE3D ? sizeof(double) * n : 0);
         L.partial = take(sizeof(i128) * 2 * nblk);
-        int op_end[16];
-        L.ops = take(topo == SIM_CUBE3D ? 0 : sizeof(int2) * gather_ops(topo, R, lattice_gather_nodes(topo, N), op_end).size());
+        if (topo != SIM_CUBE3D) L.gather = gather_ops(topo, R, lattice_gather_nodes(topo, N), L.op_end);
+        L.ops = take(sizeof(int2) * L.gather.size());
     }
     L.ctrs = take(64);
     L.obs = take(sizeof(double) * kObsCap);
@@ -298,7 +300,6 @@ struct sim_handle {
     RingPlan ring{};
     int cluster = 0; // CTAs of the cluster-resident RK4 kernel (0: the streaming kernels)
     LatticePlan lat{};
-    std::vector<int2> gather_ops; // host copy (the upload reads it asynchronously)
     unsigned *err = nullptr;
     unsigned long long *obs_ctr = nullptr;
     double *obs = nullptr;
@@ -669,10 +670,10 @@ static int create_impl(sim_t *out, int model, int topology, int64_t N, int64_t r
         p.obs_ctr = h->obs_ctr;
         p.ops = nullptr;
         if (topology != SIM_CUBE3D) {
-            h->gather_ops = gather_ops(topology, radius, lattice_gather_nodes(topology, N), p.op_end);
-            p.nops = (int)h->gather_ops.size();
+            p.nops = (int)L.gather.size(); // the handle's layout: the upload reads it asynchronously
+            std::copy(L.op_end, L.op_end + 16, p.op_end);
             p.ops = reinterpret_cast<const int2 *>(b + L.ops);
-            e = cudaMemcpyAsync(b + L.ops, h->gather_ops.data(), sizeof(int2) * h->gather_ops.size(),
+            e = cudaMemcpyAsync(b + L.ops, L.gather.data(), sizeof(int2) * L.gather.size(),
                                 cudaMemcpyHostToDevice, h->stream);
         }
         static PerDevice<cudaError_t> lat_done;
