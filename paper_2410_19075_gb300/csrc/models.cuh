@@ -227,11 +227,11 @@ template <> struct Model<1> {
     // (|u|, |v| < 8, so |u - u^3/3| < 171), and each slope takes one conversion; k_u = G_u / eps with
     // 1/eps in two parts (its rounding would be the largest systematic error left).
     // Every product is truncated at 2^-54 or finer (|error| of a bracket < 3 2^-54,
-    // against roundings of 2^-53 |u| in FP64): rms error of k_u from this arithmetic 2.3e-15 on the
-    // circle of radius 2, 3.3e-15 in FP64; 7e-16 against 3e-16 next to the rest point, where the
-    // grid of u and v itself makes 3.3e-15.  Ring of 10^6: 35 -> 23 us per stage launch.  fx = 0 (coupling constants or a beyond the range the
-    // host checks, windows of fewer than 65 nodes): FP64, c[2..5] carrying
-    // 2^(ksh - F).
+    // against roundings of 2^-53 |u| in FP64): rms error of k_u from this arithmetic
+    // 2.3e-15 on the circle of radius 2, 3.3e-15 in FP64; 7e-16 against 3e-16 next to the
+    // rest point, where the grid of u and v itself makes 3.3e-15.  Ring of 10^6: 35 -> 23 us
+    // per stage launch.  fx = 0 (coupling constants or a beyond the range the host checks,
+    // windows of fewer than 65 nodes): FP64, c[2..5] carrying 2^(ksh - F).
     __device__ __forceinline__ static void rhs_ring(const ModelParams &P, const int64_t (&qo)[NQ],
                                                     const int64_t (&S)[NQ], const double *, double, double (&k)[D])
     {
